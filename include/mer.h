@@ -407,8 +407,9 @@ int mer_precond_apply(const int64_t* row_ptr, const int32_t* col, int64_t V, flo
 size_t mer_precond_solve_workspace_size(int64_t V);
 /* Solve (I + lambda L) x = b by conjugate gradients on the device (FP32 vectors, FP64 dot products), the
  * three columns as one block-diagonal system.  x holds the initial guess (a warm start) and receives the
- * solution.  Runs at most max_iters iterations as a fixed launch sequence; the iterations after the
- * residual norm falls to rel_tol * |b| return immediately.  workspace: 256-byte aligned device memory of
+ * solution.  Runs at most max_iters iterations and ends when the residual norm falls to rel_tol * |b|: in
+ * one launch while the rows fit one resident grid (about 260,000 on GB300), beyond that as a fixed
+ * launch sequence whose later iterations return immediately.  Either can be captured in a graph.  workspace: 256-byte aligned device memory of
  * mer_precond_solve_workspace_size(V) bytes, owned by the caller. */
 int mer_precond_solve(const int64_t* row_ptr, const int32_t* col, int64_t V, float lambda, const float* b,
                       float* x, int max_iters, float rel_tol, void* workspace, size_t workspace_bytes,
