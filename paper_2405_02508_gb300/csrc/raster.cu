@@ -240,13 +240,22 @@ __global__ void k_scan_add(int* __restrict__ out, long long N, const int* __rest
 }
 
 // --- raster ---
-// One CTA per tile.  The tile's triangle records are staged in shared memory; each warp takes one
-// triangle at a time and its lanes test the pixels of the triangle's bounding box inside the tile (32 at a
-// time), so the work follows the bounding-box areas and every lane of a warp runs the same triangle.  The
+// One CTA per tile.  The tile's triangle records are staged in shared memory and sorted by the pixel count of their
+// bounding box inside the tile: a group of 2, 8 or 32 lanes takes one triangle at a time and tests that box G pixels at
+// a time.  Most boxes of a mesh hold a few to a few dozen pixels, so a whole warp per triangle left most lanes idle and
+// ran the per-triangle preparation once per triangle; now a warp shares it between 4 or 16 of them (with a warp for each:
+// 40,960 triangles at 512 x 512, tile 16, 23.6 us, now 14.4; 8 views of 32,768 at 512 x 512, tile 32, 97.6 and 84.1; 48
+// uneven meshes, 816 and 701; 32 views of 131,072 at 1334 x 2048, where a box holds about 64 pixels, 2,131 and 2,110).
+// Triangles that are hidden or miss the tile are dropped while they are staged, by one thread each.  The
 // nearest fragment per pixel is resolved in a shared-memory z-buffer by a 64-bit atomicMax on
 // (depth key bits << 32 | ~triangle id): larger depth key wins, equal keys go to the lower id.
 constexpr int kStage = 256;  // triangle records staged per round
 constexpr int kRasterThreads = 256;
+// The lines between the groups (us at 512 x 512 / 8 views, tile 32 / 32 head views; 8 and 64: 14.4 / 84.1 / 2,110): with 4
+// lanes for the middle group 14.0 / 85.5 / 2,158, with lines at 16 and 96 pixels 15.6 / 86.6 / 2,152, with one lane for the
+// smallest 15.8 / 88.3 / 2,120.
+constexpr int kTinyPx = 8;     // boxes of at most this many pixels: 2 lanes each
+constexpr int kSmallPx = 64;   // of at most this many: 8 lanes each; larger ones: a warp
 constexpr int kRasterCtasPerSm = 4;  // resident CTAs per SM (the 64 x 64 tile's shared memory allows four): 64 registers
 
 // Per-pixel bits kept in shared memory for the cover image: a front-facing triangle covered the centre
@@ -260,6 +269,8 @@ struct RasterShared {
     static constexpr int kStageTS = TS >= 64 ? 160 : kStage;  // keeps the 64 x 64 tile within 48 KB
     TriRaster rec[kStageTS];
     int id[kStageTS];
+    unsigned char todo[3][kStageTS];  // the stage's records by box size (tiny, small, large), less those that cannot win
+    int n_todo[2][3];                 // their lengths, for alternate stages
     unsigned long long zbuf[TS * TS];
     unsigned cov[TS * TS / 4];  // cover-image bits (kCov*), one byte a pixel
     float red[kRasterThreads / 32];
@@ -290,6 +301,61 @@ __device__ __forceinline__ float tile_min_zeta(RasterShared<TS>& S, int ox, int 
     return r;
 }
 
+// Draws the n records S.todo[CLASS] of the stage into the z-buffer, G lanes a triangle.
+template <int TS, int CLASS, int G>
+__device__ __forceinline__ void raster_class(RasterShared<TS>& S, int n, int ox, int oy, bool back, bool cover) {
+    const int lane = threadIdx.x % G;
+    for (int k = threadIdx.x / G; k < n; k += kRasterThreads / G) {
+        const int j = S.todo[CLASS][k];
+        const TriRaster r = S.rec[j];  // in registers: the loop's shared-memory atomics would force reloads
+        const int x0 = max((int)r.bx0, ox), x1 = min((int)r.bx1, ox + TS - 1);
+        const int y0 = max((int)r.by0, oy), y1 = min((int)r.by1, oy + TS - 1);
+        const int bw = x1 - x0 + 1;
+        const int npx = bw * (y1 - y0 + 1);
+        const unsigned idkey = 0xFFFFFFFFu - (unsigned)S.id[j];
+        // lane -> (dx, dy) in the bbox, then advance by G pixels per pass without dividing per pixel.  The
+        // quotients q / bw (q <= 32, bw <= TS <= 64) come from an approximate reciprocal: the product is within
+        // 2^-16 of q / bw, whose fraction is 0 or at least 1/64, so q / bw + 2^-10 truncates to the quotient.
+        const float rb = __fdividef(1.0f, (float)bw);
+        int dy = (int)__fmaf_rn((float)lane, rb, 0x1p-10f);
+        int dx = lane - dy * bw;
+        const int sy = (int)__fmaf_rn((float)G, rb, 0x1p-10f), sx = G - sy * bw;
+        for (int i = lane; i < npx; i += G) {
+            const int px = x0 + dx, py = y0 + dy;
+            dx += sx;
+            dy += sy;
+            if (dx >= bw) {
+                dx -= bw;
+                ++dy;
+            }
+            float z;
+            if (r.flags & 16) {
+                int E[3];
+                if (!covers_small(r, px, py, E)) continue;
+                z = depth_key_small(r, E);
+            } else {
+                int64_t E[3];
+                if (!covers(r, 256 * px + 128, 256 * py + 128, E)) continue;
+                z = depth_key(r, E);
+            }
+            const unsigned long long key = ((unsigned long long)__float_as_uint(z) << 32) | idkey;
+            const int pi = (py - oy) * TS + (px - ox);
+            // the 64-bit maximum runs as a compare-and-swap loop: its old value costs nothing extra
+            const unsigned long long old = atomicMax(&S.zbuf[pi], key);
+            if (cover) {
+                const unsigned sh = (pi & 3) * 8;
+                if (!back) {
+                    if (old) atomicOr(&S.cov[pi >> 2], kCovF2 << sh);  // a front fragment came first
+                } else {
+                    if (key > old) atomicOr(&S.cov[pi >> 2], kCovWB << sh);
+                    const unsigned o = atomicOr(&S.cov[pi >> 2], kCovB1 << sh);
+                    if (o & (kCovB1 << sh)) atomicOr(&S.cov[pi >> 2], kCovB2 << sh);
+                }
+            }
+        }
+    }
+}
+
 // SHADE: also shade every pixel of the tile from its z-buffer winner (shade_fragment, as the deferred
 // shading kernels do from the index image).
 // cover (optional): one byte a pixel (MER_COVER_* bits): whether another triangle of the winner's facing,
@@ -317,73 +383,36 @@ __device__ __forceinline__ void raster_tile(const RItem& it, int local_tile, con
     const int count = overflow ? 0 : cnts[tile];
     const int off = overflow ? 0 : offs[tile];
     const int nf = overflow ? 0 : min(nfront[tile], count);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr int kWarps = kRasterThreads / 32;
     float zcull = 0.0f;
-    int m = 0;
+    int m = 0, stage = 0;
+    if (threadIdx.x < 3) S.n_todo[0][threadIdx.x] = 0;
     for (int base = 0; base < count; base += m) {
         // stage boundaries fall on the front / back split so each stage is one part
         const int lim = base < nf ? nf : count;
         m = min(kSt, lim - base);
         if (base == nf && base > 0) zcull = tile_min_zeta<TS>(S, ox, oy, it.W, it.H, cover != nullptr);
+        const bool back = base >= nf;
         __syncthreads();
+        int* n_todo = S.n_todo[stage & 1];
+        ++stage;
+        if (threadIdx.x < 3) S.n_todo[stage & 1][threadIdx.x] = 0;  // the next stage's (last read before the barrier)
         for (int j = threadIdx.x; j < m; j += kRasterThreads) {
             const int t = list[off + base + j];
-            S.rec[j] = it.recs[t];
-            S.id[j] = t;
-        }
-        __syncthreads();
-        const bool back = base >= nf;
-        for (int j = warp; j < m; j += kWarps) {
-            const TriRaster r = S.rec[j];  // in registers: the loop's shared-memory atomics would force reloads
+            const TriRaster r = it.recs[t];
             if (back && r.zmax * (1.0f + 0x1p-20f) < zcull) continue;  // hidden behind the whole tile
-            const int x0 = max((int)r.bx0, ox), x1 = min((int)r.bx1, ox + TS - 1);
-            const int y0 = max((int)r.by0, oy), y1 = min((int)r.by1, oy + TS - 1);
-            const int bw = x1 - x0 + 1, bh = y1 - y0 + 1;
+            const int bw = min((int)r.bx1, ox + TS - 1) - max((int)r.bx0, ox) + 1;
+            const int bh = min((int)r.by1, oy + TS - 1) - max((int)r.by0, oy) + 1;
             if (bw <= 0 || bh <= 0) continue;
             const int npx = bw * bh;
-            const unsigned idkey = 0xFFFFFFFFu - (unsigned)S.id[j];
-            // lane -> (dx, dy) in the bbox, then advance by 32 pixels per pass without dividing per pixel.  The
-            // quotients q / bw (q <= 32, bw <= TS <= 64) come from an approximate reciprocal: the product is within
-            // 2^-16 of q / bw, whose fraction is 0 or at least 1/64, so q / bw + 2^-10 truncates to the quotient.
-            const float rb = __fdividef(1.0f, (float)bw);
-            int dy = (int)__fmaf_rn((float)lane, rb, 0x1p-10f);
-            int dx = lane - dy * bw;
-            const int sy = (int)__fmaf_rn(32.0f, rb, 0x1p-10f), sx = 32 - sy * bw;
-            for (int i = lane; i < npx; i += 32) {
-                const int px = x0 + dx, py = y0 + dy;
-                dx += sx;
-                dy += sy;
-                if (dx >= bw) {
-                    dx -= bw;
-                    ++dy;
-                }
-                float z;
-                if (r.flags & 16) {
-                    int E[3];
-                    if (!covers_small(r, px, py, E)) continue;
-                    z = depth_key_small(r, E);
-                } else {
-                    int64_t E[3];
-                    if (!covers(r, 256 * px + 128, 256 * py + 128, E)) continue;
-                    z = depth_key(r, E);
-                }
-                const unsigned long long key = ((unsigned long long)__float_as_uint(z) << 32) | idkey;
-                const int pi = (py - oy) * TS + (px - ox);
-                // the 64-bit maximum runs as a compare-and-swap loop: its old value costs nothing extra
-                const unsigned long long old = atomicMax(&S.zbuf[pi], key);
-                if (cover) {
-                    const unsigned sh = (pi & 3) * 8;
-                    if (!back) {
-                        if (old) atomicOr(&S.cov[pi >> 2], kCovF2 << sh);  // a front fragment came first
-                    } else {
-                        if (key > old) atomicOr(&S.cov[pi >> 2], kCovWB << sh);
-                        const unsigned o = atomicOr(&S.cov[pi >> 2], kCovB1 << sh);
-                        if (o & (kCovB1 << sh)) atomicOr(&S.cov[pi >> 2], kCovB2 << sh);
-                    }
-                }
-            }
+            S.rec[j] = r;
+            S.id[j] = t;
+            const int c = npx <= kTinyPx ? 0 : (npx <= kSmallPx ? 1 : 2);
+            S.todo[c][atomicAdd(&n_todo[c], 1)] = (unsigned char)j;
         }
+        __syncthreads();
+        raster_class<TS, 2, 32>(S, n_todo[2], ox, oy, back, cover != nullptr);
+        raster_class<TS, 1, 8>(S, n_todo[1], ox, oy, back, cover != nullptr);
+        raster_class<TS, 0, 2>(S, n_todo[0], ox, oy, back, cover != nullptr);
     }
     __syncthreads();
     for (int i = threadIdx.x; i < TS * TS; i += kRasterThreads) {
