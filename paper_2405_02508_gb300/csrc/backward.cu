@@ -22,7 +22,7 @@
 
 #include <cstdint>
 
-#include "mer_device.cuh"
+#include "shade_device.cuh"
 
 namespace mer {
 
@@ -30,7 +30,12 @@ constexpr int kTW = kBwdTileW, kTH = kBwdTileH;  // tile: 8 warps, two rows each
 constexpr int kRows = 2;                          // rows per warp
 constexpr int kHW = kTW + 2, kHH = kTH + 2;
 constexpr int kThreads = 256;
-constexpr int kCtasPerSm = 6;                     // resident CTAs per SM: at most 42 registers a thread
+// Resident CTAs per SM.  The batched kernel works on whole batches and wants the warps (6: at most 42 registers a thread; 32
+// head views 2,381 us with 6, 2,386 with 5, 2,506 with 4; 48 uneven meshes 640, 658, 723); a per-view launch is a few
+// thousand tiles, whose chains gain from the registers (3 views at 333 x 517: 19.6 us with 6, 17.5 with 5; 1024 x 1024 with
+// attribute gradients: 52.4 and 48.3, with 4 16.5 and 48.9).
+constexpr int kCtasPerSm = 6;
+constexpr int kViewCtasPerSm = 5;
 static_assert(kTW == 32 && kTH == kRows * kThreads / 32, "a warp spans the tile's width");
 // Per-tile triangle table of 2^BITS slots: a 32x16 tile of the head-scale workloads holds ~20-80 triangles.
 // 128 slots keep six CTAs resident with most of the SM's on-chip memory left to the L1 cache that serves the
@@ -71,11 +76,8 @@ struct BwdArgs {
 // Vertex ids of triangle t; false if one is out of range.
 __device__ __forceinline__ bool tri_ids(const int* __restrict__ tris, int t, int V, int id[3]) {
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        id[k] = __ldg(tris + 3 * (size_t)t + k);
-        if ((unsigned)id[k] >= (unsigned)V) return false;
-    }
-    return true;
+    for (int k = 0; k < 3; ++k) id[k] = __ldg(tris + 3 * (size_t)t + k);
+    return max(max((unsigned)id[0], (unsigned)id[1]), (unsigned)id[2]) < (unsigned)V;
 }
 
 // Plane normal (v1 - v0) x (v2 - v0) in (x_s, y_s, zeta) from accurate differences.
@@ -411,7 +413,9 @@ __device__ __forceinline__ bool tile_halo(const BItem& it, const BwdArgs& a, int
 // the row's edge buffers).
 // NA > 0: also produce the attribute gradients (channels [a0, a0 + NA) of each vertex's attribute row, NA <= 4:
 // the interpolated channels, or (u, v) in texture mode), aggregated like the vertex gradients.
-template <int NA, bool EXACT, int BITS>
+// FORM: the layout of the main channels (ShadeForm).  Without it the pass spilled 48 registers and a twelfth of its
+// instructions decoded the layout: 32 head views 2,764 us, now 2,381; 48 uneven meshes with attribute gradients 761 and 640.
+template <int FORM, int NA, bool EXACT, int BITS>
 __device__ __forceinline__ void row_pass(const BItem& it, int tx, int ty, int row, int lane, bool pairs,
                                          const BwdArgs& a, const float* __restrict__ tex, BwdShared<NA, EXACT, BITS>& S,
                                          void* ws) {
@@ -453,16 +457,31 @@ __device__ __forceinline__ void row_pass(const BItem& it, int tx, int ty, int ro
 
         if (a.terms & MER_INTERIOR) {
             const float z[3] = {rv[0].zeta, rv[1].zeta, rv[2].zeta};
-            const float s = B.lam[0] * z[0] + B.lam[1] * z[1] + B.lam[2] * z[2];
+            const float s = __fmaf_rn(B.lam[2], z[2], __fmaf_rn(B.lam[0], z[0], __fmul_rn(B.lam[1], z[1])));
             const float is = rcp_nr(s);
             float b[3];
 #pragma unroll
-            for (int k = 0; k < 3; ++k) b[k] = B.lam[k] * z[k] * is;
+            for (int k = 0; k < 3; ++k) b[k] = __fmul_rn(__fmul_rn(B.lam[k], z[k]), is);
             // G_k = dL/db_k.  Only the differences G_k - G_i enter (sum_i b_i = 1), so they are formed from
             // attribute differences: D01 = G_0 - G_1, D02 = G_0 - G_2, D12 = G_1 - G_2.
             float D01 = 0.f, D02 = 0.f, D12 = 0.f;
             const int Ca = a.sh.C_attr;
-            if (a.sh.uv_offset < 0) {
+            if (FORM == kAttr3) {
+                const float *q0 = attr + (long long)vid[0] * Ca, *q1 = attr + (long long)vid[1] * Ca,
+                            *q2 = attr + (long long)vid[2] * Ca;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const float gc = __ldg(gp + c);
+                    const float a0 = __ldg(q0 + c), a1 = __ldg(q1 + c), a2 = __ldg(q2 + c);
+                    D01 += gc * (a0 - a1);
+                    D02 += gc * (a0 - a2);
+                    D12 += gc * (a1 - a2);
+                    if (NA > 0) {
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) ca[k][c < NA ? c : 0] = b[k] * gc;
+                    }
+                }
+            } else if (FORM != kTex3 && a.sh.uv_offset < 0) {
                 for (int c = 0; c < a.sh.n_main; ++c) {
                     const float gc = __ldg(gp + c);
                     const float a0 = __ldg(attr + (size_t)vid[0] * Ca + c);
@@ -483,16 +502,22 @@ __device__ __forceinline__ void row_pass(const BItem& it, int tx, int ty, int ro
                 }
             } else {
                 float uk[3], vk[3];
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    uk[k] = __ldg(attr + (size_t)vid[k] * Ca + a.sh.uv_offset);
-                    vk[k] = __ldg(attr + (size_t)vid[k] * Ca + a.sh.uv_offset + 1);
-                }
+                load_uv<FORM>(attr, Ca, a.sh.uv_offset, vid, uk, vk);
                 const TexCoord cx = tex_coord(uk[0], uk[1], uk[2], b[1], b[2], a.sh.tex_w);
                 const TexCoord cy = tex_coord(vk[0], vk[1], vk[2], b[1], b[2], a.sh.tex_h);
                 const TexTaps taps = tex_taps(a.sh.tex_h, a.sh.tex_w, cx, cy);
                 float gu, gv;
-                tex_grad_uv(tex, a.sh.tex_h, a.sh.tex_w, a.tex_stride, a.tex_vec4, a.sh.n_main, taps, gp, gu, gv);
+                if (FORM == kTex3) {
+                    const TexQuad q = tex_quad(tex, a.sh.tex_w, taps);
+                    float su = 0.f, sv = 0.f;
+                    tex_lerp_grad(q.a00.x, q.a10.x, q.a01.x, q.a11.x, taps, __ldg(gp), su, sv);
+                    tex_lerp_grad(q.a00.y, q.a10.y, q.a01.y, q.a11.y, taps, __ldg(gp + 1), su, sv);
+                    tex_lerp_grad(q.a00.z, q.a10.z, q.a01.z, q.a11.z, taps, __ldg(gp + 2), su, sv);
+                    gu = (float)a.sh.tex_w * su;
+                    gv = taps.clamped ? 0.0f : (float)a.sh.tex_h * sv;
+                } else {
+                    tex_grad_uv(tex, a.sh.tex_h, a.sh.tex_w, a.tex_stride, a.tex_vec4, a.sh.n_main, taps, gp, gu, gv);
+                }
                 D01 = gu * (uk[0] - uk[1]) + gv * (vk[0] - vk[1]);
                 D02 = gu * (uk[0] - uk[2]) + gv * (vk[0] - vk[2]);
                 D12 = gu * (uk[1] - uk[2]) + gv * (vk[1] - vk[2]);
@@ -623,13 +648,13 @@ __device__ __forceinline__ void row_pass(const BItem& it, int tx, int ty, int ro
 
 // The tile (tx, ty) of an item, after tile_halo and a barrier: each warp takes rows kRows * warp ..
 // kRows * warp + kRows - 1, first their edge pairs together, then each row's pixels.
-template <int NA, bool EXACT, int BITS>
+template <int FORM, int NA, bool EXACT, int BITS>
 __device__ __forceinline__ void tile_compute(const BItem& it, int tx, int ty, const BwdArgs& a,
                                              const float* __restrict__ tex, BwdShared<NA, EXACT, BITS>& S, void* ws) {
     const int lane = threadIdx.x & 31, r0 = (threadIdx.x >> 5) * kRows;
     const bool pairs = (a.terms & MER_EDGE) && edge_rows<NA, EXACT, BITS>(it, a, S, ws, r0, lane, tx * kTW, ty * kTH);
 #pragma unroll 1
-    for (int k = 0; k < kRows; ++k) row_pass<NA, EXACT, BITS>(it, tx, ty, r0 + k, lane, pairs, a, tex, S, ws);
+    for (int k = 0; k < kRows; ++k) row_pass<FORM, NA, EXACT, BITS>(it, tx, ty, r0 + k, lane, pairs, a, tex, S, ws);
 }
 
 // After tile_compute and a barrier: add the table to global memory and clear it.
@@ -665,8 +690,8 @@ __device__ __forceinline__ void tile_flush(const BItem& it, const BwdArgs& a, Bw
     }
 }
 
-template <int NA, bool EXACT, int BITS>
-__global__ void __launch_bounds__(kThreads, kCtasPerSm) k_backward(const mer_vertex* __restrict__ vpix, const int* __restrict__ tris,
+template <int FORM, int NA, bool EXACT, int BITS>
+__global__ void __launch_bounds__(kThreads, kViewCtasPerSm) k_backward(const mer_vertex* __restrict__ vpix, const int* __restrict__ tris,
                                                        const int* __restrict__ index,
                                                        const unsigned char* __restrict__ cover,
                                                        const float* __restrict__ image,
@@ -688,13 +713,13 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_backward(const mer_ver
     table_clear(S);
     const bool covered = tile_halo(it, a, local % a.ntx, local / a.ntx, S);
     if (!__syncthreads_or(covered)) return;  // background tile
-    tile_compute<NA, EXACT, BITS>(it, local % a.ntx, local / a.ntx, a, tex, S, ws);
+    tile_compute<FORM, NA, EXACT, BITS>(it, local % a.ntx, local / a.ntx, a, tex, S, ws);
     __syncthreads();
     tile_flush(it, a, S);
 }
 
 // Persistent: each CTA takes the next backward tile of any item from the work queue.
-template <int NA, bool EXACT, int BITS>
+template <int FORM, int NA, bool EXACT, int BITS>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_backward_batch(const mer_vertex* __restrict__ vpix,
                                                              const int* __restrict__ tris,
                                                              const mer_item* __restrict__ items, int n_items,
@@ -741,7 +766,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_backward_batch(const m
         tile_halo(it, a, tx, ty, S);
         __syncthreads();
         if (threadIdx.x == 0) s_tile = (long long)atomicAdd(&hdr->queue_backward, 1ull);
-        tile_compute<NA, EXACT, BITS>(it, tx, ty, a, tex, S, ws);
+        tile_compute<FORM, NA, EXACT, BITS>(it, tx, ty, a, tex, S, ws);
         __syncthreads();
         tile_flush(it, a, S);
     }
@@ -760,6 +785,39 @@ int attr_channels(const mer_shading* sh, const float* grad_attr) {
     return A >= 1 && A <= kMaxA ? A : -1;
 }
 }  // namespace
+
+// Launches L(form, attribute-gradient channels, exact crossing, table bits) for the call.  The layouts in use have their
+// own form (see ShadeForm) with the channels they can have; other layouts and the exact-crossing option are generic.
+#define MER_BWD_DISPATCH(L)                                                                                            \
+    do {                                                                                                               \
+        const int na = attr_channels(sh, grad_attr);                                                                   \
+        const int form = exact ? kGeneric : shade_form(attr, tex, sh);                                                 \
+        if (na == 0 && !exact && dense) {                                                                              \
+            if (form == kTex3) L(kTex3, 0, false, kTableBitsDense);                                                    \
+            else if (form == kAttr3) L(kAttr3, 0, false, kTableBitsDense);                                             \
+            else L(kGeneric, 0, false, kTableBitsDense);                                                               \
+        } else if (form == kTex3) {                                                                                    \
+            if (na == 0) L(kTex3, 0, false, kTableBits);                                                               \
+            else L(kTex3, 2, false, kTableBits);                                                                       \
+        } else if (form == kAttr3) {                                                                                   \
+            if (na == 0) L(kAttr3, 0, false, kTableBits);                                                              \
+            else L(kAttr3, 3, false, kTableBits);                                                                      \
+        } else {                                                                                                       \
+            switch (na * 2 + (exact ? 1 : 0)) {                                                                        \
+                case 0: L(kGeneric, 0, false, kTableBits); break;                                                      \
+                case 1: L(kGeneric, 0, true, kTableBits); break;                                                       \
+                case 2: L(kGeneric, 1, false, kTableBits); break;                                                      \
+                case 3: L(kGeneric, 1, true, kTableBits); break;                                                       \
+                case 4: L(kGeneric, 2, false, kTableBits); break;                                                      \
+                case 5: L(kGeneric, 2, true, kTableBits); break;                                                       \
+                case 6: L(kGeneric, 3, false, kTableBits); break;                                                      \
+                case 7: L(kGeneric, 3, true, kTableBits); break;                                                       \
+                case 8: L(kGeneric, 4, false, kTableBits); break;                                                      \
+                case 9: L(kGeneric, 4, true, kTableBits); break;                                                       \
+                default: return 1;                                                                                     \
+            }                                                                                                          \
+        }                                                                                                              \
+    } while (0)
 
 // max_tri_density: the largest T / (H W) over the items (the table size follows the densest item).
 extern "C" int mer_launch_backward_batch(const mer_vertex* vpix, const int* tris, const mer_item* items, int n_items,
@@ -796,38 +854,16 @@ extern "C" int mer_launch_backward_batch(const mer_vertex* vpix, const int* tris
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kThreads, 0) != cudaSuccess) return 0u;
         return (unsigned)(sms * (per_sm > 0 ? per_sm : 1));
     };
-#define MER_BWD_BATCH(A, E)                                                                                        \
+#define MER_BWD_BATCH(F, A, E, BITS)                                                                               \
     do {                                                                                                           \
-        grid = grid_of((const void*)k_backward_batch<A, E, kTableBits>);                                           \
+        grid = grid_of((const void*)k_backward_batch<F, A, E, BITS>);                                              \
         if (grid == 0) return 2;                                                                                   \
-        k_backward_batch<A, E, kTableBits><<<grid, kThreads, 0, s>>>(vpix, tris, items, n_items, btiles, index,   \
-                                                                     cover, image, grad_image, attr, tex, a,      \
-                                                                     grad_vpix, grad_attr, ws);                   \
+        k_backward_batch<F, A, E, BITS><<<grid, kThreads, 0, s>>>(vpix, tris, items, n_items, btiles, index,      \
+                                                                  cover, image, grad_image, attr, tex, a,         \
+                                                                  grad_vpix, grad_attr, ws);                      \
     } while (0)
     const bool dense = max_tri_density > kDenseTrianglesPerPixel;
-    switch (attr_channels(sh, grad_attr) * 2 + (exact ? 1 : 0)) {
-        case 0:
-            if (dense) {
-                grid = grid_of((const void*)k_backward_batch<0, false, kTableBitsDense>);
-                if (grid == 0) return 2;
-                k_backward_batch<0, false, kTableBitsDense><<<grid, kThreads, 0, s>>>(
-                    vpix, tris, items, n_items, btiles, index, cover, image, grad_image, attr, tex, a, grad_vpix,
-                    grad_attr, ws);
-            } else {
-                MER_BWD_BATCH(0, false);
-            }
-            break;
-        case 1: MER_BWD_BATCH(0, true); break;
-        case 2: MER_BWD_BATCH(1, false); break;
-        case 3: MER_BWD_BATCH(1, true); break;
-        case 4: MER_BWD_BATCH(2, false); break;
-        case 5: MER_BWD_BATCH(2, true); break;
-        case 6: MER_BWD_BATCH(3, false); break;
-        case 7: MER_BWD_BATCH(3, true); break;
-        case 8: MER_BWD_BATCH(4, false); break;
-        case 9: MER_BWD_BATCH(4, true); break;
-        default: return 1;
-    }
+    MER_BWD_DISPATCH(MER_BWD_BATCH);
 #undef MER_BWD_BATCH
     return cudaGetLastError() == cudaSuccess ? 0 : 2;
 }
@@ -849,29 +885,11 @@ extern "C" int mer_launch_backward(const mer_vertex* vpix, int V, const int* tri
     const long long blocks = (long long)a.ntx * a.nty * n;
     if (blocks == 0) return 0;
     const bool exact = (terms & MER_EXACT_CROSSING) != 0;
-#define MER_BWD(A, E)                                                                                             \
-    k_backward<A, E, kTableBits><<<(unsigned)blocks, kThreads, 0, s>>>(vpix, tris, index, cover, image, grad_image, attr, tex, a, \
-                                                           grad_vpix, grad_attr, ws)
+#define MER_BWD(F, A, E, BITS)                                                                                      \
+    k_backward<F, A, E, BITS><<<(unsigned)blocks, kThreads, 0, s>>>(vpix, tris, index, cover, image, grad_image, attr, \
+                                                                    tex, a, grad_vpix, grad_attr, ws)
     const bool dense = (double)T > kDenseTrianglesPerPixel * (double)H * (double)W;
-    switch (attr_channels(sh, grad_attr) * 2 + (exact ? 1 : 0)) {
-        case 0:
-            if (dense)
-                k_backward<0, false, kTableBitsDense><<<(unsigned)blocks, kThreads, 0, s>>>(
-                    vpix, tris, index, cover, image, grad_image, attr, tex, a, grad_vpix, grad_attr, ws);
-            else
-                MER_BWD(0, false);
-            break;
-        case 1: MER_BWD(0, true); break;
-        case 2: MER_BWD(1, false); break;
-        case 3: MER_BWD(1, true); break;
-        case 4: MER_BWD(2, false); break;
-        case 5: MER_BWD(2, true); break;
-        case 6: MER_BWD(3, false); break;
-        case 7: MER_BWD(3, true); break;
-        case 8: MER_BWD(4, false); break;
-        case 9: MER_BWD(4, true); break;
-        default: return 1;
-    }
+    MER_BWD_DISPATCH(MER_BWD);
 #undef MER_BWD
     return cudaGetLastError() == cudaSuccess ? 0 : 2;
 }

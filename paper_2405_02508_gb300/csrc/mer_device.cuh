@@ -171,11 +171,13 @@ __device__ __forceinline__ int floor_i(float x) { return __float2int_rd(x); }
 // r1 = r0 + r0 (1 - x r0) with both operations fused (the quadratic convergence of Newton's iteration for the
 // reciprocal; the residual is formed exactly by the FMA), so r1 is within about half an ulp of 1 / x and in
 // almost every case the correctly rounded value.  Zero, infinite and NaN inputs keep r0 (the residual of
-// 0 * inf is NaN there).  Three instructions instead of the correctly rounded reciprocal's longer sequence.
+// 0 * inf is NaN there); a denormal input counts as zero.  Five instructions; the approximate division
+// 1 / x that gave r0 before spent several more on scaling its operands.
 __device__ __forceinline__ float rcp_nr(float x) {
-    const float r0 = __fdividef(1.0f, x);
+    float r0;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(x));
     const float r1 = __fmaf_rn(r0, __fmaf_rn(-x, r0, 1.0f), r0);
-    return isfinite(r1) ? r1 : r0;
+    return r1 == r1 ? r1 : r0;
 }
 
 // Non-negative int64 -> float, exact below 2^23 with one integer add and one float subtract (the bits of
@@ -255,6 +257,11 @@ __device__ __forceinline__ float diff_of_products(float a, float d, float b, flo
     return f + e;
 }
 
+// a*b - c*d, the second product rounded.  The values that decide which texel cell a pixel reads (barycentrics, perspective
+// weights, texel coordinates) are written with their roundings fixed: left to the compiler, the contraction into FMAs
+// depends on the code around them, and a kernel's variants then disagree at cell borders, where the derivative jumps.
+__device__ __forceinline__ float det2(float a, float b, float c, float d) { return __fmaf_rn(a, b, -__fmul_rn(c, d)); }
+
 // A projected vertex record loaded with two 128-bit loads (records are 32-byte aligned).
 struct VRec {
     int X, Y;
@@ -304,19 +311,20 @@ __device__ __forceinline__ Bary screen_bary(const VRec v[3], int x, int y) {
     if ((span >> 16) == 0u) {
         // Every vertex within 128 px of the centre (the common case): |ix|, |iy| < 2^15, so the integer edge
         // functions fit 32 bits, the coordinates convert exactly, and differences of the converted
-        // coordinates are exact.  The same values as the general path below.
+        // coordinates are exact.  The same values as the general path below, with the powers of two that scale
+        // snapped units to pixels folded into the FMAs.
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
-            a[i] = __int2float_rn(ix[i]) * (1.0f / 256.0f);
-            b[i] = __int2float_rn(iy[i]) * (1.0f / 256.0f);
+            a[i] = __int2float_rn(ix[i]);
+            b[i] = __int2float_rn(iy[i]);
         }
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             const int j = (i + 1) % 3, k = (i + 2) % 3;
             const int E = ix[j] * iy[k] - iy[j] * ix[k];
-            const float lin = (a[j] * s[k] - s[j] * a[k]) + (r[j] * b[k] - b[j] * r[k]);
-            const float quad = r[j] * s[k] - s[j] * r[k];
-            e[i] = __fmaf_rn(__int2float_rn(E), 1.0f / 65536.0f, lin + quad);
+            const float lin = __fadd_rn(det2(a[j], s[k], s[j], a[k]), det2(r[j], b[k], b[j], r[k]));
+            const float quad = det2(r[j], s[k], s[j], r[k]);
+            e[i] = __fmaf_rn(__int2float_rn(E), 1.0f / 65536.0f, __fmaf_rn(lin, 1.0f / 256.0f, quad));
         }
         B.d = (e[0] + e[1]) + e[2];
         const float inv = rcp_nr(B.d);
@@ -324,8 +332,8 @@ __device__ __forceinline__ Bary screen_bary(const VRec v[3], int x, int y) {
         for (int i = 0; i < 3; ++i) {
             const int j = (i + 1) % 3, k = (i + 2) % 3;
             B.lam[i] = e[i] * inv;
-            B.gx[i] = ((b[j] - b[k]) + (s[j] - s[k])) * inv;
-            B.gy[i] = ((a[k] - a[j]) + (r[k] - r[j])) * inv;
+            B.gx[i] = __fmaf_rn(b[j] - b[k], 1.0f / 256.0f, s[j] - s[k]) * inv;
+            B.gy[i] = __fmaf_rn(a[k] - a[j], 1.0f / 256.0f, r[k] - r[j]) * inv;
         }
         return B;
     }
@@ -338,9 +346,9 @@ __device__ __forceinline__ Bary screen_bary(const VRec v[3], int x, int y) {
     for (int i = 0; i < 3; ++i) {
         const int j = (i + 1) % 3, k = (i + 2) % 3;
         const int64_t E = (int64_t)ix[j] * iy[k] - (int64_t)iy[j] * ix[k];
-        const float lin = (a[j] * s[k] - s[j] * a[k]) + (r[j] * b[k] - b[j] * r[k]);
-        const float quad = r[j] * s[k] - s[j] * r[k];
-        e[i] = __fmaf_rn(signed_ll2f_rn(E), 1.0f / 65536.0f, lin + quad);
+        const float lin = __fadd_rn(det2(a[j], s[k], s[j], a[k]), det2(r[j], b[k], b[j], r[k]));
+        const float quad = det2(r[j], s[k], s[j], r[k]);
+        e[i] = __fmaf_rn(signed_ll2f_rn(E), 1.0f / 65536.0f, __fadd_rn(lin, quad));
     }
     B.d = (e[0] + e[1]) + e[2];
     const float inv = rcp_nr(B.d);
@@ -366,27 +374,19 @@ struct TexCoord {
 
 __device__ __forceinline__ TexCoord tex_coord(float u0, float u1, float u2, float b1, float b2, int N) {
     const float u = u0 + (b1 * (u1 - u0) + b2 * (u2 - u0));
-    TexCoord t;
-    if (!(fabsf(u) < 1024.0f)) {
-        t.cell = -1;
-        t.frac = 0.5f;
-        return t;
-    }
+    const bool in = fabsf(u) < 1024.0f;
     const float Nf = (float)N;
-    const float xb = u0 * Nf - 0.5f;
-    const float d = b1 * ((u1 * Nf - 0.5f) - xb) + b2 * ((u2 * Nf - 0.5f) - xb);
+    const float xb = __fmaf_rn(u0, Nf, -0.5f);
+    const float d = __fmaf_rn(b1, __fmaf_rn(u1, Nf, -0.5f) - xb, __fmul_rn(b2, __fmaf_rn(u2, Nf, -0.5f) - xb));
     const int fli = floor_i(xb);
     const float fl = i2f_exact(fli);
     const float f = (xb - fl) + d;  // xb - fl is exact
     const int ci = floor_i(f);
-    float fr = f - i2f_exact(ci);
-    int cell = fli + ci;
-    if (fr >= 1.0f) {  // f just below an integer rounded up: the next cell at fraction 0
-        fr = 0.0f;
-        cell += 1;
-    }
-    t.cell = cell;
-    t.frac = fr;
+    const float fr = f - i2f_exact(ci);
+    const bool wrap = fr >= 1.0f;  // f just below an integer rounded up: the next cell at fraction 0
+    TexCoord t;
+    t.cell = in ? fli + ci + (wrap ? 1 : 0) : -1;
+    t.frac = in ? (wrap ? 0.0f : fr) : 0.5f;
     return t;
 }
 
@@ -408,15 +408,27 @@ __device__ __forceinline__ TexTaps tex_taps(int TH, int TW, TexCoord cx, TexCoor
     }
     t.i1 = (t.i0 + 1 == TW) ? 0 : t.i0 + 1;
     t.fx = cx.frac;
-    t.clamped = false;
-    if (cy.cell < 0) {
-        t.j0 = 0; t.j1 = TH > 1 ? 1 : 0; t.fy = 0.0f; t.clamped = true;
-    } else if (cy.cell > TH - 1 || (cy.cell == TH - 1 && cy.frac > 0.0f)) {
-        t.j0 = TH - 1; t.j1 = TH - 1; t.fy = 0.0f; t.clamped = true;
-    } else {
-        t.j0 = cy.cell; t.j1 = t.j0 + 1 < TH ? t.j0 + 1 : TH - 1; t.fy = cy.frac;
-    }
+    t.clamped = cy.cell < 0 || cy.cell > TH - 1 || (cy.cell == TH - 1 && cy.frac > 0.0f);
+    t.j0 = min(max(cy.cell, 0), TH - 1);
+    t.j1 = min(t.j0 + 1, TH - 1);
+    t.fy = t.clamped ? 0.0f : cy.frac;
     return t;
+}
+
+// The four texels of a lookup in a texture of float4 texels with at most 2^27 of them (32-bit texel numbers).
+struct TexQuad {
+    float4 a00, a10, a01, a11;  // (i0, j0), (i1, j0), (i0, j1), (i1, j1)
+};
+
+__device__ __forceinline__ TexQuad tex_quad(const float* __restrict__ tex, int TW, const TexTaps& t) {
+    const float4* q = reinterpret_cast<const float4*>(tex);
+    const unsigned r0 = (unsigned)t.j0 * (unsigned)TW, r1 = (unsigned)t.j1 * (unsigned)TW;
+    TexQuad v;
+    v.a00 = __ldg(q + (r0 + (unsigned)t.i0));
+    v.a10 = __ldg(q + (r0 + (unsigned)t.i1));
+    v.a01 = __ldg(q + (r1 + (unsigned)t.i0));
+    v.a11 = __ldg(q + (r1 + (unsigned)t.i1));
+    return v;
 }
 
 // Texel (j, i) of a texture with `stride` floats per texel; vec4: stride == 4 and 16-byte aligned (one
@@ -435,6 +447,21 @@ __device__ __forceinline__ float4 texel4(const float* __restrict__ tex, int TW, 
 
 __device__ __forceinline__ float comp(const float4& v, int c) { return c == 0 ? v.x : (c == 1 ? v.y : (c == 2 ? v.z : v.w)); }
 
+// One channel's bilinear value, and g times its derivatives along the texel axes added to (su, sv).
+__device__ __forceinline__ float tex_lerp(float t00, float t10, float t01, float t11, const TexTaps& t) {
+    const float a = t00 + t.fx * (t10 - t00);
+    const float b = t01 + t.fx * (t11 - t01);
+    return a + t.fy * (b - a);
+}
+
+__device__ __forceinline__ void tex_lerp_grad(float t00, float t10, float t01, float t11, const TexTaps& t, float g,
+                                              float& su, float& sv) {
+    su += g * ((1.0f - t.fy) * (t10 - t00) + t.fy * (t11 - t01));
+    const float a = t00 + t.fx * (t10 - t00);
+    const float b = t01 + t.fx * (t11 - t01);
+    sv += g * (b - a);
+}
+
 // Bilinear values of channels 0..nc-1 written to out[0..nc-1].
 __device__ __forceinline__ void tex_values(const float* __restrict__ tex, int TW, int stride, bool vec4, int nc,
                                            const TexTaps& t, float* out) {
@@ -445,9 +472,7 @@ __device__ __forceinline__ void tex_values(const float* __restrict__ tex, int TW
         for (int c = 0; c < 4; ++c) {
             if (c >= nc) break;
             const float t00 = comp(a00, c), t10 = comp(a10, c), t01 = comp(a01, c), t11 = comp(a11, c);
-            const float a = t00 + t.fx * (t10 - t00);
-            const float b = t01 + t.fx * (t11 - t01);
-            out[c] = a + t.fy * (b - a);
+            out[c] = tex_lerp(t00, t10, t01, t11, t);
         }
         return;
     }
@@ -456,9 +481,7 @@ __device__ __forceinline__ void tex_values(const float* __restrict__ tex, int TW
     for (int c = 0; c < nc; ++c) {
         const float t00 = __ldg(r0 + (size_t)t.i0 * stride + c), t10 = __ldg(r0 + (size_t)t.i1 * stride + c);
         const float t01 = __ldg(r1 + (size_t)t.i0 * stride + c), t11 = __ldg(r1 + (size_t)t.i1 * stride + c);
-        const float a = t00 + t.fx * (t10 - t00);
-        const float b = t01 + t.fx * (t11 - t01);
-        out[c] = a + t.fy * (b - a);
+        out[c] = tex_lerp(t00, t10, t01, t11, t);
     }
 }
 
@@ -474,11 +497,7 @@ __device__ __forceinline__ void tex_grad_uv(const float* __restrict__ tex, int T
         for (int c = 0; c < 4; ++c) {
             if (c >= nc) break;
             const float t00 = comp(a00, c), t10 = comp(a10, c), t01 = comp(a01, c), t11 = comp(a11, c);
-            const float gc = __ldg(g + c);
-            su += gc * ((1.0f - t.fy) * (t10 - t00) + t.fy * (t11 - t01));
-            const float a = t00 + t.fx * (t10 - t00);
-            const float b = t01 + t.fx * (t11 - t01);
-            sv += gc * (b - a);
+            tex_lerp_grad(t00, t10, t01, t11, t, __ldg(g + c), su, sv);
         }
     } else {
         const float* r0 = tex + (size_t)t.j0 * TW * stride;
@@ -486,11 +505,7 @@ __device__ __forceinline__ void tex_grad_uv(const float* __restrict__ tex, int T
         for (int c = 0; c < nc; ++c) {
             const float t00 = __ldg(r0 + (size_t)t.i0 * stride + c), t10 = __ldg(r0 + (size_t)t.i1 * stride + c);
             const float t01 = __ldg(r1 + (size_t)t.i0 * stride + c), t11 = __ldg(r1 + (size_t)t.i1 * stride + c);
-            const float gc = __ldg(g + c);
-            su += gc * ((1.0f - t.fy) * (t10 - t00) + t.fy * (t11 - t01));
-            const float a = t00 + t.fx * (t10 - t00);
-            const float b = t01 + t.fx * (t11 - t01);
-            sv += gc * (b - a);
+            tex_lerp_grad(t00, t10, t01, t11, t, __ldg(g + c), su, sv);
         }
     }
     gu = (float)TW * su;

@@ -356,8 +356,8 @@ __device__ __forceinline__ void raster_class(RasterShared<TS>& S, int n, int ox,
     }
 }
 
-// SHADE: also shade every pixel of the tile from its z-buffer winner (shade_fragment, as the deferred
-// shading kernels do from the index image).
+// FORM (ShadeForm): also shade every pixel of the tile from its z-buffer winner (shade_fragment, as the deferred
+// shading kernels do from the index image); kShadeOff: no shading.
 // cover (optional): one byte a pixel (MER_COVER_* bits): whether another triangle of the winner's facing,
 // or one of the other facing, covers the pixel centre, the facing of the winner and which borders of its bin
 // tile the pixel lies on, from the kCov* bits.  The counts leave out the triangles of the second part that
@@ -366,7 +366,7 @@ __device__ __forceinline__ void raster_class(RasterShared<TS>& S, int n, int ox,
 // The tile's list holds the camera-facing triangles first (nfront of them) and the others after; before
 // the second part the tile's smallest depth key is taken, and a triangle of that part whose largest vertex
 // zeta (with a margin above the FP32 rounding of the key) is below it cannot win any pixel: it is skipped.
-template <int TS, bool SHADE>
+template <int TS, int FORM>
 __device__ __forceinline__ void raster_tile(const RItem& it, int local_tile, const int* __restrict__ offs,
                                             const int* __restrict__ cnts, const int* __restrict__ nfront,
                                             const int* __restrict__ list, bool overflow, RasterShared<TS>& S,
@@ -437,10 +437,10 @@ __device__ __forceinline__ void raster_tile(const RItem& it, int local_tile, con
             }
             cover[p] = (unsigned char)c;
         }
-        if (SHADE)
-            shade_fragment(it.vpix, it.V, it.tris, it.T, t, px, py,
-                           so.attr ? so.attr + (size_t)it.vert * so.a.sh.C_attr : nullptr, so.tex, so.a,
-                           so.image + p * so.a.sh.C, ws);
+        if (FORM != kShadeOff)
+            shade_fragment<FORM, false>(it.vpix, it.V, it.tris, it.T, t, px, py,
+                                        so.attr ? so.attr + (size_t)it.vert * so.a.sh.C_attr : nullptr, so.tex, so.a,
+                                        so.image + p * so.a.sh.C, ws);
         if (!depth && !bary) continue;
         float Z = 0.f, b1 = 0.f, b2 = 0.f;
         if (t >= 0) {
@@ -517,7 +517,7 @@ __global__ void __launch_bounds__(kRasterThreads, kRasterCtasPerSm) k_raster(Tri
     const int local = (int)(tile % g.tiles_per_view);
     ShadeOut none;
     none.attr = nullptr; none.tex = nullptr; none.image = nullptr;
-    raster_tile<TS, false>(view_item(g, vpix, tris, recs, view), local, offs, cnts, nfront, list, overflow, S, index,
+    raster_tile<TS, kShadeOff>(view_item(g, vpix, tris, recs, view), local, offs, cnts, nfront, list, overflow, S, index,
                            depth, bary, cover, none, ws);
 }
 
@@ -565,7 +565,7 @@ __global__ void k_bin_fill_batch(const mer_vertex* __restrict__ vpix, const int*
 }
 
 // Persistent: each CTA takes the next global tile from the work queue until none is left.
-template <int TS, bool SHADE>
+template <int TS, int FORM>
 __global__ void __launch_bounds__(kRasterThreads, kRasterCtasPerSm) k_raster_batch(TriRaster* __restrict__ recs, BatchGeom b,
                                                                  const int* __restrict__ offs,
                                                                  const int* __restrict__ cnts,
@@ -595,7 +595,7 @@ __global__ void __launch_bounds__(kRasterThreads, kRasterCtasPerSm) k_raster_bat
             hi = lo + (long long)((c.W + TS - 1) / TS) * ((c.H + TS - 1) / TS);
         }
         const mer_item m = b.items[cur];
-        raster_tile<TS, SHADE>(batch_item(m, b.tile, vpix, tris, recs), (int)(g - m.tile), offs, cnts, nfront, list,
+        raster_tile<TS, FORM>(batch_item(m, b.tile, vpix, tris, recs), (int)(g - m.tile), offs, cnts, nfront, list,
                                overflow, S, index, depth, bary, cover, so, ws);  // ends with a barrier: s_tile may be overwritten after it
     }
 }
@@ -696,7 +696,7 @@ extern "C" size_t mer_batch_raster_workspace_size(long long tiles, long long tre
     return layout_for(tiles, trecs, capacity).total;
 }
 
-template <int TS, bool SHADE>
+template <int TS, int FORM>
 static int launch_raster_batch(unsigned grid, TriRaster* recs, BatchGeom b, const int* offs, const int* counts,
                                const int* nfront, const int* list, const mer_vertex* vpix, const int* tris, void* hdr, long long capacity,
                                int* index, float* depth, float* bary, unsigned char* cover, const ShadeOut& so,
@@ -705,25 +705,25 @@ static int launch_raster_batch(unsigned grid, TriRaster* recs, BatchGeom b, cons
         int per_sm = 0, sms = 0, dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess) return 2;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 2;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_raster_batch<TS, SHADE>, kRasterThreads, 0) !=
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_raster_batch<TS, FORM>, kRasterThreads, 0) !=
             cudaSuccess)
             return 2;
         grid = (unsigned)(sms * (per_sm > 0 ? per_sm : 1));
     }
-    k_raster_batch<TS, SHADE><<<grid, kRasterThreads, 0, s>>>(recs, b, offs, counts, nfront, list, vpix, tris, hdr, capacity,
+    k_raster_batch<TS, FORM><<<grid, kRasterThreads, 0, s>>>(recs, b, offs, counts, nfront, list, vpix, tris, hdr, capacity,
                                                               index, depth, bary, cover, so);
     return 0;
 }
 
-template <bool SHADE>
+template <int FORM>
 static int launch_raster_batch_tile(int tile, unsigned grid, TriRaster* recs, BatchGeom b, const int* offs,
                                     const int* counts, const int* nfront, const int* list, const mer_vertex* vpix, const int* tris,
                                     void* hdr, long long capacity, int* index, float* depth, float* bary,
                                     unsigned char* cover, const ShadeOut& so, cudaStream_t s) {
     switch (tile) {
-        case 16: return launch_raster_batch<16, SHADE>(grid, recs, b, offs, counts, nfront, list, vpix, tris, hdr, capacity, index, depth, bary, cover, so, s);
-        case 32: return launch_raster_batch<32, SHADE>(grid, recs, b, offs, counts, nfront, list, vpix, tris, hdr, capacity, index, depth, bary, cover, so, s);
-        case 64: return launch_raster_batch<64, SHADE>(grid, recs, b, offs, counts, nfront, list, vpix, tris, hdr, capacity, index, depth, bary, cover, so, s);
+        case 16: return launch_raster_batch<16, FORM>(grid, recs, b, offs, counts, nfront, list, vpix, tris, hdr, capacity, index, depth, bary, cover, so, s);
+        case 32: return launch_raster_batch<32, FORM>(grid, recs, b, offs, counts, nfront, list, vpix, tris, hdr, capacity, index, depth, bary, cover, so, s);
+        case 64: return launch_raster_batch<64, FORM>(grid, recs, b, offs, counts, nfront, list, vpix, tris, hdr, capacity, index, depth, bary, cover, so, s);
         default: return 1;
     }
 }
@@ -755,10 +755,18 @@ static int batch_raster(const mer_vertex* vpix, const int* tris, const mer_item*
         const unsigned grid = persistent_ctas > 0 ? (unsigned)persistent_ctas : 0u;
         ShadeOut none;
         none.attr = nullptr; none.tex = nullptr; none.image = nullptr;
-        const int rc = so ? launch_raster_batch_tile<true>(tile, grid, recs, b, offs, counts, cursor, list, vpix, tris, hdr,
-                                                           capacity, index, depth, bary, cover, *so, s)
-                          : launch_raster_batch_tile<false>(tile, grid, recs, b, offs, counts, cursor, list, vpix, tris, hdr,
-                                                            capacity, index, depth, bary, cover, none, s);
+        const ShadeOut& o = so ? *so : none;
+        int rc = 0;
+#define MER_RASTER(F) \
+    rc = launch_raster_batch_tile<F>(tile, grid, recs, b, offs, counts, cursor, list, vpix, tris, hdr, capacity, index, depth, \
+                                     bary, cover, o, s)
+        switch (so ? shade_form(so->attr, so->tex, &so->a.sh) : kShadeOff) {
+            case kShadeOff: MER_RASTER(kShadeOff); break;
+            case kTex3: MER_RASTER(kTex3); break;
+            case kAttr3: MER_RASTER(kAttr3); break;
+            default: MER_RASTER(kGeneric); break;
+        }
+#undef MER_RASTER
         if (rc) return rc;
     }
     return cudaGetLastError() == cudaSuccess ? 0 : 2;
