@@ -178,6 +178,42 @@ int mer_project_screen(const double* scr, int V, int n, mer_vertex* vpix, void* 
 int mer_rasterize(const mer_vertex* vpix, int V, const int32_t* tris, int T, int n, int H, int W,
                   int tile, void* workspace, size_t workspace_bytes,
                   int32_t* index, float* depth, float* bary, uint8_t* cover, void* stream);
+/* One mesh seen by n cameras, with the caller's buffers: what the three calls below work on. */
+typedef struct mer_view {
+    const int32_t* tris;
+    int V, T, n, H, W, tile;
+    void* workspace; /* as for mer_rasterize */
+    size_t workspace_bytes;
+    mer_vertex* vpix;       /* [n, V] */
+    int32_t* index;         /* [n, H, W] */
+    uint8_t* cover;         /* [n, H, W] or NULL */
+    float* image;           /* [n, H, W, C] */
+    const float* bg_host;   /* HOST pointer to C floats, or NULL (0) */
+    const mer_shading* sh;  /* HOST pointer */
+} mer_view;
+
+/* A whole forward pass: mer_project, mer_rasterize and mer_shade with the same results, the shading in the
+ * rasterizer's last pass (Supp. B's modules in order).  depth / bary: optional outputs of mer_rasterize.
+ * vpix_copy / index_copy / image_copy (all or none): second copies of those outputs, written by the same kernels.
+ * host_status (or NULL): two int64 words of page-locked HOST memory that the device can write.  With it the call also
+ * does mer_sync_status's part for the rasterization: it returns MER_EOVERFLOW / MER_ERANGE / MER_EFIXED (clearing the
+ * status word) and sets *total_bins, after waiting only until the binning is done; the rest is still queued.  A
+ * capturing stream cannot be waited for: MER_ECUDA. */
+int mer_view_render(const mer_view* v, const float* verts, const mer_camera* cams, const float* attr,
+                    const float* tex, float* depth, float* bary, mer_vertex* vpix_copy, int32_t* index_copy,
+                    float* image_copy, int64_t* host_status, int64_t* total_bins, void* stream);
+
+/* A whole backward pass from v's vpix, index, image and cover: mer_backward, then mer_project_backward.
+ * zero: 0 all gradients are added to; 1 grad_vpix and grad_verts are overwritten; 2 grad_attr (if given) too.
+ * grad_verts_copy (or NULL): a second copy of grad_verts. */
+int mer_view_backward(const mer_view* v, const mer_camera* cams, const float* grad_image, const float* attr,
+                      const float* tex, int terms, double* grad_vpix, float* grad_attr, float* grad_verts,
+                      float* grad_verts_copy, int zero, void* stream);
+
+/* mer_project_jvp, then mer_forward_grad, from v's vpix, index and image; tangent_vpix [n, V, 3] is scratch. */
+int mer_view_forward_grad(const mer_view* v, const mer_camera* cams, const float* tangent_world, const float* attr,
+                          const float* tex, int terms, float* tangent_vpix, float* out, void* stream);
+
 /* mer_project followed by mer_rasterize: world-space vertices [V,3] and n cameras in, index / depth /
  * bary out, the projected records written to vpix [n,V] (the other calls take them).  Arguments, errors and
  * workspace as the two calls. */

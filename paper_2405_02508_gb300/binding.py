@@ -47,6 +47,15 @@ class MerBatchTotals(ctypes.Structure):
                 ("tile", ctypes.c_int), ("mesh_rows", ctypes.c_int64), ("max_tri_density", ctypes.c_double)]
 
 
+class MerView(ctypes.Structure):
+    """One mesh seen by n cameras, with the caller's buffers (mer_view)."""
+    _fields_ = [("tris", ctypes.c_void_p), ("V", ctypes.c_int), ("T", ctypes.c_int), ("n", ctypes.c_int),
+                ("H", ctypes.c_int), ("W", ctypes.c_int), ("tile", ctypes.c_int), ("workspace", ctypes.c_void_p),
+                ("workspace_bytes", ctypes.c_size_t), ("vpix", ctypes.c_void_p), ("index", ctypes.c_void_p),
+                ("cover", ctypes.c_void_p), ("image", ctypes.c_void_p), ("bg_host", ctypes.c_void_p),
+                ("sh", ctypes.POINTER(MerShading))]
+
+
 # (name, argtypes, restype); P = pointer, I = int, Z = size_t, L = int64
 _P, _I, _Z, _L = ctypes.c_void_p, ctypes.c_int, ctypes.c_size_t, ctypes.c_int64
 _SIGS = {
@@ -71,6 +80,9 @@ _SIGS = {
     "mer_vertex_normals_backward": ([_P, _I, _P, ctypes.c_int64, _P, _P, _P, _P, _P], _I),
     "mer_l2_loss_grad": ([_P, _P, ctypes.c_int64, _P, _P, _P], _I),
     "mer_rasterize_world": ([_P, _I, _P, _I, _P, _I, _I, _I, _I, _P, _Z, _P, _P, _P, _P, _P], _I),
+    "mer_view_render": ([ctypes.POINTER(MerView), _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, ctypes.POINTER(ctypes.c_int64), _P], _I),
+    "mer_view_backward": ([ctypes.POINTER(MerView), _P, _P, _P, _P, _I, _P, _P, _P, _P, _I, _P], _I),
+    "mer_view_forward_grad": ([ctypes.POINTER(MerView), _P, _P, _P, _P, _I, _P, _P, _P], _I),
     "mer_laplacian_csr": ([_P, ctypes.c_int64, ctypes.c_int64, _P, _P], _I),
     "mer_precond_apply": ([_P, _P, ctypes.c_int64, ctypes.c_float, _P, _P, _P], _I),
     "mer_precond_solve_workspace_size": ([ctypes.c_int64], _Z),
@@ -139,11 +151,11 @@ def _ptr(t: torch.Tensor | None):
         raise ValueError("libmer takes device tensors")
     if not t.is_contiguous():
         raise ValueError("libmer takes contiguous tensors")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _nbytes(t: torch.Tensor | None) -> int:
@@ -279,6 +291,41 @@ def mer_vertex_normals_backward(verts, tris, acc, grad_normals, grad_verts, stat
 def mer_l2_loss_grad(image, target, grad, loss):
     _check(lib().mer_l2_loss_grad(_ptr(image), _ptr(target), image.numel(), _ptr(grad), _ptr(loss), _stream()),
            "mer_l2_loss_grad")
+
+
+def view_struct(tris, V, n, H, W, tile, workspace, vpix, index, cover, image, sh: MerShading, bg=None) -> MerView:
+    """The mer_view of these tensors, for one call (it holds plain pointers); bg: the background values (rendering)."""
+    v = MerView(_ptr(tris), V, tris.shape[0], n, H, W, tile, _ptr(workspace), _nbytes(workspace), _ptr(vpix),
+                _ptr(index), _ptr(cover), _ptr(image), None, ctypes.pointer(sh))
+    if bg is not None:
+        v.keep = (ctypes.c_float * max(1, sh.C))(*[float(x) for x in bg])
+        v.bg_host = ctypes.addressof(v.keep)
+    return v
+
+
+def mer_view_render(view: MerView, verts, cams, attr, tex, depth=None, bary=None, copies=(None, None, None),
+                    host_status: torch.Tensor | None = None) -> tuple[int, int]:
+    """copies: (vpix, index, image) tensors that receive second copies; host_status: two int64 in pinned memory.
+    Returns (code, bin entries); the code is MER_OK, or the device status if host_status is given."""
+    tot = ctypes.c_int64(0)
+    code = lib().mer_view_render(view, _ptr(verts), _ptr(cams), _ptr(attr), _ptr(tex), _ptr(depth), _ptr(bary),
+                                 _ptr(copies[0]), _ptr(copies[1]), _ptr(copies[2]),
+                                 None if host_status is None else host_status.data_ptr(), tot, _stream())
+    if code in (MER_EINVAL, MER_ECUDA):
+        raise MerError(code, "mer_view_render")
+    return code, tot.value
+
+
+def mer_view_backward(view: MerView, cams, grad_image, attr, tex, terms: int, grad_vpix, grad_attr, grad_verts,
+                      grad_verts_copy=None, zero: int = 1):
+    _check(lib().mer_view_backward(view, _ptr(cams), _ptr(grad_image), _ptr(attr), _ptr(tex), terms, _ptr(grad_vpix),
+                                   _ptr(grad_attr), _ptr(grad_verts), _ptr(grad_verts_copy), zero, _stream()),
+           "mer_view_backward")
+
+
+def mer_view_forward_grad(view: MerView, cams, tangent_world, attr, tex, terms: int, tangent_vpix, out):
+    _check(lib().mer_view_forward_grad(view, _ptr(cams), _ptr(tangent_world), _ptr(attr), _ptr(tex), terms,
+                                       _ptr(tangent_vpix), _ptr(out), _stream()), "mer_view_forward_grad")
 
 
 def mer_rasterize_world(verts, tris, cams, H, W, tile, workspace, index, vpix, depth=None, bary=None):

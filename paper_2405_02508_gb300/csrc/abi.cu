@@ -6,10 +6,14 @@
 
 #include "mer_device.cuh"
 
-extern "C" int mer_launch_project(const float*, int, const mer_camera*, int, mer_vertex*, cudaStream_t);
+extern "C" int mer_launch_project(const float*, int, const mer_camera*, int, mer_vertex*, mer_vertex*, int*, long long,
+                                  cudaStream_t);
 extern "C" int mer_launch_project_screen(const double*, int, int, mer_vertex*, cudaStream_t);
-extern "C" int mer_launch_project_backward(int, const mer_camera*, int, const mer_vertex*, const double*, float*,
-                                           cudaStream_t);
+extern "C" int mer_launch_project_backward(int, const mer_camera*, int, const mer_vertex*, const double*, float*, float*,
+                                           int, cudaStream_t);
+extern "C" int mer_launch_clear(double*, long long, float*, long long, cudaStream_t);
+extern "C" int mer_launch_view_render(const mer_view*, const float*, const mer_camera*, const float*, const float*, float*,
+                                      float*, mer_vertex*, int*, float*, long long*, cudaStream_t);
 extern "C" size_t mer_raster_workspace_size(int, int, int, int, int, int, long long);
 extern "C" int mer_launch_rasterize(const mer_vertex*, int, const int*, int, int, int, int, int, void*, size_t, int*,
                                     float*, float*, unsigned char*, cudaStream_t);
@@ -117,7 +121,7 @@ int mer_project(const float* verts, int V, const mer_camera* cams, int n, mer_ve
     if (V < 0 || n < 0) return MER_EINVAL;
     if ((long long)V * n == 0) return MER_OK;
     if (!verts || !cams || !vpix) return MER_EINVAL;
-    return mer_launch_project(verts, V, cams, n, vpix, S(stream));
+    return mer_launch_project(verts, V, cams, n, vpix, nullptr, nullptr, 0, S(stream));
 }
 
 int mer_rasterize_world(const float* verts, int V, const int32_t* tris, int T, const mer_camera* cams, int n, int H,
@@ -242,7 +246,121 @@ int mer_project_backward(int V, const mer_camera* cams, int n, const mer_vertex*
     if (V < 0 || n < 0) return MER_EINVAL;
     if ((long long)V * n == 0) return MER_OK;
     if (!cams || !vpix || !grad_vpix || !grad_verts) return MER_EINVAL;
-    return mer_launch_project_backward(V, cams, n, vpix, grad_vpix, grad_verts, S(stream));
+    return mer_launch_project_backward(V, cams, n, vpix, grad_vpix, grad_verts, nullptr, 0, S(stream));
+}
+
+// ---- one mesh, n views: whole passes ----
+
+// Clears the sticky status word and turns it into a code (the stream has reached the point that set it).
+static int take_status(int status, void* workspace, cudaStream_t s) {
+    if (status != 0) {
+        const int zero = 0;
+        if (cudaMemcpyAsync(workspace, &zero, sizeof(int), cudaMemcpyHostToDevice, s) != cudaSuccess) return MER_ECUDA;
+        if (cudaStreamSynchronize(s) != cudaSuccess) return MER_ECUDA;
+    }
+    if (status & mer::kStatusOverflow) return MER_EOVERFLOW;
+    if (status & mer::kStatusRange) return MER_ERANGE;
+    if (status & mer::kStatusFixed) return MER_EFIXED;
+    return MER_OK;
+}
+
+// Waits until the device has written the two host words (the kernel that does is queued on s).  Polling them costs a
+// microsecond or two; a copy to the host and a synchronisation of the stream waited for the whole raster as well.  Ends
+// when the stream does: if it is idle or has failed without the words, that is an error.
+static int wait_words(int64_t* host, cudaStream_t s) {
+    const int64_t ready = (int64_t)1 << 32;
+    for (unsigned k = 1;; ++k) {
+        if (__atomic_load_n(host, __ATOMIC_ACQUIRE) >= ready) return MER_OK;
+        if (k % 4096 == 0) {
+            const cudaError_t e = cudaStreamQuery(s);
+            if (e == cudaErrorNotReady) {
+                (void)cudaGetLastError();  // not an error
+                continue;
+            }
+            if (e != cudaSuccess) return MER_ECUDA;
+            return __atomic_load_n(host, __ATOMIC_ACQUIRE) >= ready ? MER_OK : MER_ECUDA;
+        }
+    }
+}
+
+static bool view_ok(const mer_view* v) {
+    return v && v->V >= 0 && v->T >= 0 && dims_ok(v->n, v->H, v->W) && shading_ok(v->sh) &&
+           (v->tile == 8 || v->tile == 16 || v->tile == 32);
+}
+
+int mer_view_render(const mer_view* v, const float* verts, const mer_camera* cams, const float* attr, const float* tex,
+                    float* depth, float* bary, mer_vertex* vpix_copy, int32_t* index_copy, float* image_copy,
+                    int64_t* host_status, int64_t* total_bins, void* stream) {
+    if (!view_ok(v)) return MER_EINVAL;
+    const long long px = (long long)v->n * v->H * v->W, rows = (long long)v->n * v->V;
+    if (rows > 0 && (!verts || !cams || !v->vpix)) return MER_EINVAL;
+    const bool copies = vpix_copy || index_copy || image_copy;
+    if (copies && (!index_copy || !image_copy || (rows > 0 && !vpix_copy))) return MER_EINVAL;
+    if (px > 0) {
+        if (!v->workspace || !aligned256(v->workspace) || !v->index || !v->image) return MER_EINVAL;
+        if (v->T > 0 && (!v->tris || !v->vpix)) return MER_EINVAL;
+        if (v->workspace_bytes < mer_raster_workspace_size(v->V, v->T, v->n, v->H, v->W, v->tile, 1)) return MER_EINVAL;
+        if (v->sh->n_main > 0 && !attr) return MER_EINVAL;
+        if (v->sh->uv_offset >= 0 && !tex) return MER_EINVAL;
+    }
+    cudaStream_t s = S(stream);
+    if (host_status) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return MER_ECUDA;
+    }
+    if (px == 0 || rows == 0 || v->T == 0) {  // nothing to draw or nowhere to draw it
+        int rc = mer_project(verts, v->V, cams, v->n, v->vpix, stream);
+        if (rc == MER_OK)
+            rc = mer_rasterize(v->vpix, v->V, v->tris, v->T, v->n, v->H, v->W, v->tile, v->workspace, v->workspace_bytes,
+                               v->index, depth, bary, v->cover, stream);
+        if (rc == MER_OK && host_status && v->workspace) rc = mer_sync_status(v->workspace, total_bins, stream);
+        if (rc == MER_OK)
+            rc = mer_shade(v->vpix, v->V, v->tris, v->T, v->n, v->H, v->W, v->index, attr, tex, v->bg_host, v->sh, v->image,
+                           v->workspace, stream);
+        if (rc != MER_OK || !copies) return rc;
+        if (rows > 0 && cudaMemcpyAsync(vpix_copy, v->vpix, rows * sizeof(mer_vertex), cudaMemcpyDeviceToDevice, s) != cudaSuccess)
+            return MER_ECUDA;
+        if (px > 0 &&
+            (cudaMemcpyAsync(index_copy, v->index, px * sizeof(int), cudaMemcpyDeviceToDevice, s) != cudaSuccess ||
+             cudaMemcpyAsync(image_copy, v->image, px * v->sh->C * sizeof(float), cudaMemcpyDeviceToDevice, s) != cudaSuccess))
+            return MER_ECUDA;
+        return MER_OK;
+    }
+    if (host_status) __atomic_store_n(host_status, (int64_t)0, __ATOMIC_RELEASE);
+    const int rc = mer_launch_view_render(v, verts, cams, attr, tex, depth, bary, vpix_copy, index_copy, image_copy,
+                                          reinterpret_cast<long long*>(host_status), s);
+    if (rc != MER_OK || !host_status) return rc;
+    if (wait_words(host_status, s) != MER_OK) return MER_ECUDA;
+    if (total_bins) *total_bins = __atomic_load_n(host_status + 1, __ATOMIC_ACQUIRE);
+    return take_status((int)(__atomic_load_n(host_status, __ATOMIC_ACQUIRE) & 0xffffffff), v->workspace, s);
+}
+
+int mer_view_backward(const mer_view* v, const mer_camera* cams, const float* grad_image, const float* attr,
+                      const float* tex, int terms, double* grad_vpix, float* grad_attr, float* grad_verts,
+                      float* grad_verts_copy, int zero, void* stream) {
+    if (!view_ok(v)) return MER_EINVAL;
+    const long long rows = (long long)v->n * v->V;
+    if (zero < 0 || zero > 2) return MER_EINVAL;
+    if (rows > 0 && (!cams || !v->vpix || !grad_vpix || !grad_verts)) return MER_EINVAL;
+    cudaStream_t s = S(stream);
+    if (zero) {
+        const int rc = mer_launch_clear(grad_vpix, 3 * rows, grad_attr,
+                                        zero > 1 && grad_attr ? (long long)v->V * v->sh->C_attr : 0, s);
+        if (rc) return rc;
+    }
+    const int rc = mer_backward(v->vpix, v->V, v->tris, v->T, v->n, v->H, v->W, v->index, v->cover, v->image, grad_image, attr,
+                                tex, v->sh, terms, grad_vpix, grad_attr, v->workspace, v->workspace_bytes, stream);
+    if (rc != MER_OK) return rc;
+    return mer_launch_project_backward(v->V, cams, v->n, v->vpix, grad_vpix, grad_verts, grad_verts_copy, zero, s);
+}
+
+int mer_view_forward_grad(const mer_view* v, const mer_camera* cams, const float* tangent_world, const float* attr,
+                          const float* tex, int terms, float* tangent_vpix, float* out, void* stream) {
+    if (!view_ok(v)) return MER_EINVAL;
+    const int rc = mer_project_jvp(tangent_world, v->V, cams, v->n, v->vpix, tangent_vpix, stream);
+    if (rc != MER_OK) return rc;
+    return mer_forward_grad(v->vpix, v->V, v->tris, v->T, v->n, v->H, v->W, v->index, v->image, tangent_vpix, attr, tex, v->sh,
+                            terms, out, v->workspace, stream);
 }
 
 // ---- batched path ----

@@ -11,7 +11,8 @@
 
 namespace mer {
 
-__device__ __forceinline__ void write_vertex(double xs, double ys, double zeta, bool front, mer_vertex* out) {
+__device__ __forceinline__ void write_vertex(double xs, double ys, double zeta, bool front, mer_vertex* out,
+                                             mer_vertex* out2 = nullptr) {
     mer_vertex r;
     r.X = 0; r.Y = 0; r.rx = 0.f; r.ry = 0.f; r.zeta = 0.f; r.zeta_lo = 0.f; r.flags = 0u; r.pad = 0.f;
     if (front) {
@@ -29,9 +30,11 @@ __device__ __forceinline__ void write_vertex(double xs, double ys, double zeta, 
         r.zeta_lo = __double2float_rn(__dsub_rn(zeta, (double)r.zeta));
     }
     *out = r;
+    if (out2) *out2 = r;
 }
 
-__device__ __forceinline__ void project_one(const float* __restrict__ w, const mer_camera& c, mer_vertex* out) {
+__device__ __forceinline__ void project_one(const float* __restrict__ w, const mer_camera& c, mer_vertex* out,
+                                            mer_vertex* out2 = nullptr) {
     const double x = w[0], y = w[1], z = w[2];
     const double* R = c.R;
     const double Xc = __dadd_rn(__dadd_rn(__dadd_rn(__dmul_rn(R[0], x), __dmul_rn(R[1], y)), __dmul_rn(R[2], z)), c.t[0]);
@@ -44,15 +47,19 @@ __device__ __forceinline__ void project_one(const float* __restrict__ w, const m
         xs = __dadd_rn(__dmul_rn(__dmul_rn(c.fx, Xc), zeta), c.cx);
         ys = __dadd_rn(__dmul_rn(__dmul_rn(c.fy, Yc), zeta), c.cy);
     }
-    write_vertex(xs, ys, zeta, front, out);
+    write_vertex(xs, ys, zeta, front, out, out2);
 }
 
+// out2 (optional): a second copy.  clear (optional): n_clear words set to zero (the raster's tile counts, which the next
+// kernel adds to: one launch less).
 __global__ void k_project(const float* __restrict__ verts, int V, const mer_camera* __restrict__ cams, int n,
-                          mer_vertex* __restrict__ out) {
+                          mer_vertex* __restrict__ out, mer_vertex* __restrict__ out2, int* __restrict__ clear,
+                          long long n_clear) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    for (long long k = i; k < n_clear; k += (long long)gridDim.x * blockDim.x) clear[k] = 0;
     if (i >= (long long)V * n) return;
     const int view = (int)(i / V), v = (int)(i % V);
-    project_one(verts + 3 * (size_t)v, cams[view], out + i);
+    project_one(verts + 3 * (size_t)v, cams[view], out + i, out2 ? out2 + i : nullptr);
 }
 
 __global__ void k_project_batch(const float* __restrict__ verts, const mer_camera* __restrict__ cams,
@@ -159,10 +166,12 @@ __global__ void k_world_finalize(const unsigned long long* __restrict__ acc, lon
     grad_verts[i] += __double2float_rn((double)hi * (1.0 / 1048576.0) + (double)(lo & 0xffffffffll) * (1.0 / 4503599627370496.0));
 }
 
-// One thread per vertex, looping over the views: grad_world = sum_views R^T J^T g (FP64).
+// One thread per vertex, looping over the views: grad_world = sum_views R^T J^T g (FP64).  STORE: overwrite grad_verts (and
+// the second copy) instead of adding to it.
+template <bool STORE>
 __global__ void k_project_backward(int V, const mer_camera* __restrict__ cams, int n,
                                    const mer_vertex* __restrict__ vpix, const double* __restrict__ grad_vpix,
-                                   float* __restrict__ grad_verts) {
+                                   float* __restrict__ grad_verts, float* __restrict__ copy) {
     const int v = blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= V) return;
     double a0 = 0.0, a1 = 0.0, a2 = 0.0;
@@ -174,9 +183,14 @@ __global__ void k_project_backward(int V, const mer_camera* __restrict__ cams, i
         a1 += w[1];
         a2 += w[2];
     }
-    grad_verts[3 * (size_t)v] += (float)a0;
-    grad_verts[3 * (size_t)v + 1] += (float)a1;
-    grad_verts[3 * (size_t)v + 2] += (float)a2;
+    float* o = grad_verts + 3 * (size_t)v;
+    const float g[3] = {(float)a0, (float)a1, (float)a2};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const float r = STORE ? g[c] : o[c] + g[c];
+        o[c] = r;
+        if (copy) copy[3 * (size_t)v + c] = r;
+    }
 }
 
 }  // namespace mer
@@ -184,10 +198,10 @@ __global__ void k_project_backward(int V, const mer_camera* __restrict__ cams, i
 using namespace mer;
 
 extern "C" int mer_launch_project(const float* verts, int V, const mer_camera* cams, int n, mer_vertex* vpix,
-                                  cudaStream_t s) {
+                                  mer_vertex* copy, int* clear, long long n_clear, cudaStream_t s) {
     const long long N = (long long)V * n;
     if (N == 0) return 0;
-    k_project<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(verts, V, cams, n, vpix);
+    k_project<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(verts, V, cams, n, vpix, copy, clear, n_clear);
     return cudaGetLastError() == cudaSuccess ? 0 : 2;
 }
 
@@ -199,9 +213,13 @@ extern "C" int mer_launch_project_screen(const double* scr, int V, int n, mer_ve
 }
 
 extern "C" int mer_launch_project_backward(int V, const mer_camera* cams, int n, const mer_vertex* vpix,
-                                           const double* grad_vpix, float* grad_verts, cudaStream_t s) {
+                                           const double* grad_vpix, float* grad_verts, float* copy, int store,
+                                           cudaStream_t s) {
     if (V == 0 || n == 0) return 0;
-    k_project_backward<<<(V + 255) / 256, 256, 0, s>>>(V, cams, n, vpix, grad_vpix, grad_verts);
+    if (store)
+        k_project_backward<true><<<(V + 255) / 256, 256, 0, s>>>(V, cams, n, vpix, grad_vpix, grad_verts, copy);
+    else
+        k_project_backward<false><<<(V + 255) / 256, 256, 0, s>>>(V, cams, n, vpix, grad_vpix, grad_verts, copy);
     return cudaGetLastError() == cudaSuccess ? 0 : 2;
 }
 
@@ -230,5 +248,20 @@ extern "C" int mer_launch_project_backward_batch(const mer_camera* cams, const m
     }
     k_project_backward_batch<<<(unsigned)((vrecs + 255) / 256), 256, 0, s>>>(cams, items, n_items, vrecs, vpix,
                                                                              grad_vpix, grad_verts);
+    return cudaGetLastError() == cudaSuccess ? 0 : 2;
+}
+
+namespace mer {
+__global__ void k_clear(double* __restrict__ a, long long na, float* __restrict__ b, long long nb) {
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < na) a[i] = 0.0;
+    if (i < nb) b[i] = 0.f;
+}
+}  // namespace mer
+
+// Zeroes two gradient arrays in one launch.
+extern "C" int mer_launch_clear(double* a, long long na, float* b, long long nb, cudaStream_t s) {
+    const long long m = na > nb ? na : nb;
+    if (m > 0) k_clear<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(a, na, b, nb);
     return cudaGetLastError() == cudaSuccess ? 0 : 2;
 }

@@ -37,6 +37,8 @@ struct ShadeOut {
     const float* attr;  // attribute rows of all meshes
     const float* tex;
     float* image;       // [pixels, C]
+    float* image2;      // second copies of the image and the index, or null
+    int* index2;
 };
 
 __device__ __forceinline__ int floordiv256(int a) { return a >> 8; }  // arithmetic shift = floor
@@ -239,6 +241,58 @@ __global__ void k_scan_add(int* __restrict__ out, long long N, const int* __rest
     }
 }
 
+// The whole scan in one CTA while every thread holds at most kScanEach counts (a launch of a few thousand tiles: 1.9 us
+// instead of three launches of 1.5 to 1.9 us with the gaps between them).  host (optional): the status word and the number
+// of bin entries, in memory that the host polls; a status of at least kHostReady marks them as written.
+constexpr int kScanEach = 16;
+constexpr long long kHostReady = 1LL << 32;
+
+__global__ void __launch_bounds__(kScanBlock) k_scan_all(const int* __restrict__ in, int N, int* __restrict__ out,
+                                                         int* __restrict__ cursor, void* ws, long long capacity,
+                                                         volatile long long* host) {
+    __shared__ int sh[32];
+    const int each = (N + kScanBlock - 1) / kScanBlock;
+    const int i0 = threadIdx.x * each;
+    int v[kScanEach], sum = 0;
+#pragma unroll
+    for (int k = 0; k < kScanEach; ++k) {
+        v[k] = k < each && i0 + k < N ? in[i0 + k] : 0;
+        sum += v[k];
+    }
+    int total;
+    int before = block_exclusive_scan(sum, sh, total);
+    if (threadIdx.x == 0) {
+        WsHeader* h = reinterpret_cast<WsHeader*>(ws);
+        h->total_bins = total;
+        h->capacity = capacity;
+        h->queue_raster = 0ull;
+        const int status = h->status | (total > capacity ? kStatusOverflow : 0);
+        h->status = status;
+        if (host) {
+            host[1] = total;
+            __threadfence_system();
+            host[0] = kHostReady + status;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < kScanEach; ++k) {
+        if (k < each && i0 + k < N) {
+            out[i0 + k] = before;
+            cursor[i0 + k] = 0;
+            cursor[N + i0 + k] = 0;
+        }
+        before += v[k];
+    }
+}
+
+// The same two words for the host after a scan in several launches.
+__global__ void k_host_status(const void* ws, volatile long long* host) {
+    const WsHeader* h = reinterpret_cast<const WsHeader*>(ws);
+    host[1] = h->total_bins;
+    __threadfence_system();
+    host[0] = kHostReady + h->status;
+}
+
 // --- raster ---
 // One CTA per tile.  The tile's triangle records are staged in shared memory and sorted by the pixel count of their
 // bounding box inside the tile: a group of 2, 8 or 32 lanes takes one triangle at a time and tests that box G pixels at
@@ -366,7 +420,8 @@ __device__ __forceinline__ void raster_class(RasterShared<TS>& S, int n, int ox,
 // The tile's list holds the camera-facing triangles first (nfront of them) and the others after; before
 // the second part the tile's smallest depth key is taken, and a triangle of that part whose largest vertex
 // zeta (with a margin above the FP32 rounding of the key) is below it cannot win any pixel: it is skipped.
-template <int TS, int FORM>
+// DUAL: the index image and the shaded image are also written to so.index2 and so.image2.
+template <int TS, int FORM, bool DUAL = false>
 __device__ __forceinline__ void raster_tile(const RItem& it, int local_tile, const int* __restrict__ offs,
                                             const int* __restrict__ cnts, const int* __restrict__ nfront,
                                             const int* __restrict__ list, bool overflow, RasterShared<TS>& S,
@@ -422,6 +477,7 @@ __device__ __forceinline__ void raster_tile(const RItem& it, int local_tile, con
         const int t = key ? (int)(0xFFFFFFFFu - (unsigned)(key & 0xFFFFFFFFull)) : -1;
         const size_t p = (size_t)it.pix0 + (size_t)py * it.W + px;
         index[p] = t;
+        if (DUAL) so.index2[p] = t;
         if (cover) {
             const int lx = i % TS, ly = i / TS;
             unsigned c = (lx == 0 ? MER_COVER_BORDER_L : 0u) | (lx == TS - 1 ? MER_COVER_BORDER_R : 0u) |
@@ -438,9 +494,9 @@ __device__ __forceinline__ void raster_tile(const RItem& it, int local_tile, con
             cover[p] = (unsigned char)c;
         }
         if (FORM != kShadeOff)
-            shade_fragment<FORM, false>(it.vpix, it.V, it.tris, it.T, t, px, py,
+            shade_fragment<FORM, false, DUAL>(it.vpix, it.V, it.tris, it.T, t, px, py,
                                         so.attr ? so.attr + (size_t)it.vert * so.a.sh.C_attr : nullptr, so.tex, so.a,
-                                        so.image + p * so.a.sh.C, ws);
+                                        so.image + p * so.a.sh.C, ws, DUAL ? so.image2 + p * so.a.sh.C : nullptr);
         if (!depth && !bary) continue;
         float Z = 0.f, b1 = 0.f, b2 = 0.f;
         if (t >= 0) {
@@ -501,24 +557,23 @@ __global__ void k_bin_fill(const mer_vertex* __restrict__ vpix, const int* __res
              cursor + (long long)g.n * g.tiles_per_view, list, capacity);
 }
 
-template <int TS>
+template <int TS, int FORM, bool DUAL>
 __global__ void __launch_bounds__(kRasterThreads, kRasterCtasPerSm) k_raster(TriRaster* __restrict__ recs, BinGeom g,
                                                            const int* __restrict__ offs, const int* __restrict__ cnts,
                                                            const int* __restrict__ nfront,
                                                            const int* __restrict__ list, const mer_vertex* __restrict__ vpix,
                                                            const int* __restrict__ tris, void* ws, long long capacity,
                                                            int* __restrict__ index, float* __restrict__ depth,
-                                                           float* __restrict__ bary, unsigned char* __restrict__ cover) {
+                                                           float* __restrict__ bary, unsigned char* __restrict__ cover,
+                                                           ShadeOut so) {
     __shared__ RasterShared<TS> S;
     const WsHeader* hdr = reinterpret_cast<const WsHeader*>(ws);
     const bool overflow = hdr->total_bins > capacity;
     const long long tile = blockIdx.x;
     const int view = (int)(tile / g.tiles_per_view);
     const int local = (int)(tile % g.tiles_per_view);
-    ShadeOut none;
-    none.attr = nullptr; none.tex = nullptr; none.image = nullptr;
-    raster_tile<TS, kShadeOff>(view_item(g, vpix, tris, recs, view), local, offs, cnts, nfront, list, overflow, S, index,
-                           depth, bary, cover, none, ws);
+    raster_tile<TS, FORM, DUAL>(view_item(g, vpix, tris, recs, view), local, offs, cnts, nfront, list, overflow, S, index,
+                                depth, bary, cover, so, ws);
 }
 
 // ---- batched entry: items from a table ----
@@ -637,15 +692,20 @@ RasterLayout raster_layout(int V, int T, int n, int H, int W, int tile, long lon
 }
 
 // Scan of the per-tile counts and the header totals.
-int launch_scan(const RasterLayout& L, char* base, long long capacity, cudaStream_t s) {
+int launch_scan(const RasterLayout& L, char* base, long long capacity, cudaStream_t s, long long* host = nullptr) {
     WsHeader* hdr = reinterpret_cast<WsHeader*>(base + L.hdr);
     int* counts = reinterpret_cast<int*>(base + L.counts);
     int* offs = reinterpret_cast<int*>(base + L.offs);
     int* cursor = reinterpret_cast<int*>(base + L.cursor);
     int* sums = reinterpret_cast<int*>(base + L.sums);
+    if (L.ntiles <= (long long)kScanBlock * kScanEach) {
+        k_scan_all<<<1, kScanBlock, 0, s>>>(counts, (int)L.ntiles, offs, cursor, hdr, capacity, host);
+        return 0;
+    }
     if (L.nblocks > 0) k_scan_blocks<<<(unsigned)L.nblocks, kScanBlock, 0, s>>>(counts, L.ntiles, offs, sums);
     k_scan_sums<<<1, kScanBlock, 0, s>>>(sums, (int)L.nblocks, hdr, capacity);
     if (L.nblocks > 0) k_scan_add<<<(unsigned)L.nblocks, kScanBlock, 0, s>>>(offs, L.ntiles, sums, cursor);
+    if (host) k_host_status<<<1, 1, 0, s>>>(hdr, host);
     return 0;
 }
 }  // namespace
@@ -654,9 +714,25 @@ extern "C" size_t mer_raster_workspace_size(int V, int T, int n, int H, int W, i
     return raster_layout(V, T, n, H, W, tile, capacity).total;
 }
 
-extern "C" int mer_launch_rasterize(const mer_vertex* vpix, int V, const int* tris, int T, int n, int H, int W,
-                                    int tile, void* ws, size_t ws_bytes, int* index, float* depth, float* bary,
-                                    unsigned char* cover, cudaStream_t s) {
+extern "C" int mer_launch_project(const float*, int, const mer_camera*, int, mer_vertex*, mer_vertex*, int*, long long,
+                                  cudaStream_t);
+extern "C" int mer_launch_shade(const mer_vertex*, int, const int*, int, int, int, int, const int*, const float*,
+                                const float*, const float*, const mer_shading*, float*, void*, cudaStream_t);
+
+template <int TS, int FORM, bool DUAL>
+static void launch_view_tile(unsigned grid, TriRaster* recs, const BinGeom& g, const int* offs, const int* counts,
+                             const int* cursor, const int* list, const mer_vertex* vpix, const int* tris, void* hdr,
+                             long long capacity, int* index, float* depth, float* bary, unsigned char* cover,
+                             const ShadeOut& so, cudaStream_t s) {
+    k_raster<TS, FORM, DUAL><<<grid, kRasterThreads, 0, s>>>(recs, g, offs, counts, cursor, list, vpix, tris, hdr, capacity,
+                                                             index, depth, bary, cover, so);
+}
+
+// Setup, binning and raster of n views; with `so`, each resolved tile is shaded in the same pass (so->image2 / index2: and
+// written twice).  cleared: the tile counts are zero already.  host: see k_scan_all.
+static int view_raster(const mer_vertex* vpix, int V, const int* tris, int T, int n, int H, int W, int tile, void* ws,
+                       size_t ws_bytes, int* index, float* depth, float* bary, unsigned char* cover, const ShadeOut* so,
+                       bool cleared, long long* host, cudaStream_t s) {
     // capacity: whatever the workspace holds beyond the fixed part
     RasterLayout L = raster_layout(V, T, n, H, W, tile, 1);
     if (ws_bytes < L.total) return 1;
@@ -674,22 +750,76 @@ extern "C" int mer_launch_rasterize(const mer_vertex* vpix, int V, const int* tr
     g.ntx = (W + tile - 1) / tile;
     g.nty = (H + tile - 1) / tile;
     g.tiles_per_view = (long long)g.ntx * g.nty;
-    // header: the status word is sticky until mer_sync_status; k_scan_sums writes the totals
-    if (cudaMemsetAsync(counts, 0, (size_t)L.ntiles * 4, s) != cudaSuccess) return 2;
+    // header: the status word is sticky until mer_sync_status; the scan writes the totals
+    if (!cleared && cudaMemsetAsync(counts, 0, (size_t)L.ntiles * 4, s) != cudaSuccess) return 2;
     const long long NT = (long long)T * n;
     if (NT > 0) k_setup_count<<<(unsigned)((NT + 255) / 256), 256, 0, s>>>(vpix, tris, g, recs, counts, hdr);
-    launch_scan(L, base, capacity, s);
+    launch_scan(L, base, capacity, s, host);
     if (NT > 0)
         k_bin_fill<<<(unsigned)((NT + 255) / 256), 256, 0, s>>>(vpix, tris, g, recs, offs, counts, cursor, list,
                                                                 capacity);
     const unsigned grid = (unsigned)L.ntiles;
+    ShadeOut none;
+    none.attr = nullptr; none.tex = nullptr; none.image = nullptr; none.image2 = nullptr; none.index2 = nullptr;
+    const ShadeOut& o = so ? *so : none;
+    const int form = so ? shade_form(so->attr, so->tex, &so->a.sh) : kShadeOff;
+    const bool dual = o.image2 != nullptr;
+#define MER_TILE(TS, F, D)                                                                                               \
+    launch_view_tile<TS, F, D>(grid, recs, g, offs, counts, cursor, list, vpix, tris, hdr, capacity, index, depth, bary, \
+                               cover, o, s)
+#define MER_FORM(TS)                                                                       \
+    switch (form) {                                                                        \
+        case kShadeOff: MER_TILE(TS, kShadeOff, false); break;                             \
+        case kTex3: if (dual) MER_TILE(TS, kTex3, true); else MER_TILE(TS, kTex3, false); break;    \
+        case kAttr3: if (dual) MER_TILE(TS, kAttr3, true); else MER_TILE(TS, kAttr3, false); break; \
+        default: if (dual) MER_TILE(TS, kGeneric, true); else MER_TILE(TS, kGeneric, false); break; \
+    }
     switch (tile) {
-        case 8: k_raster<8><<<grid, kRasterThreads, 0, s>>>(recs, g, offs, counts, cursor, list, vpix, tris, hdr, capacity, index, depth, bary, cover); break;
-        case 16: k_raster<16><<<grid, kRasterThreads, 0, s>>>(recs, g, offs, counts, cursor, list, vpix, tris, hdr, capacity, index, depth, bary, cover); break;
-        case 32: k_raster<32><<<grid, kRasterThreads, 0, s>>>(recs, g, offs, counts, cursor, list, vpix, tris, hdr, capacity, index, depth, bary, cover); break;
+        case 8: MER_FORM(8) break;
+        case 16: MER_FORM(16) break;
+        case 32: MER_FORM(32) break;
         default: return 1;
     }
+#undef MER_FORM
+#undef MER_TILE
     return cudaGetLastError() == cudaSuccess ? 0 : 2;
+}
+
+extern "C" int mer_launch_rasterize(const mer_vertex* vpix, int V, const int* tris, int T, int n, int H, int W,
+                                    int tile, void* ws, size_t ws_bytes, int* index, float* depth, float* bary,
+                                    unsigned char* cover, cudaStream_t s) {
+    return view_raster(vpix, V, tris, T, n, H, W, tile, ws, ws_bytes, index, depth, bary, cover, nullptr, false, nullptr, s);
+}
+
+// Projection, binning, raster and shading of n views (V, T, n, H, W > 0).
+extern "C" int mer_launch_view_render(const mer_view* v, const float* verts, const mer_camera* cams, const float* attr,
+                                      const float* tex, float* depth, float* bary, mer_vertex* vpix2, int* index2,
+                                      float* image2, long long* host, cudaStream_t s) {
+    const RasterLayout L = raster_layout(v->V, v->T, v->n, v->H, v->W, v->tile, 1);
+    int* counts = reinterpret_cast<int*>(static_cast<char*>(v->workspace) + L.counts);
+    // the projection's threads clear the tile counts on the way unless there are many more of those
+    const bool cleared = L.ntiles <= 4LL * v->V * v->n;
+    int rc = mer_launch_project(verts, v->V, cams, v->n, v->vpix, vpix2, counts, cleared ? L.ntiles : 0, s);
+    if (rc) return rc;
+    ShadeOut so;
+    so.a = make_shade_args(tex, v->bg_host, v->sh);
+    so.attr = attr;
+    so.tex = tex;
+    so.image = v->image;
+    so.image2 = image2;
+    so.index2 = index2;
+    const bool precise = v->sh->precise != 0;  // FP64 shading is a pass of its own, over the index image
+    rc = view_raster(v->vpix, v->V, v->tris, v->T, v->n, v->H, v->W, v->tile, v->workspace, v->workspace_bytes, v->index,
+                     depth, bary, v->cover, precise ? nullptr : &so, cleared, host, s);
+    if (rc || !precise) return rc;
+    rc = mer_launch_shade(v->vpix, v->V, v->tris, v->T, v->n, v->H, v->W, v->index, attr, tex, v->bg_host, v->sh, v->image,
+                          v->workspace, s);
+    if (rc || !image2) return rc;
+    const size_t px = (size_t)v->n * v->H * v->W;
+    if (cudaMemcpyAsync(image2, v->image, px * v->sh->C * sizeof(float), cudaMemcpyDeviceToDevice, s) != cudaSuccess ||
+        cudaMemcpyAsync(index2, v->index, px * sizeof(int), cudaMemcpyDeviceToDevice, s) != cudaSuccess)
+        return 2;
+    return 0;
 }
 
 extern "C" size_t mer_batch_raster_workspace_size(long long tiles, long long trecs, long long capacity) {
@@ -754,7 +884,7 @@ static int batch_raster(const mer_vertex* vpix, const int* tris, const mer_item*
     if (tiles > 0) {
         const unsigned grid = persistent_ctas > 0 ? (unsigned)persistent_ctas : 0u;
         ShadeOut none;
-        none.attr = nullptr; none.tex = nullptr; none.image = nullptr;
+        none.attr = nullptr; none.tex = nullptr; none.image = nullptr; none.image2 = nullptr; none.index2 = nullptr;
         const ShadeOut& o = so ? *so : none;
         int rc = 0;
 #define MER_RASTER(F) \
@@ -802,6 +932,8 @@ extern "C" int mer_launch_batch_render(const mer_vertex* vpix, const int* tris, 
     so.attr = attr;
     so.tex = tex;
     so.image = image;
+    so.image2 = nullptr;
+    so.index2 = nullptr;
     return batch_raster(vpix, tris, items, n_items, trecs, tiles, tile, ws, ws_bytes, index, depth, bary, cover, &so,
                         persistent_ctas, s);
 }

@@ -63,13 +63,17 @@ __device__ __forceinline__ void load_uv(const float* __restrict__ attr, int Ca, 
 
 // The C channels of pixel (x, y) covered by triangle t (t < 0: background), written to o[0..C).  vb / tris /
 // attr are the item's bases.  CHECK: t and the vertex ids may be out of range (the fused raster's are not: its setup
-// drops such triangles).
-template <int FORM, bool CHECK>
+// drops such triangles).  DUAL: also to o2.
+template <int FORM, bool CHECK, bool DUAL = false>
 __device__ __forceinline__ void shade_fragment(const mer_vertex* __restrict__ vb, int V, const int* __restrict__ tris,
                                                int T, int t, int x, int y, const float* __restrict__ attr,
                                                const float* __restrict__ tex, const ShadeArgs& a,
-                                               float* __restrict__ o, void* ws) {
+                                               float* __restrict__ o, void* ws, float* __restrict__ o2 = nullptr) {
     const int C = a.sh.C;
+    auto put = [&](int c, float value) {
+        o[c] = value;
+        if (DUAL) o2[c] = value;
+    };
     int vid[3] = {0, 0, 0};
     bool ok = t >= 0;
     if (CHECK && t >= T) {
@@ -87,7 +91,7 @@ __device__ __forceinline__ void shade_fragment(const mer_vertex* __restrict__ vb
     if (!ok) {
 #pragma unroll
         for (int c = 0; c < kMaxC; ++c)  // static indices keep the arguments out of local memory
-            if (c < C) o[c] = a.bg[c];
+            if (c < C) put(c, a.bg[c]);
         return;
     }
     const VRec v[3] = {load_vrec(vb + vid[0]), load_vrec(vb + vid[1]), load_vrec(vb + vid[2])};
@@ -108,13 +112,13 @@ __device__ __forceinline__ void shade_fragment(const mer_vertex* __restrict__ vb
             for (int c = 0; c < 3; ++c) acc[c] += b[k] * __ldg(q + c);
         }
 #pragma unroll
-        for (int c = 0; c < 3; ++c) o[c] = acc[c];
+        for (int c = 0; c < 3; ++c) put(c, acc[c]);
     } else if (FORM != kTex3 && a.sh.uv_offset < 0) {
         for (int c = 0; c < a.sh.n_main; ++c) {
             float acc = 0.f;
 #pragma unroll
             for (int k = 0; k < 3; ++k) acc += b[k] * __ldg(attr + (size_t)vid[k] * Ca + c);
-            o[c] = acc;
+            put(c, acc);
         }
     } else {
         float uk[3], vk[3];
@@ -124,27 +128,27 @@ __device__ __forceinline__ void shade_fragment(const mer_vertex* __restrict__ vb
         const TexTaps taps = tex_taps(a.sh.tex_h, a.sh.tex_w, cx, cy);
         if (FORM == kTex3) {
             const TexQuad x = tex_quad(tex, a.sh.tex_w, taps);
-            o[0] = tex_lerp(x.a00.x, x.a10.x, x.a01.x, x.a11.x, taps);
-            o[1] = tex_lerp(x.a00.y, x.a10.y, x.a01.y, x.a11.y, taps);
-            o[2] = tex_lerp(x.a00.z, x.a10.z, x.a01.z, x.a11.z, taps);
+            put(0, tex_lerp(x.a00.x, x.a10.x, x.a01.x, x.a11.x, taps));
+            put(1, tex_lerp(x.a00.y, x.a10.y, x.a01.y, x.a11.y, taps));
+            put(2, tex_lerp(x.a00.z, x.a10.z, x.a01.z, x.a11.z, taps));
         } else if (a.sh.n_main <= 4) {
             float v4[4];
             tex_values(tex, a.sh.tex_w, a.tex_stride, a.tex_vec4, a.sh.n_main, taps, v4);
 #pragma unroll
             for (int c = 0; c < 4; ++c)
-                if (c < a.sh.n_main) o[c] = v4[c];
+                if (c < a.sh.n_main) put(c, v4[c]);
         } else {
             float vk_[kMaxC];
             tex_values(tex, a.sh.tex_w, a.tex_stride, false, a.sh.n_main, taps, vk_);
-            for (int c = 0; c < a.sh.n_main && c < kMaxC; ++c) o[c] = vk_[c];
+            for (int c = 0; c < a.sh.n_main && c < kMaxC; ++c) put(c, vk_[c]);
         }
     }
-    if (a.sh.mask_ch >= 0) o[a.sh.mask_ch] = 1.0f;
-    if (a.sh.depth_ch >= 0) o[a.sh.depth_ch] = is;
+    if (a.sh.mask_ch >= 0) put(a.sh.mask_ch, 1.0f);
+    if (a.sh.depth_ch >= 0) put(a.sh.depth_ch, is);
     if (a.sh.backface_ch >= 0) {
         // back-face image: the exact sign of the snapped screen area (positive = facing away, y down)
         const int64_t area = (int64_t)(v[1].X - v[0].X) * (v[2].Y - v[0].Y) - (int64_t)(v[1].Y - v[0].Y) * (v[2].X - v[0].X);
-        o[a.sh.backface_ch] = area > 0 ? 1.0f : 0.0f;
+        put(a.sh.backface_ch, area > 0 ? 1.0f : 0.0f);
     }
 }
 

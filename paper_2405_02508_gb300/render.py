@@ -1,10 +1,13 @@
 """Forward/backward calls over the C-ABI, and the ``torch.autograd.Function``.
 
 ``Renderer`` owns the caller-side buffers (workspace, vertex records, images)
-for one mesh and a batch of views and chains the library calls:
+for one mesh and a batch of views and makes the library calls, one per pass:
 
-    forward : mer_project -> mer_rasterize -> mer_shade
-    backward: mer_backward (edge + interior) -> mer_project_backward
+    forward : mer_view_render (mer_project -> mer_rasterize -> mer_shade)
+    backward: mer_view_backward (mer_backward (edge + interior) -> mer_project_backward)
+
+A small render is a few dozen microseconds on the device, less than the host took for a dozen calls
+with their arguments; the stages stay available one by one (``project``, ``rasterize``, ``shade``).
 
 With ``cover_hint`` (default) the rasterizer also writes the cover image (which facings cover each pixel
 centre, one byte a pixel) and the backward uses it to skip pixel pairs that cannot scatter; the results are
@@ -52,6 +55,8 @@ class Renderer:
         self.grad_vpix = torch.zeros((n, self.V, 3), dtype=torch.float64, device=device)
         self.grad_verts = torch.zeros((self.V, 3), dtype=torch.float32, device=device)
         self.terms = B.MER_EDGE | B.MER_INTERIOR | B.MER_INTERSECT
+        self.renders = 0      # times the buffers were drawn to
+        self._status = None   # pinned words the device reports the binning's status in (made by the first checked pass)
         self._alloc_workspace(0)
 
     def _alloc_workspace(self, capacity: int, at_least: int = 0):
@@ -65,12 +70,15 @@ class Renderer:
 
     # -- forward -----------------------------------------------------------------------------------
     def project(self, verts: torch.Tensor, cams: torch.Tensor):
+        self.renders += 1
         B.mer_project(verts.contiguous(), cams, self.vpix)
 
     def project_screen(self, scr: torch.Tensor):
+        self.renders += 1
         B.mer_project_screen(scr.contiguous(), self.vpix)
 
     def rasterize(self, depth: torch.Tensor | None = None, bary: torch.Tensor | None = None, checked: bool = True):
+        self.renders += 1
         B.mer_rasterize(self.vpix, self.tris, self.H, self.W, self.tile, self.workspace, self.index, depth, bary,
                         self.cover)
         if checked:
@@ -84,18 +92,59 @@ class Renderer:
                 raise B.MerError(code, "mer_rasterize")
 
     def shade(self, attr: torch.Tensor, tex: torch.Tensor | None):
+        self.renders += 1
         B.mer_shade(self.vpix, self.tris, self.index, attr.contiguous(), tex, self.bg, self.sh, self.image,
                     self.workspace)
 
-    def forward(self, verts, cams, attr, tex=None, depth=None, bary=None, checked=True):
-        self.project(verts, cams)
-        self.rasterize(depth, bary, checked)
-        self.shade(attr, tex)
+    def _view(self, bg=None) -> B.MerView:
+        """The renderer's buffers for one call."""
+        return B.view_struct(self.tris, self.V, self.n, self.H, self.W, self.tile, self.workspace, self.vpix, self.index,
+                             self.cover, self.image, self.sh, bg)
+
+    def forward(self, verts, cams, attr, tex=None, depth=None, bary=None, checked=True, copies=None):
+        """copies (optional): (vpix, index, image) tensors that receive second copies of those buffers."""
+        if verts.shape[0] != self.V or cams.shape[0] != self.n:  # fewer vertices or cameras than the buffers hold
+            self.project(verts, cams)
+            self.rasterize(depth, bary, checked)
+            self.shade(attr, tex)
+            if copies is not None:
+                for dst, src in zip(copies, (self.vpix, self.index, self.image)):
+                    dst.copy_(src)
+            return self.image
+        status = None
+        if checked:
+            if self._status is None:
+                self._status = torch.zeros(2, dtype=torch.int64, pin_memory=True)
+            status = self._status
+        self.renders += 1
+        verts, attr = verts.contiguous(), attr.contiguous()
+        args = (verts, cams, attr, tex, depth, bary, copies or (None, None, None), status)
+        code, total = B.mer_view_render(self._view(self.bg), *args)
+        if code == B.MER_EOVERFLOW:  # size the bin list exactly and redo
+            self._alloc_workspace(int(total * 1.25) + 1024)
+            code, total = B.mer_view_render(self._view(self.bg), *args)
+        if code != B.MER_OK:
+            raise B.MerError(code, "mer_rasterize")
         return self.image
 
     # -- backward ----------------------------------------------------------------------------------
     def backward(self, grad_image: torch.Tensor, cams: torch.Tensor, attr: torch.Tensor, tex=None,
                  terms: int = B.MER_EDGE | B.MER_INTERIOR | B.MER_INTERSECT, grad_attr=None, zero: bool = True):
+        if cams.shape[0] != self.n:
+            return self._backward_stages(grad_image, cams, attr, tex, terms, grad_attr, zero)
+        return self._backward((self.vpix, self.index, self.cover, self.image), grad_image, cams, attr, tex, terms, grad_attr,
+                              None, int(bool(zero)))
+
+    def _backward(self, drawn, grad_image, cams, attr, tex, terms, grad_attr, grad_verts_copy, zero):
+        """drawn: the vpix, index, cover and image that the gradient is of; zero: 0, 1 or 2 as in mer_view_backward."""
+        if terms & B.MER_DETERMINISTIC:
+            self._ensure_backward_workspace(terms, grad_attr)
+        view = B.view_struct(self.tris, self.V, self.n, self.H, self.W, self.tile, self.workspace, *drawn, self.sh)
+        B.mer_view_backward(view, cams, grad_image.contiguous(), attr.contiguous(), tex, terms, self.grad_vpix,
+                            grad_attr, self.grad_verts, grad_verts_copy, zero)
+        return self.grad_verts
+
+    def _backward_stages(self, grad_image, cams, attr, tex, terms, grad_attr, zero):
         if zero:
             self.grad_vpix.zero_()
             self.grad_verts.zero_()
@@ -110,10 +159,13 @@ class Renderer:
                      terms: int = B.MER_EDGE | B.MER_INTERIOR | B.MER_INTERSECT) -> torch.Tensor:
         """d(image)/d(theta) [n,H,W,C] for a world-space vertex tangent [V,3] (after ``forward``)."""
         tv = torch.empty((self.n, self.V, 3), dtype=torch.float32, device=self.device)
-        B.mer_project_jvp(tangent_world.contiguous(), cams, self.vpix, tv)
         out = torch.empty_like(self.image)
-        B.mer_forward_grad(self.vpix, self.tris, self.index, self.image, tv, attr.contiguous(), tex, self.sh, terms,
-                           out, self.workspace)
+        if tangent_world.shape[0] != self.V or cams.shape[0] != self.n:
+            B.mer_project_jvp(tangent_world.contiguous(), cams, self.vpix, tv)
+            B.mer_forward_grad(self.vpix, self.tris, self.index, self.image, tv, attr.contiguous(), tex, self.sh, terms,
+                               out, self.workspace)
+            return out
+        B.mer_view_forward_grad(self._view(), cams, tangent_world.contiguous(), attr.contiguous(), tex, terms, tv, out)
         return out
 
     def check_status(self):
@@ -135,13 +187,14 @@ class MerRender(torch.autograd.Function):
         bary = None
         if not recompute_bary:
             bary = torch.empty((r.n, r.H, r.W, 2), dtype=torch.float32, device=r.device)
-        r.forward(verts, cams, attr, tex, bary=bary)
-        image = r.image.clone()
+        saved = torch.empty_like(r.vpix), torch.empty_like(r.index), torch.empty_like(r.image)
+        r.forward(verts, cams, attr, tex, bary=bary, copies=saved)
         ctx.renderer = r
-        ctx.save_for_backward(verts, attr, cams, r.vpix.clone(), r.index.clone(), image,
-                              *(() if tex is None else (tex,)), *(() if bary is None else (bary,)))
+        ctx.renders = r.renders
+        ctx.save_for_backward(verts, attr, cams, *saved, *(() if tex is None else (tex,)),
+                              *(() if bary is None else (bary,)))
         ctx.has_tex = tex is not None
-        return image
+        return saved[2]
 
     @staticmethod
     def backward(ctx, grad_image):
@@ -149,9 +202,19 @@ class MerRender(torch.autograd.Function):
         saved = ctx.saved_tensors
         verts, attr, cams, vpix, index, image = saved[:6]
         tex = saved[6] if ctx.has_tex else None
-        r.vpix.copy_(vpix)
-        r.index.copy_(index)
-        r.image.copy_(image)
-        grad_attr = torch.zeros_like(attr) if ctx.needs_input_grad[1] else None
-        gv = r.backward(grad_image, cams, attr, tex, terms=r.terms, grad_attr=grad_attr)
-        return gv.clone(), grad_attr, None, None, None, None
+        cover = r.cover
+        if r.renders != ctx.renders:  # the renderer has drawn something else since: its cover image is of that
+            r.vpix.copy_(vpix)
+            r.index.copy_(index)
+            r.image.copy_(image)
+            r.renders += 1
+            cover = None
+        grad_attr, zero = None, 1
+        if ctx.needs_input_grad[1]:
+            if attr.shape == (r.V, r.sh.C_attr):
+                grad_attr, zero = torch.empty_like(attr), 2
+            else:
+                grad_attr = torch.zeros_like(attr)
+        gv = torch.empty_like(r.grad_verts)
+        r._backward((vpix, index, cover, image), grad_image, cams, attr, tex, r.terms, grad_attr, gv, zero)
+        return gv, grad_attr, None, None, None, None
