@@ -257,6 +257,29 @@ __device__ __forceinline__ float diff_of_products(float a, float d, float b, flo
     return f + e;
 }
 
+// ---- FP64 without the conversions ----
+// GB300 issues one FP64 warp instruction in 16 cycles on an SM, and a conversion to or from a 64-bit type is one of them.
+// The exact ones are done here with integer instructions instead, on pipes that the FP64 kernels leave idle.
+
+// (No branches: they would end the compiler's blocks between the operations around them, and with them what it contracts.)
+
+// (double)x.  A denormal is scaled up first; the exponents of infinities and NaN are not rebased but filled.
+__device__ __forceinline__ double f2d(float x) {
+    const bool tiny = (__float_as_uint(x) & 0x7f800000u) == 0u;
+    const unsigned u = __float_as_uint(tiny ? x * 4294967296.0f : x), m = u & 0x7fffffffu;
+    const unsigned base = tiny ? 0x38000000u - (32u << 20) : (m >= 0x7f800000u ? 0x70000000u : 0x38000000u);
+    return __hiloint2double((int)((u & 0x80000000u) | (m == 0u ? 0u : (m >> 3) + base)), (int)(m << 29));
+}
+
+// (double)v.
+__device__ __forceinline__ double i2d(int v) {
+    const unsigned a = v < 0 ? 0u - (unsigned)v : (unsigned)v;
+    const int lz = __clz((int)a);
+    const unsigned n = a << (lz & 31);  // leading one at bit 31
+    const unsigned hi = ((unsigned)v & 0x80000000u) | (((unsigned)(1023 + 31 - lz) << 20) + ((n >> 11) & 0xfffffu));
+    return __hiloint2double(a == 0u ? 0 : (int)hi, (int)(n << 21));
+}
+
 // a*b - c*d, the second product rounded.  The values that decide which texel cell a pixel reads (barycentrics, perspective
 // weights, texel coordinates) are written with their roundings fixed: left to the compiler, the contraction into FMAs
 // depends on the code around them, and a kernel's variants then disagree at cell borders, where the derivative jumps.
