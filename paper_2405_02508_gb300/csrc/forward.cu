@@ -13,12 +13,16 @@
 //    (intersection); Eq. 11 then changes both pixels by 1/2 (I_A - I_B) dp/dtheta.
 //
 // One thread per pixel (32 x 8 tiles, index tile with a one-pixel halo in shared memory), no atomics: each
-// pixel evaluates its own four pairs.
+// pixel evaluates its own four pairs.  Classifying a pair is the long part, and most end there (the two triangles are
+// neighbours on a surface), so a warp compacts its row's pairs of all four directions into one list, classifies them with
+// full lanes, compacts the ones that move an edge again and takes their rates; the pixels then add their pairs in the
+// order of the directions.  512 x 512, 32,768 triangles: 27.0 us with every lane going through its own four pairs, 19.5 now
+// (with the layout's form, see ShadeForm).
 #include <cuda_runtime.h>
 
 #include <cstdint>
 
-#include "mer_device.cuh"
+#include "shade_device.cuh"
 
 namespace mer {
 
@@ -68,18 +72,18 @@ __device__ __forceinline__ float overhang_rate(const VRec rv[3], const int vid[3
         const int X[3] = {rv[0].X, rv[1].X, rv[2].X}, Y[3] = {rv[0].Y, rv[1].Y, rv[2].Y};
         const int k = exit_edge(X, Y, 256 * fx + 128, 256 * fy + 128, 256 * ox + 128, 256 * oy + 128);
         if (k >= 0) {
-            const int j = (k + 1) % 3, l = (k + 2) % 3;
-            const float u = axis == 0 ? crossing_u(rv[j].Y, rv[j].ry, rv[l].Y, rv[l].ry, 256 * fy + 128)
-                                      : crossing_u(rv[j].X, rv[j].rx, rv[l].X, rv[l].rx, 256 * fx + 128);
-            float tj[3], tl[3];
-            load_tangent(tb, vid[j], tj);
-            load_tangent(tb, vid[l], tl);
-            return (1.0f - u) * tj[axis] + u * tl[axis];
+            // j = k + 1, l = k + 2 (mod 3), picked without indexing (that would put the records into local memory)
+            const VRec &vj = k == 0 ? rv[1] : (k == 1 ? rv[2] : rv[0]), &vl = k == 0 ? rv[2] : (k == 1 ? rv[0] : rv[1]);
+            const int ij = k == 0 ? vid[1] : (k == 1 ? vid[2] : vid[0]), il = k == 0 ? vid[2] : (k == 1 ? vid[0] : vid[1]);
+            const float u = axis == 0 ? crossing_u(vj.Y, vj.ry, vl.Y, vl.ry, 256 * fy + 128)
+                                      : crossing_u(vj.X, vj.rx, vl.X, vl.rx, 256 * fx + 128);
+            const float tj = __ldg(tb + 3 * (size_t)ij + axis), tl = __ldg(tb + 3 * (size_t)il + axis);
+            return (1.0f - u) * tj + u * tl;
         }
     }
     float dr[3];
     frag_motion(rv, vid, tb, fx, fy, dr);
-    return dr[axis];
+    return axis == 0 ? dr[0] : dr[1];
 }
 
 __device__ __forceinline__ void plane_normal(const VRec r[3], float N[3]) {
@@ -97,6 +101,24 @@ __device__ __forceinline__ void plane_normal(const VRec r[3], float N[3]) {
     N[2] = diff_of_products(u[0], w[1], u[1], w[0]);
 }
 
+// Whether the centre of pixel (x, y) lies in the triangle of vertices v.
+__device__ __forceinline__ bool covers_centre(const mer_vertex* __restrict__ vb, const int v[3], int x, int y) {
+    int X[3], Y[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {  // snapped position only: one 64-bit load per vertex
+        const int2 xy = __ldg(reinterpret_cast<const int2*>(vb + v[k]));
+        X[k] = xy.x;
+        Y[k] = xy.y;
+    }
+    return covers_xy(X, Y, 256 * x + 128, 256 * y + 128);
+}
+
+constexpr int kNoRate = 0x7fffffff;  // bits of a NaN that no rate has (arithmetic gives 0x7fffffff only as itself negated)
+
+// FORM: the layout of the main channels (ShadeForm); the fixed ones hold at most kFastC channels.
+constexpr int kFastC = 8;
+
+template <int FORM>
 __global__ void __launch_bounds__(kFTW * kFTH) k_forward_grad(const mer_vertex* __restrict__ vpix,
                                                             const int* __restrict__ tris,
                                                             const int* __restrict__ index,
@@ -105,7 +127,11 @@ __global__ void __launch_bounds__(kFTW * kFTH) k_forward_grad(const mer_vertex* 
                                                             const float* __restrict__ attr,
                                                             const float* __restrict__ tex, FwdArgs a,
                                                             float* __restrict__ out, void* ws) {
+    constexpr int kC = FORM == kGeneric ? kMaxC : kFastC;
     __shared__ int sidx[kFTH + 2][kFTW + 2];
+    __shared__ int sown[kFTH][kFTW];            // the pixels' triangles, -1 if none or out of range
+    __shared__ float srate[kFTH][kFTW][4];      // dp/dtheta of the pixel's pair in each direction, or kNoRate
+    __shared__ unsigned short slist[kFTH][4 * kFTW];
     const int view = blockIdx.z;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int x = blockIdx.x * kFTW + tx, y = blockIdx.y * kFTH + ty;
@@ -117,17 +143,17 @@ __global__ void __launch_bounds__(kFTW * kFTH) k_forward_grad(const mer_vertex* 
         sidx[hy][hx] = (gx >= 0 && gx < a.W && gy >= 0 && gy < a.H) ? __ldg(idx + (size_t)gy * a.W + gx) : -2;
     }
     __syncthreads();
-    if (x >= a.W || y >= a.H) return;
+    const bool live = x < a.W && y < a.H;  // a row's lanes stay together for its list of pairs
     const int C = a.sh.C;
     const mer_vertex* vb = vpix + (size_t)view * a.V;
     const float* tb = tangent + (size_t)view * a.V * 3;
     const float* img = image + (size_t)view * plane * C;
     const size_t p = (size_t)y * a.W + x;
-    float acc[kMaxC];
+    float acc[kC];
 #pragma unroll
-    for (int c = 0; c < kMaxC; ++c) acc[c] = 0.f;
+    for (int c = 0; c < kC; ++c) acc[c] = 0.f;
 
-    int t = sidx[ty + 1][tx + 1];
+    int t = live ? sidx[ty + 1][tx + 1] : -1;
     int vid[3] = {0, 0, 0};
     if (t >= a.T || (t >= 0 && !fwd_tri_ids(tris, t, a.V, vid))) {
         set_status(ws, kStatusRange);
@@ -164,116 +190,166 @@ __global__ void __launch_bounds__(kFTW * kFTH) k_forward_grad(const mer_vertex* 
             db[k] = (dl[k] * z[k] + B.lam[k] * tv[k][2]) * is - b[k] * ds * is;
         }
         const int Ca = a.sh.C_attr;
-        if (a.sh.uv_offset < 0) {
+        if (FORM == kAttr3 || (FORM == kGeneric && a.sh.uv_offset < 0)) {
+            const float *q0 = attr + (long long)vid[0] * Ca, *q1 = attr + (long long)vid[1] * Ca,
+                        *q2 = attr + (long long)vid[2] * Ca;
 #pragma unroll
-            for (int c = 0; c < kMaxC; ++c) {
-                if (c >= a.sh.n_main) break;
-                const float a0 = __ldg(attr + (size_t)vid[0] * Ca + c);
-                const float a1 = __ldg(attr + (size_t)vid[1] * Ca + c);
-                const float a2 = __ldg(attr + (size_t)vid[2] * Ca + c);
+            for (int c = 0; c < (FORM == kAttr3 ? 3 : kC); ++c) {
+                if (FORM == kGeneric && c >= a.sh.n_main) break;
+                const float a0 = __ldg(q0 + c), a1 = __ldg(q1 + c), a2 = __ldg(q2 + c);
                 acc[c] += db[1] * (a1 - a0) + db[2] * (a2 - a0);  // sum_k db_k = 0
             }
         } else {
             float uk[3], vk[3];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                uk[k] = __ldg(attr + (size_t)vid[k] * Ca + a.sh.uv_offset);
-                vk[k] = __ldg(attr + (size_t)vid[k] * Ca + a.sh.uv_offset + 1);
-            }
+            load_uv<FORM>(attr, Ca, a.sh.uv_offset, vid, uk, vk);
             const float du = db[1] * (uk[1] - uk[0]) + db[2] * (uk[2] - uk[0]);
             const float dv = db[1] * (vk[1] - vk[0]) + db[2] * (vk[2] - vk[0]);
             const TexCoord cx = tex_coord(uk[0], uk[1], uk[2], b[1], b[2], a.sh.tex_w);
             const TexCoord cy = tex_coord(vk[0], vk[1], vk[2], b[1], b[2], a.sh.tex_h);
             const TexTaps taps = tex_taps(a.sh.tex_h, a.sh.tex_w, cx, cy);
             const float dfx = (float)a.sh.tex_w * du, dfy = taps.clamped ? 0.f : (float)a.sh.tex_h * dv;
-#pragma unroll
-            for (int c = 0; c < kMaxC; ++c) {
-                if (c >= a.sh.n_main) break;
-                const float* r0 = tex + (size_t)taps.j0 * a.sh.tex_w * a.tex_stride;
-                const float* r1 = tex + (size_t)taps.j1 * a.sh.tex_w * a.tex_stride;
-                const float t00 = __ldg(r0 + (size_t)taps.i0 * a.tex_stride + c);
-                const float t10 = __ldg(r0 + (size_t)taps.i1 * a.tex_stride + c);
-                const float t01 = __ldg(r1 + (size_t)taps.i0 * a.tex_stride + c);
-                const float t11 = __ldg(r1 + (size_t)taps.i1 * a.tex_stride + c);
+            auto tap = [&](float t00, float t10, float t01, float t11) {
                 const float dTx = (1.0f - taps.fy) * (t10 - t00) + taps.fy * (t11 - t01);
                 const float lo = t00 + taps.fx * (t10 - t00), hi = t01 + taps.fx * (t11 - t01);
-                acc[c] += dTx * dfx + (hi - lo) * dfy;
+                return dTx * dfx + (hi - lo) * dfy;
+            };
+            if (FORM == kTex3) {
+                const TexQuad q = tex_quad(tex, a.sh.tex_w, taps);
+                acc[0] += tap(q.a00.x, q.a10.x, q.a01.x, q.a11.x);
+                acc[1] += tap(q.a00.y, q.a10.y, q.a01.y, q.a11.y);
+                acc[2] += tap(q.a00.z, q.a10.z, q.a01.z, q.a11.z);
+            } else {
+#pragma unroll
+                for (int c = 0; c < kC; ++c) {
+                    if (c >= a.sh.n_main) break;
+                    const float* r0 = tex + (size_t)taps.j0 * a.sh.tex_w * a.tex_stride;
+                    const float* r1 = tex + (size_t)taps.j1 * a.sh.tex_w * a.tex_stride;
+                    acc[c] += tap(__ldg(r0 + (size_t)taps.i0 * a.tex_stride + c), __ldg(r0 + (size_t)taps.i1 * a.tex_stride + c),
+                                  __ldg(r1 + (size_t)taps.i0 * a.tex_stride + c), __ldg(r1 + (size_t)taps.i1 * a.tex_stride + c));
+                }
             }
         }
         if (a.sh.depth_ch >= 0) {
 #pragma unroll
-            for (int c = 0; c < kMaxC; ++c)
+            for (int c = 0; c < kC; ++c)
                 if (c == a.sh.depth_ch) acc[c] += -ds * is * is;
         }
     }
 
     if (a.terms & MER_EDGE) {
+        const unsigned full = 0xffffffffu;
         const bool exact = (a.terms & MER_EXACT_CROSSING) != 0;
-#pragma unroll 1
+        unsigned m[4];  // per direction: the lanes with a pair
+        int np[5];      // and how many before it
+        np[0] = 0;
+#pragma unroll
         for (int d = 0; d < 4; ++d) {
-            const int ddx = d == 0 ? -1 : (d == 1 ? 1 : 0);
-            const int ddy = d == 2 ? -1 : (d == 3 ? 1 : 0);
-            int tq = sidx[ty + 1 + ddy][tx + 1 + ddx];
-            if (tq == -2 || tq == t) continue;  // outside the image, or the same triangle
-            const int qx = x + ddx, qy = y + ddy;
-            int vq[3] = {0, 0, 0};
-            VRec rq[3];
-            if (tq >= 0) {
-                if (tq >= a.T || !fwd_tri_ids(tris, tq, a.V, vq)) {
-                    set_status(ws, kStatusRange);
-                    continue;
+            const int ddx = d == 0 ? -1 : (d == 1 ? 1 : 0), ddy = d == 2 ? -1 : (d == 3 ? 1 : 0);
+            const int tq = sidx[ty + 1 + ddy][tx + 1 + ddx];
+            // not outside the image, not the same triangle, not both background
+            m[d] = __ballot_sync(full, live && tq != -2 && tq != t && (t >= 0 || tq >= 0));
+            np[d + 1] = np[d] + __popc(m[d]);
+            srate[ty][tx][d] = __int_as_float(kNoRate);
+        }
+        sown[ty][tx] = t;
+        __syncwarp();
+        // the list's entry i: its direction and lane
+        unsigned short* list = slist[ty];
+        int nk = 0;
+        for (int i0 = 0; i0 < np[4]; i0 += 32) {
+            const int i = i0 + tx;
+            bool keep = false;
+            unsigned code = 0;
+            if (i < np[4]) {
+                const int d = (i >= np[1]) + (i >= np[2]) + (i >= np[3]);
+                const unsigned md = d == 0 ? m[0] : (d == 1 ? m[1] : (d == 2 ? m[2] : m[3]));
+                const int start = d == 0 ? 0 : (d == 1 ? np[1] : (d == 2 ? np[2] : np[3]));
+                const int src = (int)__fns(md, 0, i - start + 1);
+                const int ddx = d == 0 ? -1 : (d == 1 ? 1 : 0), ddy = d == 2 ? -1 : (d == 3 ? 1 : 0);
+                const int tp = sown[ty][src], tq = sidx[ty + 1 + ddy][src + 1 + ddx];
+                const int px = blockIdx.x * kFTW + src, qx = px + ddx, qy = y + ddy;
+                bool p_in_q = tq < 0, q_in_p = tp < 0;  // against the background, the covered pixel is on top
+                keep = true;
+                int v[3];
+                if (tq >= 0) {
+                    if (tq >= a.T || !fwd_tri_ids(tris, tq, a.V, v)) {
+                        set_status(ws, kStatusRange);
+                        keep = false;
+                    } else if (tp >= 0) {
+                        p_in_q = covers_centre(vb, v, px, y);
+                    }
                 }
-                rq[0] = load_vrec(vb + vq[0]);
-                rq[1] = load_vrec(vb + vq[1]);
-                rq[2] = load_vrec(vb + vq[2]);
-            }
-            if (t < 0 && tq < 0) continue;
-            float dpdt = 0.f;
-            if (t >= 0 && tq >= 0) {
-                const int Xp[3] = {rv[0].X, rv[1].X, rv[2].X}, Yp[3] = {rv[0].Y, rv[1].Y, rv[2].Y};
-                const int Xq[3] = {rq[0].X, rq[1].X, rq[2].X}, Yq[3] = {rq[0].Y, rq[1].Y, rq[2].Y};
-                const bool p_in_q = covers_xy(Xq, Yq, 256 * x + 128, 256 * y + 128);
-                const bool q_in_p = covers_xy(Xp, Yp, 256 * qx + 128, 256 * qy + 128);
-                if (!p_in_q && !q_in_p) continue;  // adjacent
-                const int axis = ddx != 0 ? 0 : 1;
-                if (p_in_q && q_in_p) {
-                    if (!(a.terms & MER_INTERSECT)) continue;
-                    // Eq. 12 on both fragments, slice (axis, zeta)
-                    float Np[3], Nq[3], drp[3], drq[3];
-                    plane_normal(rv, Np);
-                    plane_normal(rq, Nq);
-                    const float np0 = Np[axis], np1 = Np[2], nq0 = Nq[axis], nq1 = Nq[2];
-                    const float den_p = diff_of_products(nq0, np1, nq1, np0);  // v = p, f = q
-                    const float mag = sqrtf((np0 * np0 + np1 * np1) * (nq0 * nq0 + nq1 * nq1));
-                    if (!(fabsf(den_p) > 1e-12f * mag)) continue;
-                    const float den_q = -den_p;  // v = q, f = p
-                    frag_motion(rv, vid, tb, x, y, drp);
-                    frag_motion(rq, vq, tb, qx, qy, drq);
-                    dpdt = (-nq1 / den_p) * (np0 * drp[axis] + np1 * drp[2]) +
-                           (-np1 / den_q) * (nq0 * drq[axis] + nq1 * drq[2]);
-                } else {
-                    dpdt = p_in_q ? overhang_rate(rv, vid, tb, x, y, qx, qy, axis, exact)
-                                  : overhang_rate(rq, vq, tb, qx, qy, x, y, axis, exact);
+                if (keep && tp >= 0 && tq >= 0) {
+                    fwd_tri_ids(tris, tp, a.V, v);
+                    q_in_p = covers_centre(vb, v, qx, qy);
+                    keep = p_in_q || q_in_p;  // neither: adjacent
+                    if (p_in_q && q_in_p && !(a.terms & MER_INTERSECT)) keep = false;
                 }
-            } else {
-                const int axis = ddx != 0 ? 0 : 1;
-                dpdt = t >= 0 ? overhang_rate(rv, vid, tb, x, y, qx, qy, axis, exact)
-                              : overhang_rate(rq, vq, tb, qx, qy, x, y, axis, exact);
+                code = (unsigned)(src | (d << 5) | (p_in_q ? 128 : 0) | (q_in_p ? 256 : 0));
             }
+            const unsigned kb = __ballot_sync(full, keep);
+            if (keep) list[nk + __popc(kb & ((1u << tx) - 1u))] = (unsigned short)code;
+            nk += __popc(kb);
+        }
+        __syncwarp();
+        for (int i = tx; i < nk; i += 32) {
+            const unsigned code = list[i];
+            const int src = code & 31, d = (code >> 5) & 3;
+            const int ddx = d == 0 ? -1 : (d == 1 ? 1 : 0), ddy = d == 2 ? -1 : (d == 3 ? 1 : 0);
+            const int axis = ddx != 0 ? 0 : 1;
+            const int tp = sown[ty][src], tq = sidx[ty + 1 + ddy][src + 1 + ddx];
+            const int px = blockIdx.x * kFTW + src, qx = px + ddx, qy = y + ddy;
+            const bool p_in_q = (code & 128) != 0, q_in_p = (code & 256) != 0;
+            float rate;
+            if (p_in_q && q_in_p) {
+                // Eq. 12 on both fragments, slice (axis, zeta)
+                int vp[3], vq[3];
+                fwd_tri_ids(tris, tp, a.V, vp);
+                fwd_tri_ids(tris, tq, a.V, vq);
+                const VRec rp[3] = {load_vrec(vb + vp[0]), load_vrec(vb + vp[1]), load_vrec(vb + vp[2])};
+                const VRec rq[3] = {load_vrec(vb + vq[0]), load_vrec(vb + vq[1]), load_vrec(vb + vq[2])};
+                float Np[3], Nq[3], drp[3], drq[3];
+                plane_normal(rp, Np);
+                plane_normal(rq, Nq);
+                const float np0 = axis == 0 ? Np[0] : Np[1], np1 = Np[2], nq0 = axis == 0 ? Nq[0] : Nq[1], nq1 = Nq[2];
+                const float den_p = diff_of_products(nq0, np1, nq1, np0);  // v = p, f = q
+                const float mag = sqrtf((np0 * np0 + np1 * np1) * (nq0 * nq0 + nq1 * nq1));
+                if (!(fabsf(den_p) > 1e-12f * mag)) continue;
+                const float den_q = -den_p;  // v = q, f = p
+                frag_motion(rp, vp, tb, px, y, drp);
+                frag_motion(rq, vq, tb, qx, qy, drq);
+                rate = (-nq1 / den_p) * (np0 * (axis == 0 ? drp[0] : drp[1]) + np1 * drp[2]) +
+                       (-np1 / den_q) * (nq0 * (axis == 0 ? drq[0] : drq[1]) + nq1 * drq[2]);
+            } else {  // the fragment on top: p's if p's centre lies in q's triangle
+                int v[3];
+                fwd_tri_ids(tris, p_in_q ? tp : tq, a.V, v);
+                const VRec r[3] = {load_vrec(vb + v[0]), load_vrec(vb + v[1]), load_vrec(vb + v[2])};
+                rate = p_in_q ? overhang_rate(r, v, tb, px, y, qx, qy, axis, exact)
+                              : overhang_rate(r, v, tb, qx, qy, px, y, axis, exact);
+            }
+            srate[ty][src][d] = rate;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int d = 0; d < 4; ++d) {
+            const float rate = srate[ty][tx][d];
+            if (__float_as_int(rate) == kNoRate) continue;
+            const int ddx = d == 0 ? -1 : (d == 1 ? 1 : 0), ddy = d == 2 ? -1 : (d == 3 ? 1 : 0);
             // Eq. 11 transposed: both pixels of the pair change by 1/2 (I_A - I_B) dp/dtheta, A = left/top
-            const size_t q = (size_t)qy * a.W + qx;
+            const size_t q = (size_t)(y + ddy) * a.W + (x + ddx);
             const float* ia = (ddx > 0 || ddy > 0) ? img + p * C : img + q * C;
             const float* ib = (ddx > 0 || ddy > 0) ? img + q * C : img + p * C;
 #pragma unroll
-            for (int c = 0; c < kMaxC; ++c) {
+            for (int c = 0; c < kC; ++c) {
                 if (c >= C) break;
-                acc[c] += 0.5f * (__ldg(ia + c) - __ldg(ib + c)) * dpdt;
+                acc[c] += 0.5f * (__ldg(ia + c) - __ldg(ib + c)) * rate;
             }
         }
     }
+    if (!live) return;
     float* o = out + ((size_t)view * plane + p) * C;
 #pragma unroll
-    for (int c = 0; c < kMaxC; ++c)
+    for (int c = 0; c < kC; ++c)
         if (c < C) o[c] = acc[c];
 }
 
@@ -318,7 +394,14 @@ extern "C" int mer_launch_forward_grad(const mer_vertex* vpix, int V, const int*
     a.tex_stride = sh->tex_c > 0 ? sh->tex_c : sh->n_main;
     a.tex_vec4 = false;
     const dim3 grid((unsigned)((W + kFTW - 1) / kFTW), (unsigned)((H + kFTH - 1) / kFTH), (unsigned)n);
-    k_forward_grad<<<grid, dim3(kFTW, kFTH), 0, s>>>(vpix, tris, index, image, tangent, attr, tex, a, out, ws);
+#define MER_FWD(F) \
+    k_forward_grad<F><<<grid, dim3(kFTW, kFTH), 0, s>>>(vpix, tris, index, image, tangent, attr, tex, a, out, ws)
+    switch (sh->C <= kFastC ? shade_form(attr, tex, sh) : kGeneric) {
+        case kTex3: MER_FWD(kTex3); break;
+        case kAttr3: MER_FWD(kAttr3); break;
+        default: MER_FWD(kGeneric); break;
+    }
+#undef MER_FWD
     return cudaGetLastError() == cudaSuccess ? 0 : 2;
 }
 
