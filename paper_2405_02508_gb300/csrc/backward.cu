@@ -22,6 +22,7 @@
 
 #include <cstdint>
 
+#include "launch.cuh"
 #include "shade_device.cuh"
 
 namespace mer {
@@ -699,6 +700,7 @@ __global__ void __launch_bounds__(kThreads, kViewCtasPerSm) k_backward(const mer
                                                        const float* __restrict__ tex, BwdArgs a,
                                                        double* __restrict__ grad_vpix, float* __restrict__ grad_attr,
                                                        void* ws) {
+    after_previous();
     __shared__ BwdShared<NA, EXACT, BITS> S;
     const int tiles_per_view = a.ntx * a.nty;
     const int view = blockIdx.x / tiles_per_view;
@@ -731,6 +733,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_backward_batch(const m
                                                              const float* __restrict__ tex, BwdArgs a,
                                                              double* __restrict__ grad_vpix,
                                                              float* __restrict__ grad_attr, void* ws) {
+    after_previous();
     __shared__ BwdShared<NA, EXACT, BITS> S;
     __shared__ long long s_tile;
     WsHeader* hdr = reinterpret_cast<WsHeader*>(ws);
@@ -858,7 +861,7 @@ extern "C" int mer_launch_backward_batch(const mer_vertex* vpix, const int* tris
     do {                                                                                                           \
         grid = grid_of((const void*)k_backward_batch<F, A, E, BITS>);                                              \
         if (grid == 0) return 2;                                                                                   \
-        k_backward_batch<F, A, E, BITS><<<grid, kThreads, 0, s>>>(vpix, tris, items, n_items, btiles, index,      \
+        launch_chained(k_backward_batch<F, A, E, BITS>, grid, kThreads, s, vpix, tris, items, n_items, btiles, index,      \
                                                                   cover, image, grad_image, attr, tex, a,         \
                                                                   grad_vpix, grad_attr, ws);                      \
     } while (0)
@@ -886,7 +889,7 @@ extern "C" int mer_launch_backward(const mer_vertex* vpix, int V, const int* tri
     if (blocks == 0) return 0;
     const bool exact = (terms & MER_EXACT_CROSSING) != 0;
 #define MER_BWD(F, A, E, BITS)                                                                                      \
-    k_backward<F, A, E, BITS><<<(unsigned)blocks, kThreads, 0, s>>>(vpix, tris, index, cover, image, grad_image, attr, \
+    launch_chained(k_backward<F, A, E, BITS>, (unsigned)blocks, kThreads, s, vpix, tris, index, cover, image, grad_image, attr, \
                                                                     tex, a, grad_vpix, grad_attr, ws)
     const bool dense = (double)T > kDenseTrianglesPerPixel * (double)H * (double)W;
     MER_BWD_DISPATCH(MER_BWD);

@@ -15,6 +15,7 @@
 
 #include <cstdint>
 
+#include "launch.cuh"
 #include "shade_device.cuh"
 
 namespace mer {
@@ -358,6 +359,7 @@ __global__ void __launch_bounds__(kDetThreads) k_backward_det(const mer_vertex* 
                                                               const float* __restrict__ tex, DetArgs a, int n, int H,
                                                               int W, int V, int T, unsigned long long* acc_v,
                                                               unsigned long long* acc_a, void* ws) {
+    after_previous();
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long plane = (long long)H * W;
     const bool live = g < (long long)n * plane;
@@ -391,6 +393,7 @@ __global__ void __launch_bounds__(kDetThreads) k_backward_det_batch(const mer_ve
                                                                     const float* __restrict__ tex, DetArgs a,
                                                                     unsigned long long* acc_v,
                                                                     unsigned long long* acc_a, void* ws) {
+    after_previous();
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int k = block_find_item(items, n_items, (long long)blockIdx.x * blockDim.x, g, kFieldPix);
     const bool live = g < pixels;
@@ -421,6 +424,7 @@ __global__ void __launch_bounds__(kDetThreads) k_backward_det_batch(const mer_ve
 __global__ void k_det_finalize(const unsigned long long* __restrict__ acc_v, long long nv, double* __restrict__ grad_vpix,
                                const unsigned long long* __restrict__ acc_a, long long arows, int A, int a0, int Ca,
                                float* __restrict__ grad_attr) {
+    after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < nv) grad_vpix[i] += fix_value((long long)acc_v[2 * i], (long long)acc_v[2 * i + 1]);
     if (grad_attr && i < arows * A) {
@@ -459,7 +463,7 @@ int det_finish(unsigned long long* acc_v, long long vrows, double* grad_vpix, un
     const long long nv = 3 * vrows, na = grad_attr ? arows * a.A : 0;
     const long long m = nv > na ? nv : na;
     if (m > 0)
-        k_det_finalize<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(acc_v, nv, grad_vpix, acc_a, arows, a.A, a.a0,
+        launch_chained(k_det_finalize, (unsigned)((m + 255) / 256), 256, s, acc_v, nv, grad_vpix, acc_a, arows, a.A, a.a0,
                                                                   a.sh.C_attr, grad_attr);
     return cudaGetLastError() == cudaSuccess ? 0 : 2;
 }
@@ -480,7 +484,7 @@ extern "C" int mer_launch_backward_det(const mer_vertex* vpix, int V, const int*
     if (bytes > 0 && cudaMemsetAsync(acc_v, 0, bytes, s) != cudaSuccess) return 2;
     const long long npix = (long long)n * H * W;
     if (npix > 0)
-        k_backward_det<<<(unsigned)((npix + kDetThreads - 1) / kDetThreads), kDetThreads, 0, s>>>(
+        launch_chained(k_backward_det, (unsigned)((npix + kDetThreads - 1) / kDetThreads), kDetThreads, s, 
             vpix, tris, index, image, grad_image, attr, tex, a, n, H, W, V, T, acc_v, acc_a, ws);
     if (cudaGetLastError() != cudaSuccess) return 2;
     return det_finish(acc_v, vrows, grad_vpix, acc_a, V, a, grad_attr, s);
@@ -500,7 +504,7 @@ extern "C" int mer_launch_backward_det_batch(const mer_vertex* vpix, const int* 
     const size_t bytes = mer_det_workspace_size(vrecs, grad_attr ? mesh_rows : 0, a.A) - 256;
     if (bytes > 0 && cudaMemsetAsync(acc_v, 0, bytes, s) != cudaSuccess) return 2;
     if (pixels > 0)
-        k_backward_det_batch<<<(unsigned)((pixels + kDetThreads - 1) / kDetThreads), kDetThreads, 0, s>>>(
+        launch_chained(k_backward_det_batch, (unsigned)((pixels + kDetThreads - 1) / kDetThreads), kDetThreads, s, 
             vpix, tris, items, n_items, pixels, index, image, grad_image, attr, tex, a, acc_v, acc_a, ws);
     if (cudaGetLastError() != cudaSuccess) return 2;
     return det_finish(acc_v, vrecs, grad_vpix, acc_a, mesh_rows, a, grad_attr, s);

@@ -22,6 +22,7 @@
 
 #include <cstdint>
 
+#include "launch.cuh"
 #include "shade_device.cuh"
 
 namespace mer {
@@ -127,6 +128,7 @@ __global__ void __launch_bounds__(kFTW * kFTH) k_forward_grad(const mer_vertex* 
                                                             const float* __restrict__ attr,
                                                             const float* __restrict__ tex, FwdArgs a,
                                                             float* __restrict__ out, void* ws) {
+    after_previous();
     constexpr int kC = FORM == kGeneric ? kMaxC : kFastC;
     __shared__ int sidx[kFTH + 2][kFTW + 2];
     __shared__ int sown[kFTH][kFTW];            // the pixels' triangles, -1 if none or out of range
@@ -357,6 +359,7 @@ __global__ void __launch_bounds__(kFTW * kFTH) k_forward_grad(const mer_vertex* 
 // d(x_s, y_s, zeta) = J(X_c) R d(X_w), J as in the projection backward.
 __global__ void k_project_jvp(const float* __restrict__ tw, int V, const mer_camera* __restrict__ cams, int n,
                               const mer_vertex* __restrict__ vpix, float* __restrict__ out) {
+    after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (long long)V * n) return;
     const int view = (int)(i / V), v = (int)(i % V);
@@ -395,7 +398,7 @@ extern "C" int mer_launch_forward_grad(const mer_vertex* vpix, int V, const int*
     a.tex_vec4 = false;
     const dim3 grid((unsigned)((W + kFTW - 1) / kFTW), (unsigned)((H + kFTH - 1) / kFTH), (unsigned)n);
 #define MER_FWD(F) \
-    k_forward_grad<F><<<grid, dim3(kFTW, kFTH), 0, s>>>(vpix, tris, index, image, tangent, attr, tex, a, out, ws)
+    launch_chained(k_forward_grad<F>, grid, dim3(kFTW, kFTH), s, vpix, tris, index, image, tangent, attr, tex, a, out, ws)
     switch (sh->C <= kFastC ? shade_form(attr, tex, sh) : kGeneric) {
         case kTex3: MER_FWD(kTex3); break;
         case kAttr3: MER_FWD(kAttr3); break;
@@ -408,6 +411,6 @@ extern "C" int mer_launch_forward_grad(const mer_vertex* vpix, int V, const int*
 extern "C" int mer_launch_project_jvp(const float* tangent_world, int V, const mer_camera* cams, int n,
                                       const mer_vertex* vpix, float* out, cudaStream_t s) {
     const long long N = (long long)V * n;
-    k_project_jvp<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(tangent_world, V, cams, n, vpix, out);
+    launch_chained(k_project_jvp, (unsigned)((N + 255) / 256), 256, s, tangent_world, V, cams, n, vpix, out);
     return cudaGetLastError() == cudaSuccess ? 0 : 2;
 }

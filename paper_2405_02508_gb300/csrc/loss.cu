@@ -5,12 +5,14 @@
 
 #include <cstdint>
 
+#include "launch.cuh"
 #include "mer_device.cuh"
 
 namespace mer {
 
 __global__ void k_l2_loss_grad(const float* __restrict__ image, const float* __restrict__ target, long long n,
                                float* __restrict__ grad, double* __restrict__ loss) {
+    after_previous();
     __shared__ double sh[8];
     double acc = 0.0;
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -68,6 +70,6 @@ extern "C" int mer_l2_loss_grad(const float* image, const float* target, int64_t
         return MER_ECUDA;
     const long long want = (n / 4 + 255) / 256 + 1;
     const unsigned grid = (unsigned)(want < 8LL * sms ? want : 8LL * sms);
-    k_l2_loss_grad<<<grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(image, target, n, grad, loss);
+    launch_chained(k_l2_loss_grad, grid, 256, static_cast<cudaStream_t>(stream), image, target, n, grad, loss);
     return cudaGetLastError() == cudaSuccess ? MER_OK : MER_ECUDA;
 }

@@ -11,6 +11,7 @@
 
 #include <cstdint>
 
+#include "launch.cuh"
 #include "mer_device.cuh"
 
 namespace mer {
@@ -32,6 +33,7 @@ __device__ __forceinline__ bool tri_fetch(const int* __restrict__ tris, long lon
 
 __global__ void k_face_accumulate(const float* __restrict__ verts, const int* __restrict__ tris, long long T, int V,
                                   float* __restrict__ acc, void* ws) {
+    after_previous();
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= T) return;
     int v[3];
@@ -55,6 +57,7 @@ __global__ void k_face_accumulate(const float* __restrict__ verts, const int* __
 }
 
 __global__ void k_normalize(const float* __restrict__ acc, long long V, float* __restrict__ out) {
+    after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= V) return;
     const float a0 = acc[3 * i], a1 = acc[3 * i + 1], a2 = acc[3 * i + 2];
@@ -66,6 +69,7 @@ __global__ void k_normalize(const float* __restrict__ acc, long long V, float* _
 
 // dL/da_v in place of dL/dn_v.
 __global__ void k_normalize_backward(const float* __restrict__ acc, long long V, float* __restrict__ g) {
+    after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= V) return;
     const float a[3] = {acc[3 * i], acc[3 * i + 1], acc[3 * i + 2]};
@@ -87,6 +91,7 @@ __global__ void k_normalize_backward(const float* __restrict__ acc, long long V,
 // dL/dp1 = e2 x G, dL/dp2 = G x e1, dL/dp0 = -(dL/dp1 + dL/dp2).
 __global__ void k_face_backward(const float* __restrict__ verts, const int* __restrict__ tris, long long T, int V,
                                 const float* __restrict__ ga, float* __restrict__ grad_verts, void* ws) {
+    after_previous();
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= T) return;
     int v[3];
@@ -130,8 +135,8 @@ extern "C" int mer_vertex_normals(const float* verts, int V, const int32_t* tris
     if (!verts || !acc || !normals || (T > 0 && !tris) || acc == normals) return MER_EINVAL;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (cudaMemsetAsync(acc, 0, (size_t)V * 3 * sizeof(float), s) != cudaSuccess) return MER_ECUDA;
-    if (T > 0) k_face_accumulate<<<blocks(T), 256, 0, s>>>(verts, tris, T, V, acc, status_ws);
-    k_normalize<<<blocks(V), 256, 0, s>>>(acc, V, normals);
+    if (T > 0) launch_chained(k_face_accumulate, blocks(T), 256, s, verts, tris, T, V, acc, status_ws);
+    launch_chained(k_normalize, blocks(V), 256, s, acc, V, normals);
     return cudaGetLastError() == cudaSuccess ? MER_OK : MER_ECUDA;
 }
 
@@ -142,7 +147,7 @@ extern "C" int mer_vertex_normals_backward(const float* verts, int V, const int3
     if (V == 0) return MER_OK;
     if (!verts || !acc || !grad_normals || !grad_verts || (T > 0 && !tris)) return MER_EINVAL;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    k_normalize_backward<<<blocks(V), 256, 0, s>>>(acc, V, grad_normals);
-    if (T > 0) k_face_backward<<<blocks(T), 256, 0, s>>>(verts, tris, T, V, grad_normals, grad_verts, status_ws);
+    launch_chained(k_normalize_backward, blocks(V), 256, s, acc, V, grad_normals);
+    if (T > 0) launch_chained(k_face_backward, blocks(T), 256, s, verts, tris, T, V, grad_normals, grad_verts, status_ws);
     return cudaGetLastError() == cudaSuccess ? MER_OK : MER_ECUDA;
 }

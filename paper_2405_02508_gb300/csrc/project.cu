@@ -7,6 +7,7 @@
 // in FP32 with atomics, or, given a workspace, in FP64 with fixed-point sums (bitwise reproducible).
 #include <cuda_runtime.h>
 
+#include "launch.cuh"
 #include "mer_device.cuh"
 
 namespace mer {
@@ -64,6 +65,7 @@ __device__ __forceinline__ void project_one(const float* __restrict__ w, const m
 __global__ void k_project(const float* __restrict__ verts, int V, const mer_camera* __restrict__ cams, int n,
                           mer_vertex* __restrict__ out, mer_vertex* __restrict__ out2, int* __restrict__ clear,
                           long long n_clear) {
+    after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     for (long long k = i; k < n_clear; k += (long long)gridDim.x * blockDim.x) clear[k] = 0;
     if (i >= (long long)V * n) return;
@@ -74,6 +76,7 @@ __global__ void k_project(const float* __restrict__ verts, int V, const mer_came
 __global__ void k_project_batch(const float* __restrict__ verts, const mer_camera* __restrict__ cams,
                                 const mer_item* __restrict__ items, int n_items, long long vrecs,
                                 mer_vertex* __restrict__ out) {
+    after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int k = block_find_item(items, n_items, (long long)blockIdx.x * blockDim.x, i, kFieldVrec);
     if (i >= vrecs) return;
@@ -82,6 +85,7 @@ __global__ void k_project_batch(const float* __restrict__ verts, const mer_camer
 }
 
 __global__ void k_project_screen(const double* __restrict__ scr, int V, int n, mer_vertex* __restrict__ out) {
+    after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (long long)V * n) return;
     const double xs = scr[3 * i], ys = scr[3 * i + 1], zeta = scr[3 * i + 2];
@@ -144,6 +148,7 @@ __device__ __forceinline__ bool world_grad_f64(const mer_vertex& r, const mer_ca
 __global__ void k_project_backward_batch(const mer_camera* __restrict__ cams, const mer_item* __restrict__ items,
                                          int n_items, long long vrecs, const mer_vertex* __restrict__ vpix,
                                          const double* __restrict__ grad_vpix, float* __restrict__ grad_verts) {
+    after_previous();
     __shared__ CameraF s_cam;  // of the block's first item
     __shared__ int s_item;
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -172,6 +177,7 @@ __global__ void k_project_backward_batch_fixed(const mer_camera* __restrict__ ca
                                                int n_items, long long vrecs, const mer_vertex* __restrict__ vpix,
                                                const double* __restrict__ grad_vpix, unsigned long long* acc,
                                                void* ws) {
+    after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int k = block_find_item(items, n_items, (long long)blockIdx.x * blockDim.x, i, kFieldVrec);
     if (i >= vrecs) return;
@@ -194,6 +200,7 @@ __global__ void k_project_backward_batch_fixed(const mer_camera* __restrict__ ca
 }
 
 __global__ void k_world_finalize(const unsigned long long* __restrict__ acc, long long n, float* __restrict__ grad_verts) {
+    after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const long long lo = (long long)acc[2 * i + 1];
@@ -207,6 +214,7 @@ template <bool STORE>
 __global__ void k_project_backward(int V, const mer_camera* __restrict__ cams, int n,
                                    const mer_vertex* __restrict__ vpix, const double* __restrict__ grad_vpix,
                                    float* __restrict__ grad_verts, float* __restrict__ copy) {
+    after_previous();
     const int v = blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= V) return;
     double a0 = 0.0, a1 = 0.0, a2 = 0.0;
@@ -236,14 +244,14 @@ extern "C" int mer_launch_project(const float* verts, int V, const mer_camera* c
                                   mer_vertex* copy, int* clear, long long n_clear, cudaStream_t s) {
     const long long N = (long long)V * n;
     if (N == 0) return 0;
-    k_project<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(verts, V, cams, n, vpix, copy, clear, n_clear);
+    launch_chained(k_project, (unsigned)((N + 255) / 256), 256, s, verts, V, cams, n, vpix, copy, clear, n_clear);
     return cudaGetLastError() == cudaSuccess ? 0 : 2;
 }
 
 extern "C" int mer_launch_project_screen(const double* scr, int V, int n, mer_vertex* vpix, cudaStream_t s) {
     const long long N = (long long)V * n;
     if (N == 0) return 0;
-    k_project_screen<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(scr, V, n, vpix);
+    launch_chained(k_project_screen, (unsigned)((N + 255) / 256), 256, s, scr, V, n, vpix);
     return cudaGetLastError() == cudaSuccess ? 0 : 2;
 }
 
@@ -252,16 +260,16 @@ extern "C" int mer_launch_project_backward(int V, const mer_camera* cams, int n,
                                            cudaStream_t s) {
     if (V == 0 || n == 0) return 0;
     if (store)
-        k_project_backward<true><<<(V + 255) / 256, 256, 0, s>>>(V, cams, n, vpix, grad_vpix, grad_verts, copy);
+        launch_chained(k_project_backward<true>, (V + 255) / 256, 256, s, V, cams, n, vpix, grad_vpix, grad_verts, copy);
     else
-        k_project_backward<false><<<(V + 255) / 256, 256, 0, s>>>(V, cams, n, vpix, grad_vpix, grad_verts, copy);
+        launch_chained(k_project_backward<false>, (V + 255) / 256, 256, s, V, cams, n, vpix, grad_vpix, grad_verts, copy);
     return cudaGetLastError() == cudaSuccess ? 0 : 2;
 }
 
 extern "C" int mer_launch_project_batch(const float* verts, const mer_camera* cams, const mer_item* items, int n_items,
                                         long long vrecs, mer_vertex* vpix, cudaStream_t s) {
     if (vrecs == 0) return 0;
-    k_project_batch<<<(unsigned)((vrecs + 255) / 256), 256, 0, s>>>(verts, cams, items, n_items, vrecs, vpix);
+    launch_chained(k_project_batch, (unsigned)((vrecs + 255) / 256), 256, s, verts, cams, items, n_items, vrecs, vpix);
     return cudaGetLastError() == cudaSuccess ? 0 : 2;
 }
 
@@ -275,19 +283,20 @@ extern "C" int mer_launch_project_backward_batch(const mer_camera* cams, const m
     if (ws) {
         unsigned long long* acc = reinterpret_cast<unsigned long long*>(static_cast<char*>(ws) + 256);
         if (cudaMemsetAsync(acc, 0, (size_t)mesh_rows * 48, s) != cudaSuccess) return 2;
-        k_project_backward_batch_fixed<<<(unsigned)((vrecs + 255) / 256), 256, 0, s>>>(cams, items, n_items, vrecs,
+        launch_chained(k_project_backward_batch_fixed, (unsigned)((vrecs + 255) / 256), 256, s, cams, items, n_items, vrecs,
                                                                                        vpix, grad_vpix, acc, ws);
         const long long n = 3 * mesh_rows;
-        if (n > 0) k_world_finalize<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(acc, n, grad_verts);
+        if (n > 0) launch_chained(k_world_finalize, (unsigned)((n + 255) / 256), 256, s, acc, n, grad_verts);
         return cudaGetLastError() == cudaSuccess ? 0 : 2;
     }
-    k_project_backward_batch<<<(unsigned)((vrecs + 255) / 256), 256, 0, s>>>(cams, items, n_items, vrecs, vpix,
+    launch_chained(k_project_backward_batch, (unsigned)((vrecs + 255) / 256), 256, s, cams, items, n_items, vrecs, vpix,
                                                                              grad_vpix, grad_verts);
     return cudaGetLastError() == cudaSuccess ? 0 : 2;
 }
 
 namespace mer {
 __global__ void k_clear(double* __restrict__ a, long long na, float* __restrict__ b, long long nb) {
+    after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < na) a[i] = 0.0;
     if (i < nb) b[i] = 0.f;
@@ -297,6 +306,6 @@ __global__ void k_clear(double* __restrict__ a, long long na, float* __restrict_
 // Zeroes two gradient arrays in one launch.
 extern "C" int mer_launch_clear(double* a, long long na, float* b, long long nb, cudaStream_t s) {
     const long long m = na > nb ? na : nb;
-    if (m > 0) k_clear<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(a, na, b, nb);
+    if (m > 0) launch_chained(k_clear, (unsigned)((m + 255) / 256), 256, s, a, na, b, nb);
     return cudaGetLastError() == cudaSuccess ? 0 : 2;
 }

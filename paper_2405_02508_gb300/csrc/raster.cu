@@ -15,6 +15,7 @@
 
 #include <mutex>
 
+#include "launch.cuh"
 #include "shade_device.cuh"
 
 namespace mer {
@@ -201,6 +202,7 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* sh, int& total) 
 }
 
 __global__ void k_scan_blocks(const int* __restrict__ in, long long N, int* __restrict__ out, int* __restrict__ sums) {
+    after_previous();
     __shared__ int sh[32];
     const long long i = (long long)blockIdx.x * kScanBlock + threadIdx.x;
     const int v = i < N ? in[i] : 0;
@@ -212,6 +214,7 @@ __global__ void k_scan_blocks(const int* __restrict__ in, long long N, int* __re
 
 // Single CTA: exclusive scan of the block sums (looping), total written to the header.
 __global__ void k_scan_sums(int* __restrict__ sums, int nb, void* ws, long long capacity) {
+    after_previous();
     __shared__ int sh[32];
     int carry = 0;
     for (int base = 0; base < nb; base += kScanBlock) {
@@ -233,6 +236,7 @@ __global__ void k_scan_sums(int* __restrict__ sums, int nb, void* ws, long long 
 
 // Adds the block offsets and clears the front and back fill cursors (cursor[0, 2N)).
 __global__ void k_scan_add(int* __restrict__ out, long long N, const int* __restrict__ sums, int* __restrict__ cursor) {
+    after_previous();
     const long long i = (long long)blockIdx.x * kScanBlock + threadIdx.x;
     if (i < N) {
         out[i] += sums[blockIdx.x];
@@ -250,6 +254,7 @@ constexpr long long kHostReady = 1LL << 32;
 __global__ void __launch_bounds__(kScanBlock) k_scan_all(const int* __restrict__ in, int N, int* __restrict__ out,
                                                          int* __restrict__ cursor, void* ws, long long capacity,
                                                          volatile long long* host) {
+    after_previous();
     __shared__ int sh[32];
     const int each = (N + kScanBlock - 1) / kScanBlock;
     const int i0 = threadIdx.x * each;
@@ -287,6 +292,7 @@ __global__ void __launch_bounds__(kScanBlock) k_scan_all(const int* __restrict__
 
 // The same two words for the host after a scan in several launches.
 __global__ void k_host_status(const void* ws, volatile long long* host) {
+    after_previous();
     const WsHeader* h = reinterpret_cast<const WsHeader*>(ws);
     host[1] = h->total_bins;
     __threadfence_system();
@@ -541,6 +547,7 @@ __device__ __forceinline__ RItem view_item(const BinGeom& g, const mer_vertex* v
 
 __global__ void k_setup_count(const mer_vertex* __restrict__ vpix, const int* __restrict__ tris, BinGeom g,
                               TriRaster* __restrict__ recs, int* __restrict__ counts, void* ws) {
+    after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (long long)g.T * g.n) return;
     const int view = (int)(i / g.T), t = (int)(i % g.T);
@@ -550,6 +557,7 @@ __global__ void k_setup_count(const mer_vertex* __restrict__ vpix, const int* __
 __global__ void k_bin_fill(const mer_vertex* __restrict__ vpix, const int* __restrict__ tris, BinGeom g,
                            TriRaster* __restrict__ recs, const int* __restrict__ offs, const int* __restrict__ counts,
                            int* __restrict__ cursor, int* __restrict__ list, long long capacity) {
+    after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (long long)g.T * g.n) return;
     const int view = (int)(i / g.T), t = (int)(i % g.T);
@@ -566,6 +574,7 @@ __global__ void __launch_bounds__(kRasterThreads, kRasterCtasPerSm) k_raster(Tri
                                                            int* __restrict__ index, float* __restrict__ depth,
                                                            float* __restrict__ bary, unsigned char* __restrict__ cover,
                                                            ShadeOut so) {
+    after_previous();
     __shared__ RasterShared<TS> S;
     const WsHeader* hdr = reinterpret_cast<const WsHeader*>(ws);
     const bool overflow = hdr->total_bins > capacity;
@@ -600,6 +609,7 @@ __device__ __forceinline__ RItem batch_item(const mer_item& m, int tile, const m
 
 __global__ void k_setup_count_batch(const mer_vertex* __restrict__ vpix, const int* __restrict__ tris, BatchGeom b,
                                     TriRaster* __restrict__ recs, int* __restrict__ counts, void* ws) {
+    after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int k = block_find_item(b.items, b.n_items, (long long)blockIdx.x * blockDim.x, i, kFieldTrec);
     if (i >= b.trecs) return;
@@ -611,6 +621,7 @@ __global__ void k_bin_fill_batch(const mer_vertex* __restrict__ vpix, const int*
                                  TriRaster* __restrict__ recs, const int* __restrict__ offs,
                                  const int* __restrict__ counts, int* __restrict__ cursor, int* __restrict__ list,
                                  long long capacity) {
+    after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int k = block_find_item(b.items, b.n_items, (long long)blockIdx.x * blockDim.x, i, kFieldTrec);
     if (i >= b.trecs) return;
@@ -631,6 +642,7 @@ __global__ void __launch_bounds__(kRasterThreads, kRasterCtasPerSm) k_raster_bat
                                                                  long long capacity, int* __restrict__ index,
                                                                  float* __restrict__ depth, float* __restrict__ bary,
                                                                  unsigned char* __restrict__ cover, ShadeOut so) {
+    after_previous();
     __shared__ RasterShared<TS> S;
     __shared__ long long s_tile;
     WsHeader* hdr = reinterpret_cast<WsHeader*>(ws);
@@ -699,13 +711,13 @@ int launch_scan(const RasterLayout& L, char* base, long long capacity, cudaStrea
     int* cursor = reinterpret_cast<int*>(base + L.cursor);
     int* sums = reinterpret_cast<int*>(base + L.sums);
     if (L.ntiles <= (long long)kScanBlock * kScanEach) {
-        k_scan_all<<<1, kScanBlock, 0, s>>>(counts, (int)L.ntiles, offs, cursor, hdr, capacity, host);
+        launch_chained(k_scan_all, 1, kScanBlock, s, counts, (int)L.ntiles, offs, cursor, hdr, capacity, host);
         return 0;
     }
-    if (L.nblocks > 0) k_scan_blocks<<<(unsigned)L.nblocks, kScanBlock, 0, s>>>(counts, L.ntiles, offs, sums);
-    k_scan_sums<<<1, kScanBlock, 0, s>>>(sums, (int)L.nblocks, hdr, capacity);
-    if (L.nblocks > 0) k_scan_add<<<(unsigned)L.nblocks, kScanBlock, 0, s>>>(offs, L.ntiles, sums, cursor);
-    if (host) k_host_status<<<1, 1, 0, s>>>(hdr, host);
+    if (L.nblocks > 0) launch_chained(k_scan_blocks, (unsigned)L.nblocks, kScanBlock, s, counts, L.ntiles, offs, sums);
+    launch_chained(k_scan_sums, 1, kScanBlock, s, sums, (int)L.nblocks, hdr, capacity);
+    if (L.nblocks > 0) launch_chained(k_scan_add, (unsigned)L.nblocks, kScanBlock, s, offs, L.ntiles, sums, cursor);
+    if (host) launch_chained(k_host_status, 1, 1, s, hdr, host);
     return 0;
 }
 }  // namespace
@@ -724,7 +736,7 @@ static void launch_view_tile(unsigned grid, TriRaster* recs, const BinGeom& g, c
                              const int* cursor, const int* list, const mer_vertex* vpix, const int* tris, void* hdr,
                              long long capacity, int* index, float* depth, float* bary, unsigned char* cover,
                              const ShadeOut& so, cudaStream_t s) {
-    k_raster<TS, FORM, DUAL><<<grid, kRasterThreads, 0, s>>>(recs, g, offs, counts, cursor, list, vpix, tris, hdr, capacity,
+    launch_chained(k_raster<TS, FORM, DUAL>, grid, kRasterThreads, s, recs, g, offs, counts, cursor, list, vpix, tris, hdr, capacity,
                                                              index, depth, bary, cover, so);
 }
 
@@ -753,10 +765,10 @@ static int view_raster(const mer_vertex* vpix, int V, const int* tris, int T, in
     // header: the status word is sticky until mer_sync_status; the scan writes the totals
     if (!cleared && cudaMemsetAsync(counts, 0, (size_t)L.ntiles * 4, s) != cudaSuccess) return 2;
     const long long NT = (long long)T * n;
-    if (NT > 0) k_setup_count<<<(unsigned)((NT + 255) / 256), 256, 0, s>>>(vpix, tris, g, recs, counts, hdr);
+    if (NT > 0) launch_chained(k_setup_count, (unsigned)((NT + 255) / 256), 256, s, vpix, tris, g, recs, counts, hdr);
     launch_scan(L, base, capacity, s, host);
     if (NT > 0)
-        k_bin_fill<<<(unsigned)((NT + 255) / 256), 256, 0, s>>>(vpix, tris, g, recs, offs, counts, cursor, list,
+        launch_chained(k_bin_fill, (unsigned)((NT + 255) / 256), 256, s, vpix, tris, g, recs, offs, counts, cursor, list,
                                                                 capacity);
     const unsigned grid = (unsigned)L.ntiles;
     ShadeOut none;
@@ -840,7 +852,7 @@ static int launch_raster_batch(unsigned grid, TriRaster* recs, BatchGeom b, cons
             return 2;
         grid = (unsigned)(sms * (per_sm > 0 ? per_sm : 1));
     }
-    k_raster_batch<TS, FORM><<<grid, kRasterThreads, 0, s>>>(recs, b, offs, counts, nfront, list, vpix, tris, hdr, capacity,
+    launch_chained(k_raster_batch<TS, FORM>, grid, kRasterThreads, s, recs, b, offs, counts, nfront, list, vpix, tris, hdr, capacity,
                                                               index, depth, bary, cover, so);
     return 0;
 }
@@ -876,10 +888,10 @@ static int batch_raster(const mer_vertex* vpix, const int* tris, const mer_item*
     BatchGeom b;
     b.items = items; b.n_items = n_items; b.tile = tile; b.trecs = trecs; b.tiles = tiles;
     if (tiles > 0 && cudaMemsetAsync(counts, 0, (size_t)tiles * 4, s) != cudaSuccess) return 2;
-    if (trecs > 0) k_setup_count_batch<<<(unsigned)((trecs + 255) / 256), 256, 0, s>>>(vpix, tris, b, recs, counts, hdr);
+    if (trecs > 0) launch_chained(k_setup_count_batch, (unsigned)((trecs + 255) / 256), 256, s, vpix, tris, b, recs, counts, hdr);
     launch_scan(L, base, capacity, s);  // also resets the raster work queue
     if (trecs > 0)
-        k_bin_fill_batch<<<(unsigned)((trecs + 255) / 256), 256, 0, s>>>(vpix, tris, b, recs, offs, counts, cursor, list,
+        launch_chained(k_bin_fill_batch, (unsigned)((trecs + 255) / 256), 256, s, vpix, tris, b, recs, offs, counts, cursor, list,
                                                                         capacity);
     if (tiles > 0) {
         const unsigned grid = persistent_ctas > 0 ? (unsigned)persistent_ctas : 0u;

@@ -8,6 +8,7 @@
 
 #include <cstdint>
 
+#include "launch.cuh"
 #include "shade_device.cuh"
 
 namespace mer {
@@ -29,6 +30,7 @@ template <int FORM>
 __global__ void k_shade(const mer_vertex* __restrict__ vpix, int V, const int* __restrict__ tris, int T, int n, int H,
                         int W, const int* __restrict__ index, const float* __restrict__ attr,
                         const float* __restrict__ tex, ShadeArgs a, float* __restrict__ image, void* ws) {
+    after_previous();
     const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long npix = (long long)n * H * W;
     if (p >= npix) return;
@@ -42,6 +44,7 @@ __global__ void k_shade_batch(const mer_vertex* __restrict__ vpix, const int* __
                               const mer_item* __restrict__ items, int n_items, long long pixels,
                               const int* __restrict__ index, const float* __restrict__ attr,
                               const float* __restrict__ tex, ShadeArgs a, float* __restrict__ image, void* ws) {
+    after_previous();
     const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int k = block_find_item(items, n_items, (long long)blockIdx.x * blockDim.x, p, kFieldPix);
     if (p >= pixels) return;
@@ -63,7 +66,7 @@ extern "C" int mer_launch_shade_batch(const mer_vertex* vpix, const int* tris, c
     const ShadeArgs a = make_shade_args(tex, bg, sh);
     const unsigned blocks = (unsigned)((pixels + 255) / 256);
 #define MER_SHADE(F) \
-    k_shade_batch<F><<<blocks, 256, 0, s>>>(vpix, tris, items, n_items, pixels, index, attr, tex, a, image, ws)
+    launch_chained(k_shade_batch<F>, blocks, 256, s, vpix, tris, items, n_items, pixels, index, attr, tex, a, image, ws)
     switch (sh->precise ? kShadeOff : shade_form(attr, tex, sh)) {
         case kShadeOff: MER_SHADE(kShadeOff); break;
         case kTex3: MER_SHADE(kTex3); break;
@@ -82,7 +85,7 @@ extern "C" int mer_launch_shade(const mer_vertex* vpix, int V, const int* tris, 
     const ShadeArgs a = make_shade_args(tex, bg, sh);
     const unsigned blocks = (unsigned)((npix + 255) / 256);
 #define MER_SHADE(F) \
-    k_shade<F><<<blocks, 256, 0, s>>>(vpix, V, tris, T, n, H, W, index, attr, tex, a, image, ws)
+    launch_chained(k_shade<F>, blocks, 256, s, vpix, V, tris, T, n, H, W, index, attr, tex, a, image, ws)
     switch (sh->precise ? kShadeOff : shade_form(attr, tex, sh)) {
         case kShadeOff: MER_SHADE(kShadeOff); break;
         case kTex3: MER_SHADE(kTex3); break;

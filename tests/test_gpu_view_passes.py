@@ -143,3 +143,27 @@ def test_autograd_with_a_renderer_in_use():
             got = torch.autograd.grad(im, (v, a), g)
             assert torch.equal(im, alone[k][0]) and torch.equal(got[0], alone[k][1]) and torch.equal(got[1], alone[k][2])
             assert torch.equal(r.image, im.detach())  # the renderer's buffers hold what was differentiated
+
+
+def test_passes_back_to_back():
+    """Passes queued without waiting, over two geometries in turn, each give what they give alone (a kernel of a pass is
+    set up while the one before it runs, and must not read what that one has not written yet)."""
+    r, verts, cams, attr, tex = _setup("texture", 301, 333, 2, n=40)
+    g = torch.randn_like(r.image)
+    sets = [verts, verts * 0.8]
+    terms = 7 | B.MER_DETERMINISTIC
+
+    def once(v):
+        r.forward(v, cams, attr, tex, checked=False)
+        gv = r.backward(g, cams, attr, tex, terms=terms)
+        return r.image.clone(), r.index.clone(), gv.clone()
+
+    alone = []
+    for v in sets:
+        torch.cuda.synchronize()
+        alone.append(once(v))
+        torch.cuda.synchronize()
+    got = [once(sets[k % 2]) for k in range(40)]
+    for k, out in enumerate(got):
+        for a, b in zip(out, alone[k % 2]):
+            assert torch.equal(a, b)
