@@ -395,7 +395,7 @@ __global__ void __launch_bounds__(kDetThreads) k_backward_det_batch(const mer_ve
                                                                     unsigned long long* acc_a, void* ws) {
     after_previous();
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int k = block_find_item(items, n_items, (long long)blockIdx.x * blockDim.x, g, kFieldPix);
+    const int k = warp_find_item(items, n_items, g - (threadIdx.x & 31), g, kFieldPix);
     const bool live = g < pixels;
     const mer_item m = items[k];
     const int C = a.sh.C, Ca = a.sh.C_attr;

@@ -14,7 +14,7 @@ namespace mer {
 
 // These kernels are bound by the FP64 pipe (one warp instruction in 16 cycles on an SM), on which conversions count like
 // any operation: 2,097,216 vertices of 32 views took 60 of them each, 201 us for 67 MB.  Exact conversions run on the integer
-// pipes instead (f2d, i2d), the snap is one FMA, and the batched backward converts a camera once a block: 174 us, its
+// pipes instead (f2d, i2d), the snap is one FMA, and the batched backward converts a camera once a warp: 174 us, its
 // backward 75 -> 52.
 
 __device__ __forceinline__ void write_vertex(double xs, double ys, double zeta, bool front, mer_vertex* out,
@@ -78,7 +78,7 @@ __global__ void k_project_batch(const float* __restrict__ verts, const mer_camer
                                 mer_vertex* __restrict__ out) {
     after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int k = block_find_item(items, n_items, (long long)blockIdx.x * blockDim.x, i, kFieldVrec);
+    const int k = warp_find_item(items, n_items, i - (threadIdx.x & 31), i, kFieldVrec);
     if (i >= vrecs) return;
     const mer_item m = items[k];
     project_one(verts + 3 * (size_t)(m.vert + (i - m.vrec)), cams[m.cam], out + i);
@@ -94,7 +94,7 @@ __global__ void k_project_screen(const double* __restrict__ scr, int V, int n, m
 
 // R^T J^T g for one projected vertex, J = d(x_s, y_s, zeta)/d(X_c, Y_c, Z_c)
 // = [[fx z, 0, -(x_s-cx) z], [0, fy z, -(y_s-cy) z], [0, 0, -z^2]]; false if the vertex is behind the camera.
-// (The camera in FP32 but for its centre, converted once a block.)
+// The camera in FP32 but for its centre.
 struct CameraF {
     double cx, cy;
     float R[9], fx, fy;
@@ -149,20 +149,24 @@ __global__ void k_project_backward_batch(const mer_camera* __restrict__ cams, co
                                          int n_items, long long vrecs, const mer_vertex* __restrict__ vpix,
                                          const double* __restrict__ grad_vpix, float* __restrict__ grad_verts) {
     after_previous();
-    __shared__ CameraF s_cam;  // of the block's first item
-    __shared__ int s_item;
+    __shared__ CameraF s_cam[8];  // of each warp's first item, converted by its lanes together
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int k = block_find_item(items, n_items, (long long)blockIdx.x * blockDim.x, i, kFieldVrec);
-    if (threadIdx.x == 0) {
-        s_item = k;
-        s_cam = camera_f(cams[items[k].cam]);
-    }
-    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const int k = warp_find_item(items, n_items, i - lane, i, kFieldVrec);
+    const int first = __shfl_sync(0xffffffffu, k, 0);
+    CameraF& cam = s_cam[threadIdx.x >> 5];
+    const mer_camera& c = cams[items[first].cam];
+    if (lane < 9) cam.R[lane] = (float)c.R[lane];
+    if (lane == 9) cam.fx = (float)c.fx;
+    if (lane == 10) cam.fy = (float)c.fy;
+    if (lane == 11) cam.cx = c.cx;
+    if (lane == 12) cam.cy = c.cy;
+    __syncwarp();
     if (i >= vrecs) return;
     const mer_item m = items[k];
     float w[3];
-    if (!(k == s_item ? world_grad(vpix[i], s_cam, grad_vpix + 3 * i, w)
-                      : world_grad(vpix[i], camera_f(cams[m.cam]), grad_vpix + 3 * i, w)))
+    if (!(k == first ? world_grad(vpix[i], cam, grad_vpix + 3 * i, w)
+                     : world_grad(vpix[i], camera_f(cams[m.cam]), grad_vpix + 3 * i, w)))
         return;
     float* o = grad_verts + 3 * (size_t)(m.vert + (i - m.vrec));
     atomicAdd(o, w[0]);
@@ -179,7 +183,7 @@ __global__ void k_project_backward_batch_fixed(const mer_camera* __restrict__ ca
                                                void* ws) {
     after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int k = block_find_item(items, n_items, (long long)blockIdx.x * blockDim.x, i, kFieldVrec);
+    const int k = warp_find_item(items, n_items, i - (threadIdx.x & 31), i, kFieldVrec);
     if (i >= vrecs) return;
     const mer_item m = items[k];
     double w[3];

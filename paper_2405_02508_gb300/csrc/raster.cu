@@ -611,7 +611,7 @@ __global__ void k_setup_count_batch(const mer_vertex* __restrict__ vpix, const i
                                     TriRaster* __restrict__ recs, int* __restrict__ counts, void* ws) {
     after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int k = block_find_item(b.items, b.n_items, (long long)blockIdx.x * blockDim.x, i, kFieldTrec);
+    const int k = warp_find_item(b.items, b.n_items, i - (threadIdx.x & 31), i, kFieldTrec);
     if (i >= b.trecs) return;
     const mer_item m = b.items[k];
     setup_count_one(batch_item(m, b.tile, vpix, tris, recs), (int)(i - m.trec), b.tile, counts, ws);
@@ -623,7 +623,7 @@ __global__ void k_bin_fill_batch(const mer_vertex* __restrict__ vpix, const int*
                                  long long capacity) {
     after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int k = block_find_item(b.items, b.n_items, (long long)blockIdx.x * blockDim.x, i, kFieldTrec);
+    const int k = warp_find_item(b.items, b.n_items, i - (threadIdx.x & 31), i, kFieldTrec);
     if (i >= b.trecs) return;
     const mer_item m = b.items[k];
     fill_one(batch_item(m, b.tile, vpix, tris, recs), (int)(i - m.trec), b.tile, offs, counts, cursor,

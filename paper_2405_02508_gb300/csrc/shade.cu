@@ -46,7 +46,7 @@ __global__ void k_shade_batch(const mer_vertex* __restrict__ vpix, const int* __
                               const float* __restrict__ tex, ShadeArgs a, float* __restrict__ image, void* ws) {
     after_previous();
     const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int k = block_find_item(items, n_items, (long long)blockIdx.x * blockDim.x, p, kFieldPix);
+    const int k = warp_find_item(items, n_items, p - (threadIdx.x & 31), p, kFieldPix);
     if (p >= pixels) return;
     const mer_item m = items[k];
     const int rem = (int)(p - m.pix);
