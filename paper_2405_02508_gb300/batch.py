@@ -188,8 +188,8 @@ class PlainRenderer:
 
 
 def default_persistent_ctas() -> int:
-    """Persistent grid: the number of raster CTAs that fit on the device at once (4 per SM; the backward
-    scales it to its own 6 per SM)."""
+    """Persistent grid: four CTAs per SM (the library scales it to the five that its raster and its backward keep
+    resident)."""
     props = torch.cuda.get_device_properties(torch.cuda.current_device())
     return int(props.multi_processor_count) * 4
 

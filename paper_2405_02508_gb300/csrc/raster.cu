@@ -316,7 +316,10 @@ constexpr int kRasterThreads = 256;
 // smallest 15.8 / 88.3 / 2,120.
 constexpr int kTinyPx = 8;     // boxes of at most this many pixels: 2 lanes each
 constexpr int kSmallPx = 64;   // of at most this many: 8 lanes each; larger ones: a warp
-constexpr int kRasterCtasPerSm = 4;  // resident CTAs per SM (the 64 x 64 tile's shared memory allows four): 64 registers
+// Resident CTAs per SM: 48 registers a thread, and a stage of the 64 x 64 tile small enough that its shared memory allows
+// five.  32 head views (tile 64) 1,855 us with four and 64 registers, 1,780 with five; 48 uneven meshes (tile 32) 651 and 586,
+// 588 with six at 40 registers; 8 views at 512 x 512 (tile 32) 78, 75 and 84.
+constexpr int kRasterCtasPerSm = 5;
 
 // Per-pixel bits kept in shared memory for the cover image: a front-facing triangle covered the centre
 // (taken when the front part is done), two or more did, one / two or more back-facing ones did, and a
@@ -326,7 +329,7 @@ constexpr unsigned kCovF1 = 1, kCovF2 = 2, kCovB1 = 4, kCovB2 = 8, kCovWB = 16;
 
 template <int TS>
 struct RasterShared {
-    static constexpr int kStageTS = TS >= 64 ? 160 : kStage;  // keeps the 64 x 64 tile within 48 KB
+    static constexpr int kStageTS = TS >= 64 ? 96 : kStage;  // keeps the 64 x 64 tile within 44 KB
     TriRaster rec[kStageTS];
     int id[kStageTS];
     unsigned char todo[3][kStageTS];  // the stage's records by box size (tiny, small, large), less those that cannot win
@@ -894,7 +897,8 @@ static int batch_raster(const mer_vertex* vpix, const int* tris, const mer_item*
         launch_chained(k_bin_fill_batch, (unsigned)((trecs + 255) / 256), 256, s, vpix, tris, b, recs, offs, counts, cursor, list,
                                                                         capacity);
     if (tiles > 0) {
-        const unsigned grid = persistent_ctas > 0 ? (unsigned)persistent_ctas : 0u;
+        // persistent_ctas counts four CTAs an SM, of which five are resident
+        const unsigned grid = persistent_ctas > 0 ? (unsigned)((long long)persistent_ctas * kRasterCtasPerSm / 4) : 0u;
         ShadeOut none;
         none.attr = nullptr; none.tex = nullptr; none.image = nullptr; none.image2 = nullptr; none.index2 = nullptr;
         const ShadeOut& o = so ? *so : none;
