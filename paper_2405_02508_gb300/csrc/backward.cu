@@ -31,12 +31,11 @@ constexpr int kTW = kBwdTileW, kTH = kBwdTileH;  // tile: 8 warps, two rows each
 constexpr int kRows = 2;                          // rows per warp
 constexpr int kHW = kTW + 2, kHH = kTH + 2;
 constexpr int kThreads = 256;
-// Resident CTAs per SM.  The batched kernel works on whole batches and wants the warps (6: at most 42 registers a thread; 32
-// head views 2,381 us with 6, 2,386 with 5, 2,506 with 4; 48 uneven meshes 640, 658, 723); a per-view launch is a few
-// thousand tiles, whose chains gain from the registers (3 views at 333 x 517: 19.6 us with 6, 17.5 with 5; 1024 x 1024 with
-// attribute gradients: 52.4 and 48.3, with 4 16.5 and 48.9).
-constexpr int kCtasPerSm = 6;
-constexpr int kViewCtasPerSm = 5;
+// Resident CTAs per SM, at most 51 registers a thread.  32 head views 2,354 us with six (42 registers) and 2,320 with five,
+// 2,410 with four, once the tile's place and item were kept in shared memory; 8 views at 512 x 512 75.4, 71.9 and 72.2; 48
+// uneven meshes with attribute gradients 638, 637 and 688.  A per-view launch (three views at 333 x 517) 19.6, 17.5 and 16.5;
+// 1024 x 1024 with attribute gradients 52.4, 48.3 and 48.9.
+constexpr int kCtasPerSm = 5;
 static_assert(kTW == 32 && kTH == kRows * kThreads / 32, "a warp spans the tile's width");
 // Per-tile triangle table of 2^BITS slots: a 32x16 tile of the head-scale workloads holds ~20-80 triangles.
 // 128 slots keep six CTAs resident with most of the SM's on-chip memory left to the L1 cache that serves the
@@ -377,35 +376,50 @@ __device__ __forceinline__ void table_clear(BwdShared<NA, EXACT, BITS>& S) {
     }
 }
 
-// Returns whether this thread loaded a covered pixel of the tile itself (not the halo).  Each thread issues
-// all its loads (at most three entries and their cover bytes) before it stores any.
+// Returns whether this thread loaded a covered pixel of the tile itself (not the halo).  A warp takes whole rows (two or
+// three of the 18, lane = column), and the last two warps, which have two, also the halo columns; each thread issues all its
+// loads before it stores any.
 template <int NA, bool EXACT, int BITS>
 __device__ __forceinline__ bool tile_halo(const BItem& it, const BwdArgs& a, int tx, int ty,
                                           BwdShared<NA, EXACT, BITS>& S) {
-    constexpr int kN = (kHH * kHW + kThreads - 1) / kThreads;
-    int v[kN];
-    unsigned char c[kN];
+    constexpr int kWarps = kThreads / 32, kN = (kHH + kWarps - 1) / kWarps;
+    static_assert(kHH <= 3 * kWarps && 2 * kHH <= 64, "rows and halo columns over the warps");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int W = it.W, H = it.H;
     const int* ib = it.index(a);
     const unsigned char* cb = a.cover ? it.cover(a) : nullptr;
+    int v[kN + 1];
+    unsigned char c[kN + 1];
+    const int x = tx * kTW + lane, y0 = ty * kTH - 1;
 #pragma unroll
     for (int q = 0; q < kN; ++q) {
-        const int i = threadIdx.x + q * kThreads;
-        const int hy = i / kHW, hx = i % kHW;
-        const int gx = tx * kTW + hx - 1, gy = ty * kTH + hy - 1;
-        const bool in = i < kHH * kHW && gx >= 0 && gx < it.W && gy >= 0 && gy < it.H;
-        const size_t o = in ? (size_t)gy * it.W + gx : 0;
+        const int h = warp + q * kWarps, y = y0 + h;
+        const bool in = h < kHH && y >= 0 && y < H && x < W;
+        const int o = in ? y * W + x : 0;
         v[q] = in ? __ldg(ib + o) : -2;
-        c[q] = (in && cb) ? __ldg(cb + o) : (unsigned char)0;
+        c[q] = in && cb ? __ldg(cb + o) : (unsigned char)0;
+    }
+    const int e = (int)threadIdx.x - (kThreads - 64);  // halo entry: row e / 2, left or right
+    const bool side = e >= 0 && e < 2 * kHH;
+    if (side) {
+        const int hx = tx * kTW + (e & 1 ? kTW : -1), hy = y0 + (e >> 1);
+        const bool in = hx >= 0 && hx < W && hy >= 0 && hy < H;
+        const int o = in ? hy * W + hx : 0;
+        v[kN] = in ? __ldg(ib + o) : -2;
+        c[kN] = in && cb ? __ldg(cb + o) : (unsigned char)0;
     }
     bool covered = false;
 #pragma unroll
     for (int q = 0; q < kN; ++q) {
-        const int i = threadIdx.x + q * kThreads;
-        if (i >= kHH * kHW) break;
-        const int hy = i / kHW, hx = i % kHW;
-        S.sidx[hy][hx] = v[q];
-        if (cb) S.scov[hy][hx] = c[q];
-        covered |= v[q] >= 0 && hy >= 1 && hy <= kTH && hx >= 1 && hx <= kTW;
+        const int h = warp + q * kWarps;
+        if (h >= kHH) break;
+        S.sidx[h][lane + 1] = v[q];
+        if (cb) S.scov[h][lane + 1] = c[q];
+        covered |= v[q] >= 0 && h >= 1 && h <= kTH;
+    }
+    if (side) {
+        S.sidx[e >> 1][e & 1 ? kTW + 1 : 0] = v[kN];
+        if (cb) S.scov[e >> 1][e & 1 ? kTW + 1 : 0] = c[kN];
     }
     return covered;
 }
@@ -692,7 +706,7 @@ __device__ __forceinline__ void tile_flush(const BItem& it, const BwdArgs& a, Bw
 }
 
 template <int FORM, int NA, bool EXACT, int BITS>
-__global__ void __launch_bounds__(kThreads, kViewCtasPerSm) k_backward(const mer_vertex* __restrict__ vpix, const int* __restrict__ tris,
+__global__ void __launch_bounds__(kThreads, kCtasPerSm) k_backward(const mer_vertex* __restrict__ vpix, const int* __restrict__ tris,
                                                        const int* __restrict__ index,
                                                        const unsigned char* __restrict__ cover,
                                                        const float* __restrict__ image,
@@ -720,6 +734,46 @@ __global__ void __launch_bounds__(kThreads, kViewCtasPerSm) k_backward(const mer
     tile_flush(it, a, S);
 }
 
+// A tile of the work queue: its item and place, found by the thread that takes it and read by all from shared memory (each
+// warp searching the table and dividing for itself was a twentieth of the instructions, and the item's offsets took a
+// quarter of its registers).
+struct TileJob {
+    BItem it;
+    int tx, ty;
+    int end;     // 1: no tile left
+    int item;    // its place in the table
+    long long lo, hi;  // and its tile range
+};
+
+// One thread: the next tile, after the job `last` of the same CTA (consecutive tiles mostly belong to the same item).
+__device__ __forceinline__ void take_tile(WsHeader* hdr, const mer_item* __restrict__ items, int n_items, long long btiles,
+                                          const TileJob& last, TileJob& job) {
+    const long long g = (long long)atomicAdd(&hdr->queue_backward, 1ull);
+    job.end = g >= btiles;
+    if (job.end) return;
+    int k = last.item;
+    long long lo = last.lo, hi = last.hi;
+    const bool same = g >= lo && g < hi;
+    if (!same) k = find_item(items, n_items, g, kFieldBtile);
+    const mer_item m = items[k];
+    const int ntx = (m.W + kTW - 1) / kTW;
+    if (!same) {
+        lo = m.btile;
+        hi = lo + (long long)ntx * ((m.H + kTH - 1) / kTH);
+    }
+    job.item = k;
+    job.lo = lo;
+    job.hi = hi;
+    const int local = (int)(g - lo);
+    job.ty = local / ntx;
+    job.tx = local - job.ty * ntx;
+    job.it.vrec = m.vrec;
+    job.it.tri = m.tri;
+    job.it.pix = m.pix;
+    job.it.vert = m.vert;
+    job.it.V = m.V; job.it.T = m.T; job.it.H = m.H; job.it.W = m.W;
+}
+
 // Persistent: each CTA takes the next backward tile of any item from the work queue.
 template <int FORM, int NA, bool EXACT, int BITS>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_backward_batch(const mer_vertex* __restrict__ vpix,
@@ -735,43 +789,29 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_backward_batch(const m
                                                              float* __restrict__ grad_attr, void* ws) {
     after_previous();
     __shared__ BwdShared<NA, EXACT, BITS> S;
-    __shared__ long long s_tile;
+    __shared__ TileJob s_job[2];
     WsHeader* hdr = reinterpret_cast<WsHeader*>(ws);
     table_clear(S);
-    if (threadIdx.x == 0) s_tile = (long long)atomicAdd(&hdr->queue_backward, 1ull);
+    if (threadIdx.x == 0) {
+        s_job[1].lo = s_job[1].hi = 0;
+        s_job[1].item = 0;
+        take_tile(hdr, items, n_items, btiles, s_job[1], s_job[0]);
+    }
     __syncthreads();
-    // Per tile two barriers: after the halo load (thread 0 then takes the next tile id) and before the flush
-    // (the next id is visible after it).  The flush of a tile and the halo load of the next touch disjoint
-    // shared memory, and the next tile's table inserts come only after its first barrier.  (A background row
-    // leaves tile_compute at once; skipping whole background tiles here instead costs registers.)
-    int cur = 0;                       // item of the previous tile and its tile range [lo, hi)
-    long long lo = 0, hi = 0;
-    while (true) {
-        const long long g = s_tile;
-        if (g >= btiles) break;
-        // consecutive tiles of a CTA mostly belong to the same item: search the table only on a change
-        if (!(g >= lo && g < hi)) {
-            cur = find_item(items, n_items, g, kFieldBtile);
-            const mer_item c = items[cur];
-            lo = c.btile;
-            hi = lo + (long long)((c.W + kTW - 1) / kTW) * ((c.H + kTH - 1) / kTH);
-        }
-        const mer_item m = items[cur];
-        const int ntx = (m.W + kTW - 1) / kTW;
-        const int local = (int)(g - m.btile);
-        BItem it;
-        it.vrec = m.vrec;
-        it.tri = m.tri;
-        it.pix = m.pix;
-        it.vert = m.vert;
-        it.V = m.V; it.T = m.T; it.H = m.H; it.W = m.W;
-        const int tx = local % ntx, ty = local / ntx;
-        tile_halo(it, a, tx, ty, S);
+    // Per tile two barriers: after the halo load (thread 0 then takes the next tile, into the job that the tile before this
+    // one no longer needs) and before the flush (the next job is visible after it).  The flush of a tile and the halo load
+    // of the next touch disjoint shared memory, and the next tile's table inserts come only after its first barrier.  (A
+    // background row leaves tile_compute at once; skipping whole background tiles here instead costs registers.)
+    for (int b = 0;; b ^= 1) {
+        const TileJob& job = s_job[b];
+        if (job.end) break;
+        const int tx = job.tx, ty = job.ty;
+        tile_halo(job.it, a, tx, ty, S);
         __syncthreads();
-        if (threadIdx.x == 0) s_tile = (long long)atomicAdd(&hdr->queue_backward, 1ull);
-        tile_compute<FORM, NA, EXACT, BITS>(it, tx, ty, a, tex, S, ws);
+        if (threadIdx.x == 0) take_tile(hdr, items, n_items, btiles, job, s_job[b ^ 1]);
+        tile_compute<FORM, NA, EXACT, BITS>(job.it, tx, ty, a, tex, S, ws);
         __syncthreads();
-        tile_flush(it, a, S);
+        tile_flush(job.it, a, S);
     }
 }
 
@@ -839,7 +879,7 @@ extern "C" int mer_launch_backward_batch(const mer_vertex* vpix, const int* tris
     a.tex_vec4 = a.tex_stride == 4 && tex && (reinterpret_cast<uintptr_t>(tex) & 15u) == 0;
     WsHeader* hdr = reinterpret_cast<WsHeader*>(ws);
     if (cudaMemsetAsync(&hdr->queue_backward, 0, sizeof(unsigned long long), s) != cudaSuccess) return 2;
-    // persistent_ctas sizes the raster's grid (4 resident CTAs per SM); the backward keeps as many waves.
+    // persistent_ctas counts four CTAs per SM; the backward keeps as many waves.
     // Without it, the grid is the device's SM count times the resident CTAs of the instantiation launched.
     const unsigned fixed_grid = persistent_ctas > 0 ? (unsigned)((long long)persistent_ctas * kCtasPerSm / 4) : 0u;
     unsigned grid = fixed_grid;
