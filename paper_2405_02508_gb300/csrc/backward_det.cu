@@ -114,11 +114,14 @@ __device__ __forceinline__ bool ids_of(const int* __restrict__ tris, int t, int 
     return true;
 }
 
+// ATTR: with attribute gradients, whose sums are carried in registers (without them a pass over 512 x 512 pixels of 40,960
+// triangles took 88.7 us with the idle sums and 77.0 without; 80 registers and three CTAs per SM: 89.3).
 // The contributions of pixel (x, y) of an item: returns its triangle (or -1) with its vertex ids and the
 // fixed-point contributions cv[k][c] to vertex k's gradient component c and ca[k][j] to its attribute
 // gradient channel j.
+template <bool ATTR>
 __device__ int det_pixel(const DetItem& it, const DetArgs& a, const float* __restrict__ tex, int x, int y, void* ws,
-                         int vid[3], Fix cv[3][3], Fix ca[3][kDetMaxA]) {
+                         int vid[3], Fix cv[3][3], Fix ca[3][ATTR ? kDetMaxA : 1]) {
     const size_t p = (size_t)y * it.W + x;
     int t = __ldg(it.index + p);
     if (t < 0) return -1;
@@ -133,11 +136,12 @@ __device__ int det_pixel(const DetItem& it, const DetArgs& a, const float* __res
     double f[3] = {0.0, 0.0, 0.0};             // fragment gradient dL/dr (x_s, y_s, zeta)
     double hz[3] = {0.0, 0.0, 0.0};            // interior zeta derivative of vertex k over lambda_k
     double ev[3][2] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};  // exact-crossing parts per vertex (x, y)
-    double cat[3][kDetMaxA];
+    constexpr int kA = ATTR ? kDetMaxA : 1;
+    double cat[3][kA];
 #pragma unroll
     for (int k = 0; k < 3; ++k)
 #pragma unroll
-        for (int j = 0; j < kDetMaxA; ++j) cat[k][j] = 0.0;
+        for (int j = 0; j < kA; ++j) cat[k][j] = 0.0;
 
     if (a.terms & MER_INTERIOR) {
         const double z[3] = {zeta_f64(rv[0]), zeta_f64(rv[1]), zeta_f64(rv[2])};
@@ -158,9 +162,13 @@ __device__ int det_pixel(const DetItem& it, const DetArgs& a, const float* __res
                 D01 += gc * (a0 - a1);
                 D02 += gc * (a0 - a2);
                 D12 += gc * (a1 - a2);
-                if (c < a.A && c < kDetMaxA) {
+                if (ATTR && c < a.A) {
 #pragma unroll
-                    for (int k = 0; k < 3; ++k) cat[k][c] = b[k] * gc;
+                    for (int j = 0; j < kA; ++j)
+                        if (j == c) {
+#pragma unroll
+                            for (int k = 0; k < 3; ++k) cat[k][j] = b[k] * gc;
+                        }
                 }
             }
         } else {
@@ -179,11 +187,11 @@ __device__ int det_pixel(const DetItem& it, const DetArgs& a, const float* __res
             D01 = gu * (u0 - u1) + gv * (v0 - v1);
             D02 = gu * (u0 - u2) + gv * (v0 - v2);
             D12 = gu * (u1 - u2) + gv * (v1 - v2);
-            if (a.A >= 2) {
+            if (ATTR && a.A >= 2) {
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
                     cat[k][0] = b[k] * gu;
-                    cat[k][1] = b[k] * gv;
+                    cat[k][ATTR ? 1 : 0] = b[k] * gv;
                 }
             }
         }
@@ -288,10 +296,10 @@ __device__ int det_pixel(const DetItem& it, const DetArgs& a, const float* __res
         cv[k][1] = to_fixed(l * f[1] + ev[k][1], ws);
         cv[k][2] = to_fixed(l * (f[2] + hz[k]), ws);
 #pragma unroll
-        for (int j = 0; j < kDetMaxA; ++j) {
+        for (int j = 0; j < kA; ++j) {
             ca[k][j].hi = 0;
             ca[k][j].lo = 0;
-            if (j < a.A) ca[k][j] = to_fixed(cat[k][j], ws);
+            if (ATTR && j < a.A) ca[k][j] = to_fixed(cat[k][j], ws);
         }
     }
     return t;
@@ -315,15 +323,16 @@ __device__ __forceinline__ void atomic_fix(unsigned long long* p, const Fix& v) 
 // Adds the contributions of a warp's pixels: runs of lanes with the same (item, triangle) are summed by a
 // segmented scan (exact integer sums) and each run's last lane adds the totals to the accumulators (two
 // 64-bit words per component: the high and low parts).
+template <bool ATTR>
 __device__ __forceinline__ void det_warp_add(const DetItem& it, const DetArgs& a, int key_item, int t,
-                                             const int vid[3], Fix cv[3][3], Fix ca[3][kDetMaxA]) {
+                                             const int vid[3], Fix cv[3][3], Fix ca[3][ATTR ? kDetMaxA : 1]) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int tprev = __shfl_up_sync(full, t, 1), iprev = __shfl_up_sync(full, key_item, 1);
     const bool head = lane == 0 || tprev != t || iprev != key_item;
     const unsigned heads = __ballot_sync(full, head);
     const int seg = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
-    const bool with_attr = a.A > 0 && it.acc_a != nullptr;
+    const bool with_attr = ATTR && it.acc_a != nullptr;
 #pragma unroll
     for (int dlt = 1; dlt < 32; dlt <<= 1) {
         const bool take = lane - dlt >= seg;
@@ -333,7 +342,7 @@ __device__ __forceinline__ void det_warp_add(const DetItem& it, const DetArgs& a
             for (int c = 0; c < 3; ++c) shfl_up_add(cv[k][c], dlt, take);
             if (with_attr) {
 #pragma unroll
-                for (int j = 0; j < kDetMaxA; ++j) shfl_up_add(ca[k][j], dlt, take);
+                for (int j = 0; j < (ATTR ? kDetMaxA : 1); ++j) shfl_up_add(ca[k][j], dlt, take);
             }
         }
     }
@@ -345,12 +354,15 @@ __device__ __forceinline__ void det_warp_add(const DetItem& it, const DetArgs& a
 #pragma unroll
         for (int c = 0; c < 3; ++c) atomic_fix(it.acc_v + 2 * (3 * (size_t)vid[k] + c), cv[k][c]);
         if (with_attr) {
-            for (int j = 0; j < a.A; ++j) atomic_fix(it.acc_a + 2 * ((size_t)vid[k] * a.A + j), ca[k][j]);
+#pragma unroll
+            for (int j = 0; j < (ATTR ? kDetMaxA : 1); ++j)
+                if (j < a.A) atomic_fix(it.acc_a + 2 * ((size_t)vid[k] * a.A + j), ca[k][j]);
         }
     }
 }
 
 // Per-view launch: n views of one mesh, pixels of all views in order.
+template <bool ATTR>
 __global__ void __launch_bounds__(kDetThreads) k_backward_det(const mer_vertex* __restrict__ vpix,
                                                               const int* __restrict__ tris, const int* __restrict__ index,
                                                               const float* __restrict__ image,
@@ -377,12 +389,13 @@ __global__ void __launch_bounds__(kDetThreads) k_backward_det(const mer_vertex* 
     it.V = V; it.T = T; it.H = H; it.W = W;
     int vid[3] = {0, 0, 0};
     Fix cv[3][3] = {};
-    Fix ca[3][kDetMaxA] = {};
-    const int t = live ? det_pixel(it, a, tex, rem % W, rem / W, ws, vid, cv, ca) : -1;
-    det_warp_add(it, a, view, t, vid, cv, ca);
+    Fix ca[3][ATTR ? kDetMaxA : 1] = {};
+    const int t = live ? det_pixel<ATTR>(it, a, tex, rem % W, rem / W, ws, vid, cv, ca) : -1;
+    det_warp_add<ATTR>(it, a, view, t, vid, cv, ca);
 }
 
 // Batched launch: the pixels of all items in order (item.pix).
+template <bool ATTR>
 __global__ void __launch_bounds__(kDetThreads) k_backward_det_batch(const mer_vertex* __restrict__ vpix,
                                                                     const int* __restrict__ tris,
                                                                     const mer_item* __restrict__ items, int n_items,
@@ -411,13 +424,13 @@ __global__ void __launch_bounds__(kDetThreads) k_backward_det_batch(const mer_ve
     it.V = m.V; it.T = m.T; it.H = m.H; it.W = m.W;
     int vid[3] = {0, 0, 0};
     Fix cv[3][3] = {};
-    Fix ca[3][kDetMaxA] = {};
+    Fix ca[3][ATTR ? kDetMaxA : 1] = {};
     int t = -1;
     if (live && m.W > 0) {
         const int rem = (int)(g - m.pix);
-        t = det_pixel(it, a, tex, rem % m.W, rem / m.W, ws, vid, cv, ca);
+        t = det_pixel<ATTR>(it, a, tex, rem % m.W, rem / m.W, ws, vid, cv, ca);
     }
-    det_warp_add(it, a, k, t, vid, cv, ca);
+    det_warp_add<ATTR>(it, a, k, t, vid, cv, ca);
 }
 
 // grad_vpix += the accumulated sums (FP64); grad_attr[:, a0 + j] += those of acc_a (rounded to FP32).
@@ -484,7 +497,9 @@ extern "C" int mer_launch_backward_det(const mer_vertex* vpix, int V, const int*
     if (bytes > 0 && cudaMemsetAsync(acc_v, 0, bytes, s) != cudaSuccess) return 2;
     const long long npix = (long long)n * H * W;
     if (npix > 0)
-        launch_chained(k_backward_det, (unsigned)((npix + kDetThreads - 1) / kDetThreads), kDetThreads, s, 
+        a.A > 0 ? launch_chained(k_backward_det<true>, (unsigned)((npix + kDetThreads - 1) / kDetThreads), kDetThreads, s, 
+            vpix, tris, index, image, grad_image, attr, tex, a, n, H, W, V, T, acc_v, acc_a, ws)
+                : launch_chained(k_backward_det<false>, (unsigned)((npix + kDetThreads - 1) / kDetThreads), kDetThreads, s, 
             vpix, tris, index, image, grad_image, attr, tex, a, n, H, W, V, T, acc_v, acc_a, ws);
     if (cudaGetLastError() != cudaSuccess) return 2;
     return det_finish(acc_v, vrows, grad_vpix, acc_a, V, a, grad_attr, s);
@@ -504,7 +519,9 @@ extern "C" int mer_launch_backward_det_batch(const mer_vertex* vpix, const int* 
     const size_t bytes = mer_det_workspace_size(vrecs, grad_attr ? mesh_rows : 0, a.A) - 256;
     if (bytes > 0 && cudaMemsetAsync(acc_v, 0, bytes, s) != cudaSuccess) return 2;
     if (pixels > 0)
-        launch_chained(k_backward_det_batch, (unsigned)((pixels + kDetThreads - 1) / kDetThreads), kDetThreads, s, 
+        a.A > 0 ? launch_chained(k_backward_det_batch<true>, (unsigned)((pixels + kDetThreads - 1) / kDetThreads), kDetThreads, s, 
+            vpix, tris, items, n_items, pixels, index, image, grad_image, attr, tex, a, acc_v, acc_a, ws)
+                : launch_chained(k_backward_det_batch<false>, (unsigned)((pixels + kDetThreads - 1) / kDetThreads), kDetThreads, s, 
             vpix, tris, items, n_items, pixels, index, image, grad_image, attr, tex, a, acc_v, acc_a, ws);
     if (cudaGetLastError() != cudaSuccess) return 2;
     return det_finish(acc_v, vrecs, grad_vpix, acc_a, mesh_rows, a, grad_attr, s);
