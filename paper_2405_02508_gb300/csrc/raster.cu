@@ -321,8 +321,9 @@ constexpr int kSmallPx = 64;   // of at most this many: 8 lanes each; larger one
 // 588 with six at 40 registers; 8 views at 512 x 512 (tile 32) 78, 75 and 84.
 constexpr int kRasterCtasPerSm = 5;
 
-// Per-pixel bits kept in shared memory for the cover image: a front-facing triangle covered the centre
-// (taken when the front part is done), two or more did, one / two or more back-facing ones did, and a
+// Per-pixel bits kept in shared memory for the cover image: a front-facing triangle covered the centre of a pixel that a
+// back-facing one won (noted when a back-facing fragment takes the pixel from a front-facing one), two or more
+// front-facing ones covered it, one / two or more back-facing ones did, and a
 // back-facing fragment raised the depth buffer (the winner is then back-facing: the front part is drawn
 // first, so every later raise comes from a back-facing fragment).
 constexpr unsigned kCovF1 = 1, kCovF2 = 2, kCovB1 = 4, kCovB2 = 8, kCovWB = 16;
@@ -341,16 +342,14 @@ struct RasterShared {
 
 // Smallest depth key (zeta_test) over the tile's pixels inside the image, 0 if one of them is still empty.
 // All threads call it; it starts and ends with a barrier.
-// With `cover`, also records which pixels a front-facing triangle covers (kCovF1).
 template <int TS>
-__device__ __forceinline__ float tile_min_zeta(RasterShared<TS>& S, int ox, int oy, int W, int H, bool cover) {
+__device__ __forceinline__ float tile_min_zeta(RasterShared<TS>& S, int ox, int oy, int W, int H) {
     __syncthreads();
     float mn = 3.0e38f;
     for (int i = threadIdx.x; i < TS * TS; i += kRasterThreads) {
         const int px = ox + (i % TS), py = oy + (i / TS);
         if (px >= W || py >= H) continue;
         const unsigned long long key = S.zbuf[i];
-        if (cover && key) atomicOr(&S.cov[i >> 2], kCovF1 << ((i & 3) * 8));
         mn = fminf(mn, key ? __uint_as_float((unsigned)(key >> 32)) : 0.0f);
     }
 #pragma unroll
@@ -364,9 +363,10 @@ __device__ __forceinline__ float tile_min_zeta(RasterShared<TS>& S, int ox, int 
     return r;
 }
 
-// Draws the n records S.todo[CLASS] of the stage into the z-buffer, G lanes a triangle.
+// Draws the n records S.todo[CLASS] of the stage into the z-buffer, G lanes a triangle; recs: the item's records.
 template <int TS, int CLASS, int G>
-__device__ __forceinline__ void raster_class(RasterShared<TS>& S, int n, int ox, int oy, bool back, bool cover) {
+__device__ __forceinline__ void raster_class(RasterShared<TS>& S, const TriRaster* __restrict__ recs, int n, int ox, int oy, bool back,
+                                             bool cover) {
     const int lane = threadIdx.x % G;
     for (int k = threadIdx.x / G; k < n; k += kRasterThreads / G) {
         const int j = S.todo[CLASS][k];
@@ -410,7 +410,13 @@ __device__ __forceinline__ void raster_class(RasterShared<TS>& S, int n, int ox,
                 if (!back) {
                     if (old) atomicOr(&S.cov[pi >> 2], kCovF2 << sh);  // a front fragment came first
                 } else {
-                    if (key > old) atomicOr(&S.cov[pi >> 2], kCovWB << sh);
+                    if (key > old) {
+                        // whichever fragment takes the pixel first takes it from the front-facing winner, if there is one
+                        // (noting the front cover of every pixel beforehand was an atomic a pixel: raster of 32 head views
+                        // 1,780 us, 1,745 so; 48 uneven meshes 589 and 575)
+                        const bool front = old && (recs[0xFFFFFFFFu - (unsigned)old].flags & 8);
+                        atomicOr(&S.cov[pi >> 2], (kCovWB | (front ? kCovF1 : 0u)) << sh);
+                    }
                     const unsigned o = atomicOr(&S.cov[pi >> 2], kCovB1 << sh);
                     if (o & (kCovB1 << sh)) atomicOr(&S.cov[pi >> 2], kCovB2 << sh);
                 }
@@ -454,7 +460,7 @@ __device__ __forceinline__ void raster_tile(const RItem& it, int local_tile, con
         // stage boundaries fall on the front / back split so each stage is one part
         const int lim = base < nf ? nf : count;
         m = min(kSt, lim - base);
-        if (base == nf && base > 0) zcull = tile_min_zeta<TS>(S, ox, oy, it.W, it.H, cover != nullptr);
+        if (base == nf && base > 0) zcull = tile_min_zeta<TS>(S, ox, oy, it.W, it.H);
         const bool back = base >= nf;
         __syncthreads();
         int* n_todo = S.n_todo[stage & 1];
@@ -474,9 +480,9 @@ __device__ __forceinline__ void raster_tile(const RItem& it, int local_tile, con
             S.todo[c][atomicAdd(&n_todo[c], 1)] = (unsigned char)j;
         }
         __syncthreads();
-        raster_class<TS, 2, 32>(S, n_todo[2], ox, oy, back, cover != nullptr);
-        raster_class<TS, 1, 8>(S, n_todo[1], ox, oy, back, cover != nullptr);
-        raster_class<TS, 0, 2>(S, n_todo[0], ox, oy, back, cover != nullptr);
+        raster_class<TS, 2, 32>(S, it.recs, n_todo[2], ox, oy, back, cover != nullptr);
+        raster_class<TS, 1, 8>(S, it.recs, n_todo[1], ox, oy, back, cover != nullptr);
+        raster_class<TS, 0, 2>(S, it.recs, n_todo[0], ox, oy, back, cover != nullptr);
     }
     __syncthreads();
     for (int i = threadIdx.x; i < TS * TS; i += kRasterThreads) {
@@ -493,7 +499,7 @@ __device__ __forceinline__ void raster_tile(const RItem& it, int local_tile, con
                          (ly == 0 ? MER_COVER_BORDER_T : 0u) | (ly == TS - 1 ? MER_COVER_BORDER_B : 0u);
             if (t >= 0) {
                 const unsigned b = S.cov[i >> 2] >> ((i & 3) * 8);
-                if (b & kCovWB) {  // kCovF1 was taken before the back part (none if the tile has no front part)
+                if (b & kCovWB) {
                     c |= MER_COVER_WINNER_BACK | ((b & kCovB2) ? MER_COVER_SAME_2 : 0u) |
                          ((b & kCovF1) ? MER_COVER_OTHER_1 : 0u);
                 } else {
