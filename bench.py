@@ -127,7 +127,7 @@ def backward_sources_sha256() -> str:
     import hashlib
 
     h = hashlib.sha256()
-    for f in ("backward.cu", "mer_device.cuh"):
+    for f in ("backward.cu", "mer_device.cuh", "shade_device.cuh"):
         with open(os.path.join(ROOT, "paper_2405_02508_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()
@@ -682,7 +682,8 @@ def main():
     peak, peak_kind = peaks()
     bb = backward_bytes_per_launch(n, H, W, C, V)
     achieved = bb / (kms["bwd"] * 1e-3) / 1e9
-    launches_per_step = 9  # project 1, setup/count 1, scan 3, fill 1, raster+shade 1, backward 1, proj. backward 1
+    # project, setup/count, scan (one launch up to 16,384 bin tiles, three beyond), fill, raster+shade, backward, its projection
+    launches_per_step = 7 if br.tot.tiles <= 16384 else 9
     scaling = "strong" if split else "weak"
     parallelism = (f"views split x{world}, vertex gradient summed over the ranks (all-reduce) each step" if split
                    else f"replicas x{world}")
@@ -703,7 +704,7 @@ def main():
                        "backward": kms["bwd"]},
         "step_algorithmic_gbs": step_bytes(n, H, W, C, V, T, tex.numel() * 4) / (ms * 1e-3) / 1e9,
         "plain": None if plain_ms is None else {"value": px_step / (plain_ms * 1e-3) / 1e6, "unit": "Mpix/s",
-                                                "ms_per_step": plain_ms, "launches_per_step": 10 * n},
+                                                "ms_per_step": plain_ms, "launches_per_step": 8 * n},
         "e2e": {"value": px_step / (e2e_ms * 1e-3) / 1e6, "unit": "Mpix/s", "h2d_bytes_per_step": V * 12,
                 "d2h_bytes_per_step": V * 12, "ms_per_step": e2e_ms},
         "gpu_launches": launches_per_step * args.steps,

@@ -154,8 +154,15 @@ def _ptr(t: torch.Tensor | None):
     return t.data_ptr()
 
 
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream():
-    return torch.cuda.current_stream().cuda_stream
+    """The current stream's handle (without the Stream object, which takes longer to make than a kernel to launch:
+    2.9 us a call, 0.4 so)."""
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
 
 
 def _nbytes(t: torch.Tensor | None) -> int:
