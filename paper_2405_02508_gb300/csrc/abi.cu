@@ -271,8 +271,12 @@ static int wait_words(int64_t* host, cudaStream_t s) {
     const int64_t ready = (int64_t)1 << 32;
     for (unsigned k = 1;; ++k) {
         if (__atomic_load_n(host, __ATOMIC_ACQUIRE) >= ready) return MER_OK;
-        if (k % 4096 == 0) {
+        if (k % 65536 == 0) {
+            // relaxed: another thread's capture must not be broken by the question
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+            if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return MER_ECUDA;
             const cudaError_t e = cudaStreamQuery(s);
+            if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return MER_ECUDA;
             if (e == cudaErrorNotReady) {
                 (void)cudaGetLastError();  // not an error
                 continue;

@@ -114,7 +114,7 @@ __device__ __forceinline__ bool covers_centre(const mer_vertex* __restrict__ vb,
     return covers_xy(X, Y, 256 * x + 128, 256 * y + 128);
 }
 
-constexpr int kNoRate = 0x7fffffff;  // bits of a NaN that no rate has (arithmetic gives 0x7fffffff only as itself negated)
+constexpr int kNoRate = (int)0xffc0deadu;  // no rate: bits that arithmetic does not give (its NaN is 0x7fffffff)
 
 // FORM: the layout of the main channels (ShadeForm); the fixed ones hold at most kFastC channels.
 constexpr int kFastC = 8;

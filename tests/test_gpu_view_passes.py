@@ -167,3 +167,13 @@ def test_passes_back_to_back():
     for k, out in enumerate(got):
         for a, b in zip(out, alone[k % 2]):
             assert torch.equal(a, b)
+
+
+def test_forward_grad_keeps_nan():
+    """A tangent that is not a number reaches every pixel whose pairs it moves."""
+    r, verts, cams, attr, tex = _setup("rgb", 90, 110, 1)
+    r.forward(verts, cams, attr, tex)
+    t = torch.randn(verts.shape, generator=torch.Generator(device="cuda").manual_seed(4), device="cuda")
+    moved = r.forward_grad(t, cams, attr, tex, terms=B.MER_EDGE) != 0
+    assert moved.any()
+    assert torch.isnan(r.forward_grad(torch.full_like(t, float("nan")), cams, attr, tex, terms=B.MER_EDGE))[moved].all()
