@@ -118,9 +118,9 @@ class ClockSampler:
 # one k_backward_batch launch, from an ncu capture of the same workload at 4 views (inputs already larger than
 # L2), per pixel of the launch, with the sha256 of the kernel's sources they were taken on: a launch of n views
 # moves / issues n*H*W times these.  They are reported only while the sources are unchanged.
-BACKWARD_TRAFFIC = {"bytes_per_pixel": 24.4699, "warp_instructions_per_pixel": 31.0864,
-                    "sources_sha256": "6c09ff0940653e50a07548f9ec794d428185f7d555c26de972205dd402d7dd76",
-                    "profile": "profiles/ncu_k_backward_batch_head_4x1334x2048.md"}
+BACKWARD_TRAFFIC = {"bytes_per_pixel": 23.7104, "warp_instructions_per_pixel": 22.9500,
+                    "sources_sha256": "8d555ee5f28b14e4a4819876b9f0754fc3b945b1c685974725f0505e4b70e9ca",
+                    "profile": "profiles/ncu_head_4x1334x2048.md"}
 
 
 def backward_sources_sha256() -> str:
