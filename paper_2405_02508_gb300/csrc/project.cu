@@ -262,7 +262,8 @@ extern "C" int mer_launch_project_screen(const double* scr, int V, int n, mer_ve
 extern "C" int mer_launch_project_backward(int V, const mer_camera* cams, int n, const mer_vertex* vpix,
                                            const double* grad_vpix, float* grad_verts, float* copy, int store,
                                            cudaStream_t s) {
-    if (V == 0 || n == 0) return 0;
+    // without views the kernel's sum over them is empty: an overwritten gradient is zero, a copy is what grad_verts holds
+    if (V == 0 || (n == 0 && !(grad_verts && (store || copy)))) return 0;
     if (store)
         launch_chained(k_project_backward<true>, (V + 255) / 256, 256, s, V, cams, n, vpix, grad_vpix, grad_verts, copy);
     else
