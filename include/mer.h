@@ -198,10 +198,14 @@ typedef struct mer_view {
  * host_status (or NULL): two int64 words of page-locked HOST memory that the device can write.  With it the call also
  * does mer_sync_status's part for the rasterization: it returns MER_EOVERFLOW / MER_ERANGE / MER_EFIXED (clearing the
  * status word) and sets *total_bins, after waiting only until the binning is done; the rest is still queued.  A
- * capturing stream cannot be waited for: MER_ECUDA. */
+ * capturing stream cannot be waited for: MER_ECUDA.  mer_view_render_cover: also a second copy of the cover image
+ * (cover_copy [n, H, W] or NULL; needs v->cover), for a backward pass that runs when the buffers hold something else. */
 int mer_view_render(const mer_view* v, const float* verts, const mer_camera* cams, const float* attr,
                     const float* tex, float* depth, float* bary, mer_vertex* vpix_copy, int32_t* index_copy,
                     float* image_copy, int64_t* host_status, int64_t* total_bins, void* stream);
+int mer_view_render_cover(const mer_view* v, const float* verts, const mer_camera* cams, const float* attr,
+                          const float* tex, float* depth, float* bary, mer_vertex* vpix_copy, int32_t* index_copy,
+                          float* image_copy, uint8_t* cover_copy, int64_t* host_status, int64_t* total_bins, void* stream);
 
 /* A whole backward pass from v's vpix, index, image and cover: mer_backward, then mer_project_backward.
  * zero: 0 all gradients are added to; 1 grad_vpix and grad_verts are overwritten; 2 grad_attr (if given) too.

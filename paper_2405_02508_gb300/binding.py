@@ -81,6 +81,8 @@ _SIGS = {
     "mer_l2_loss_grad": ([_P, _P, ctypes.c_int64, _P, _P, _P], _I),
     "mer_rasterize_world": ([_P, _I, _P, _I, _P, _I, _I, _I, _I, _P, _Z, _P, _P, _P, _P, _P], _I),
     "mer_view_render": ([ctypes.POINTER(MerView), _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, ctypes.POINTER(ctypes.c_int64), _P], _I),
+    "mer_view_render_cover": ([ctypes.POINTER(MerView), _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P,
+                               ctypes.POINTER(ctypes.c_int64), _P], _I),
     "mer_view_backward": ([ctypes.POINTER(MerView), _P, _P, _P, _P, _I, _P, _P, _P, _P, _I, _P], _I),
     "mer_view_forward_grad": ([ctypes.POINTER(MerView), _P, _P, _P, _P, _I, _P, _P, _P], _I),
     "mer_laplacian_csr": ([_P, ctypes.c_int64, ctypes.c_int64, _P, _P], _I),
@@ -312,12 +314,13 @@ def view_struct(tris, V, n, H, W, tile, workspace, vpix, index, cover, image, sh
 
 def mer_view_render(view: MerView, verts, cams, attr, tex, depth=None, bary=None, copies=(None, None, None),
                     host_status: torch.Tensor | None = None) -> tuple[int, int]:
-    """copies: (vpix, index, image) tensors that receive second copies; host_status: two int64 in pinned memory.
-    Returns (code, bin entries); the code is MER_OK, or the device status if host_status is given."""
+    """copies: (vpix, index, image) or (vpix, index, image, cover) tensors that receive second copies; host_status: two
+    int64 in pinned memory.  Returns (code, bin entries); the code is MER_OK, or the device status if host_status is given."""
     tot = ctypes.c_int64(0)
-    code = lib().mer_view_render(view, _ptr(verts), _ptr(cams), _ptr(attr), _ptr(tex), _ptr(depth), _ptr(bary),
-                                 _ptr(copies[0]), _ptr(copies[1]), _ptr(copies[2]),
-                                 None if host_status is None else host_status.data_ptr(), tot, _stream())
+    code = lib().mer_view_render_cover(view, _ptr(verts), _ptr(cams), _ptr(attr), _ptr(tex), _ptr(depth), _ptr(bary),
+                                       _ptr(copies[0]), _ptr(copies[1]), _ptr(copies[2]),
+                                       _ptr(copies[3]) if len(copies) > 3 else None,
+                                       None if host_status is None else host_status.data_ptr(), tot, _stream())
     if code in (MER_EINVAL, MER_ECUDA):
         raise MerError(code, "mer_view_render")
     return code, tot.value

@@ -13,7 +13,7 @@ extern "C" int mer_launch_project_backward(int, const mer_camera*, int, const me
                                            int, cudaStream_t);
 extern "C" int mer_launch_clear(double*, long long, float*, long long, cudaStream_t);
 extern "C" int mer_launch_view_render(const mer_view*, const float*, const mer_camera*, const float*, const float*, float*,
-                                      float*, mer_vertex*, int*, float*, long long*, cudaStream_t);
+                                      float*, mer_vertex*, int*, float*, unsigned char*, long long*, cudaStream_t);
 extern "C" size_t mer_raster_workspace_size(int, int, int, int, int, int, long long);
 extern "C" int mer_launch_rasterize(const mer_vertex*, int, const int*, int, int, int, int, int, void*, size_t, int*,
                                     float*, float*, unsigned char*, cudaStream_t);
@@ -295,11 +295,19 @@ static bool view_ok(const mer_view* v) {
 int mer_view_render(const mer_view* v, const float* verts, const mer_camera* cams, const float* attr, const float* tex,
                     float* depth, float* bary, mer_vertex* vpix_copy, int32_t* index_copy, float* image_copy,
                     int64_t* host_status, int64_t* total_bins, void* stream) {
+    return mer_view_render_cover(v, verts, cams, attr, tex, depth, bary, vpix_copy, index_copy, image_copy, nullptr,
+                                 host_status, total_bins, stream);
+}
+
+int mer_view_render_cover(const mer_view* v, const float* verts, const mer_camera* cams, const float* attr,
+                          const float* tex, float* depth, float* bary, mer_vertex* vpix_copy, int32_t* index_copy,
+                          float* image_copy, uint8_t* cover_copy, int64_t* host_status, int64_t* total_bins, void* stream) {
     if (!view_ok(v)) return MER_EINVAL;
     const long long px = (long long)v->n * v->H * v->W, rows = (long long)v->n * v->V;
     if (rows > 0 && (!verts || !cams || !v->vpix)) return MER_EINVAL;
     const bool copies = vpix_copy || index_copy || image_copy;
     if (copies && (!index_copy || !image_copy || (rows > 0 && !vpix_copy))) return MER_EINVAL;
+    if (cover_copy && (!copies || !v->cover)) return MER_EINVAL;
     if (px > 0) {
         if (!v->workspace || !aligned256(v->workspace) || !v->index || !v->image) return MER_EINVAL;
         if (v->T > 0 && (!v->tris || !v->vpix)) return MER_EINVAL;
@@ -326,13 +334,14 @@ int mer_view_render(const mer_view* v, const float* verts, const mer_camera* cam
             return MER_ECUDA;
         if (px > 0 &&
             (cudaMemcpyAsync(index_copy, v->index, px * sizeof(int), cudaMemcpyDeviceToDevice, s) != cudaSuccess ||
-             cudaMemcpyAsync(image_copy, v->image, px * v->sh->C * sizeof(float), cudaMemcpyDeviceToDevice, s) != cudaSuccess))
+             cudaMemcpyAsync(image_copy, v->image, px * v->sh->C * sizeof(float), cudaMemcpyDeviceToDevice, s) != cudaSuccess ||
+             (cover_copy && cudaMemcpyAsync(cover_copy, v->cover, px, cudaMemcpyDeviceToDevice, s) != cudaSuccess)))
             return MER_ECUDA;
         return MER_OK;
     }
     if (host_status) __atomic_store_n(host_status, (int64_t)0, __ATOMIC_RELEASE);
     const int rc = mer_launch_view_render(v, verts, cams, attr, tex, depth, bary, vpix_copy, index_copy, image_copy,
-                                          reinterpret_cast<long long*>(host_status), s);
+                                          cover_copy, reinterpret_cast<long long*>(host_status), s);
     if (rc != MER_OK || !host_status) return rc;
     if (wait_words(host_status, s) != MER_OK) return MER_ECUDA;
     if (total_bins) *total_bins = __atomic_load_n(host_status + 1, __ATOMIC_ACQUIRE);

@@ -40,6 +40,7 @@ struct ShadeOut {
     float* image;       // [pixels, C]
     float* image2;      // second copies of the image and the index, or null
     int* index2;
+    unsigned char* cover2;  // with them, of the cover image (or null)
 };
 
 __device__ __forceinline__ int floordiv256(int a) { return a >> 8; }  // arithmetic shift = floor
@@ -435,7 +436,7 @@ __device__ __forceinline__ void raster_class(RasterShared<TS>& S, const TriRaste
 // The tile's list holds the camera-facing triangles first (nfront of them) and the others after; before
 // the second part the tile's smallest depth key is taken, and a triangle of that part whose largest vertex
 // zeta (with a margin above the FP32 rounding of the key) is below it cannot win any pixel: it is skipped.
-// DUAL: the index image and the shaded image are also written to so.index2 and so.image2.
+// DUAL: the index image and the shaded image are also written to so.index2 and so.image2, the cover image to so.cover2.
 template <int TS, int FORM, bool DUAL = false>
 __device__ __forceinline__ void raster_tile(const RItem& it, int local_tile, const int* __restrict__ offs,
                                             const int* __restrict__ cnts, const int* __restrict__ nfront,
@@ -507,6 +508,7 @@ __device__ __forceinline__ void raster_tile(const RItem& it, int local_tile, con
                 }
             }
             cover[p] = (unsigned char)c;
+            if (DUAL && so.cover2) so.cover2[p] = (unsigned char)c;
         }
         if (FORM != kShadeOff)
             shade_fragment<FORM, false, DUAL>(it.vpix, it.V, it.tris, it.T, t, px, py,
@@ -781,7 +783,7 @@ static int view_raster(const mer_vertex* vpix, int V, const int* tris, int T, in
                                                                 capacity);
     const unsigned grid = (unsigned)L.ntiles;
     ShadeOut none;
-    none.attr = nullptr; none.tex = nullptr; none.image = nullptr; none.image2 = nullptr; none.index2 = nullptr;
+    none.attr = nullptr; none.tex = nullptr; none.image = nullptr; none.image2 = nullptr; none.index2 = nullptr; none.cover2 = nullptr;
     const ShadeOut& o = so ? *so : none;
     const int form = so ? shade_form(so->attr, so->tex, &so->a.sh) : kShadeOff;
     const bool dual = o.image2 != nullptr;
@@ -815,7 +817,7 @@ extern "C" int mer_launch_rasterize(const mer_vertex* vpix, int V, const int* tr
 // Projection, binning, raster and shading of n views (V, T, n, H, W > 0).
 extern "C" int mer_launch_view_render(const mer_view* v, const float* verts, const mer_camera* cams, const float* attr,
                                       const float* tex, float* depth, float* bary, mer_vertex* vpix2, int* index2,
-                                      float* image2, long long* host, cudaStream_t s) {
+                                      float* image2, unsigned char* cover2, long long* host, cudaStream_t s) {
     const RasterLayout L = raster_layout(v->V, v->T, v->n, v->H, v->W, v->tile, 1);
     int* counts = reinterpret_cast<int*>(static_cast<char*>(v->workspace) + L.counts);
     // the projection's threads clear the tile counts on the way unless there are many more of those
@@ -829,6 +831,7 @@ extern "C" int mer_launch_view_render(const mer_view* v, const float* verts, con
     so.image = v->image;
     so.image2 = image2;
     so.index2 = index2;
+    so.cover2 = cover2;
     const bool precise = v->sh->precise != 0;  // FP64 shading is a pass of its own, over the index image
     rc = view_raster(v->vpix, v->V, v->tris, v->T, v->n, v->H, v->W, v->tile, v->workspace, v->workspace_bytes, v->index,
                      depth, bary, v->cover, precise ? nullptr : &so, cleared, host, s);
@@ -838,7 +841,8 @@ extern "C" int mer_launch_view_render(const mer_view* v, const float* verts, con
     if (rc || !image2) return rc;
     const size_t px = (size_t)v->n * v->H * v->W;
     if (cudaMemcpyAsync(image2, v->image, px * v->sh->C * sizeof(float), cudaMemcpyDeviceToDevice, s) != cudaSuccess ||
-        cudaMemcpyAsync(index2, v->index, px * sizeof(int), cudaMemcpyDeviceToDevice, s) != cudaSuccess)
+        cudaMemcpyAsync(index2, v->index, px * sizeof(int), cudaMemcpyDeviceToDevice, s) != cudaSuccess ||
+        (cover2 && cudaMemcpyAsync(cover2, v->cover, px, cudaMemcpyDeviceToDevice, s) != cudaSuccess))
         return 2;
     return 0;
 }
@@ -906,7 +910,7 @@ static int batch_raster(const mer_vertex* vpix, const int* tris, const mer_item*
         // persistent_ctas counts four CTAs an SM, of which five are resident
         const unsigned grid = persistent_ctas > 0 ? (unsigned)((long long)persistent_ctas * kRasterCtasPerSm / 4) : 0u;
         ShadeOut none;
-        none.attr = nullptr; none.tex = nullptr; none.image = nullptr; none.image2 = nullptr; none.index2 = nullptr;
+        none.attr = nullptr; none.tex = nullptr; none.image = nullptr; none.image2 = nullptr; none.index2 = nullptr; none.cover2 = nullptr;
         const ShadeOut& o = so ? *so : none;
         int rc = 0;
 #define MER_RASTER(F) \
@@ -956,6 +960,7 @@ extern "C" int mer_launch_batch_render(const mer_vertex* vpix, const int* tris, 
     so.image = image;
     so.image2 = nullptr;
     so.index2 = nullptr;
+    so.cover2 = nullptr;
     return batch_raster(vpix, tris, items, n_items, trecs, tiles, tile, ws, ws_bytes, index, depth, bary, cover, &so,
                         persistent_ctas, s);
 }

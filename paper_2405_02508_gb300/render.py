@@ -56,6 +56,7 @@ class Renderer:
         self.grad_verts = torch.zeros((self.V, 3), dtype=torch.float32, device=device)
         self.terms = B.MER_EDGE | B.MER_INTERIOR | B.MER_INTERSECT
         self.renders = 0      # times the buffers were drawn to
+        self.replayed = False  # drawn to under capture: replays draw again without being counted
         self._status = None   # pinned words the device reports the binning's status in (made by the first checked pass)
         self._alloc_workspace(0)
 
@@ -70,15 +71,15 @@ class Renderer:
 
     # -- forward -----------------------------------------------------------------------------------
     def project(self, verts: torch.Tensor, cams: torch.Tensor):
-        self.renders += 1
+        self._drawing()
         B.mer_project(verts.contiguous(), cams, self.vpix)
 
     def project_screen(self, scr: torch.Tensor):
-        self.renders += 1
+        self._drawing()
         B.mer_project_screen(scr.contiguous(), self.vpix)
 
     def rasterize(self, depth: torch.Tensor | None = None, bary: torch.Tensor | None = None, checked: bool = True):
-        self.renders += 1
+        self._drawing()
         B.mer_rasterize(self.vpix, self.tris, self.H, self.W, self.tile, self.workspace, self.index, depth, bary,
                         self.cover)
         if checked:
@@ -92,9 +93,18 @@ class Renderer:
                 raise B.MerError(code, "mer_rasterize")
 
     def shade(self, attr: torch.Tensor, tex: torch.Tensor | None):
-        self.renders += 1
+        self._drawing()
         B.mer_shade(self.vpix, self.tris, self.index, attr.contiguous(), tex, self.bg, self.sh, self.image,
                     self.workspace)
+
+    def drawn(self) -> tuple:
+        """The buffers that a backward pass reads: vertex records, index, image and cover image (or None)."""
+        return self.vpix, self.index, self.image, self.cover
+
+    def _drawing(self):
+        self.renders += 1
+        if not self.replayed and torch.cuda.is_current_stream_capturing():
+            self.replayed = True
 
     def _view(self, bg=None) -> B.MerView:
         """The renderer's buffers for one call."""
@@ -102,13 +112,14 @@ class Renderer:
                              self.cover, self.image, self.sh, bg)
 
     def forward(self, verts, cams, attr, tex=None, depth=None, bary=None, checked=True, copies=None):
-        """copies (optional): (vpix, index, image) tensors that receive second copies of those buffers."""
+        """copies (optional): (vpix, index, image) or (vpix, index, image, cover) tensors that receive second copies of
+        those buffers."""
         if verts.shape[0] != self.V or cams.shape[0] != self.n:  # fewer vertices or cameras than the buffers hold
             self.project(verts, cams)
             self.rasterize(depth, bary, checked)
             self.shade(attr, tex)
             if copies is not None:
-                for dst, src in zip(copies, (self.vpix, self.index, self.image)):
+                for dst, src in zip(copies, (self.vpix, self.index, self.image, self.cover)):
                     dst.copy_(src)
             return self.image
         status = None
@@ -116,7 +127,9 @@ class Renderer:
             if self._status is None:
                 self._status = torch.zeros(2, dtype=torch.int64, pin_memory=True)
             status = self._status
-        self.renders += 1
+            self.renders += 1
+        else:
+            self._drawing()
         verts, attr = verts.contiguous(), attr.contiguous()
         args = (verts, cams, attr, tex, depth, bary, copies or (None, None, None), status)
         code, total = B.mer_view_render(self._view(self.bg), *args)
@@ -132,14 +145,17 @@ class Renderer:
                  terms: int = B.MER_EDGE | B.MER_INTERIOR | B.MER_INTERSECT, grad_attr=None, zero: bool = True):
         if cams.shape[0] != self.n:
             return self._backward_stages(grad_image, cams, attr, tex, terms, grad_attr, zero)
-        return self._backward((self.vpix, self.index, self.cover, self.image), grad_image, cams, attr, tex, terms, grad_attr,
+        return self._backward(self.drawn(), grad_image, cams, attr, tex, terms, grad_attr,
                               None, int(bool(zero)))
 
     def _backward(self, drawn, grad_image, cams, attr, tex, terms, grad_attr, grad_verts_copy, zero):
-        """drawn: the vpix, index, cover and image that the gradient is of; zero: 0, 1 or 2 as in mer_view_backward."""
+        """drawn: the vpix, index, image and cover (if any) that the gradient is of; zero: 0, 1 or 2 as in
+        mer_view_backward."""
         if terms & B.MER_DETERMINISTIC:
             self._ensure_backward_workspace(terms, grad_attr)
-        view = B.view_struct(self.tris, self.V, self.n, self.H, self.W, self.tile, self.workspace, *drawn, self.sh)
+        vpix, index, image, *cover = drawn
+        view = B.view_struct(self.tris, self.V, self.n, self.H, self.W, self.tile, self.workspace, vpix, index,
+                             cover[0] if cover else None, image, self.sh)
         B.mer_view_backward(view, cams, grad_image.contiguous(), attr.contiguous(), tex, terms, self.grad_vpix,
                             grad_attr, self.grad_verts, grad_verts_copy, zero)
         return self.grad_verts
@@ -187,28 +203,23 @@ class MerRender(torch.autograd.Function):
         bary = None
         if not recompute_bary:
             bary = torch.empty((r.n, r.H, r.W, 2), dtype=torch.float32, device=r.device)
-        saved = torch.empty_like(r.vpix), torch.empty_like(r.index), torch.empty_like(r.image)
+        # the gradient is of this drawing, whatever the renderer's buffers hold by then (another forward, a replayed graph)
+        saved = [torch.empty_like(t) for t in r.drawn() if t is not None]
         r.forward(verts, cams, attr, tex, bary=bary, copies=saved)
         ctx.renderer = r
         ctx.renders = r.renders
-        ctx.save_for_backward(verts, attr, cams, *saved, *(() if tex is None else (tex,)),
-                              *(() if bary is None else (bary,)))
-        ctx.has_tex = tex is not None
+        ctx.save_for_backward(verts, attr, cams, tex, bary, *saved)
         return saved[2]
 
     @staticmethod
     def backward(ctx, grad_image):
         r = ctx.renderer
-        saved = ctx.saved_tensors
-        verts, attr, cams, vpix, index, image = saved[:6]
-        tex = saved[6] if ctx.has_tex else None
-        cover = r.cover
-        if r.renders != ctx.renders:  # the renderer has drawn something else since: its cover image is of that
-            r.vpix.copy_(vpix)
-            r.index.copy_(index)
-            r.image.copy_(image)
+        verts, attr, cams, tex, _, *saved = ctx.saved_tensors
+        if r.renders != ctx.renders or r.replayed:  # the buffers hold another drawing: put back what is differentiated
+            for dst, src in zip(r.drawn(), saved):
+                if dst is not None:
+                    dst.copy_(src)
             r.renders += 1
-            cover = None
         grad_attr, zero = None, 1
         if ctx.needs_input_grad[1]:
             if attr.shape == (r.V, r.sh.C_attr):
@@ -216,5 +227,5 @@ class MerRender(torch.autograd.Function):
             else:
                 grad_attr = torch.zeros_like(attr)
         gv = torch.empty_like(r.grad_verts)
-        r._backward((vpix, index, cover, image), grad_image, cams, attr, tex, r.terms, grad_attr, gv, zero)
+        r._backward(saved, grad_image, cams, attr, tex, r.terms, grad_attr, gv, zero)
         return gv, grad_attr, None, None, None, None

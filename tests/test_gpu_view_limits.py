@@ -30,7 +30,7 @@ def test_no_views(zero):
     r, verts, attr, cams = _setup(0)
     r.grad_verts.fill_(7.0)
     copy, ga = torch.full_like(r.grad_verts, 5.0), torch.full_like(attr, 7.0)
-    r._backward((r.vpix, r.index, r.cover, r.image), torch.empty_like(r.image), cams, attr, None, r.terms, ga, copy, zero)
+    r._backward(r.drawn(), torch.empty_like(r.image), cams, attr, None, r.terms, ga, copy, zero)
     assert (r.grad_verts == (0.0 if zero else 7.0)).all() and torch.equal(copy, r.grad_verts)
     assert (ga == (0.0 if zero == 2 else 7.0)).all()
 
