@@ -190,6 +190,13 @@ class Renderer:
             raise B.MerError(code, "device status")
 
 
+def _as_buffer(t: torch.Tensor, like: torch.Tensor | None) -> torch.Tensor:
+    """A saved tensor as the kernels read it: a hook on saved tensors may give it back in another type, place or layout."""
+    if like is None or (t.dtype == like.dtype and t.shape == like.shape and t.device == like.device and t.is_contiguous()):
+        return t
+    return torch.empty_like(like).copy_(t)
+
+
 class MerRender(torch.autograd.Function):
     """image = render(verts, attr); backward = micro-edge + interior kernels.
 
@@ -215,6 +222,7 @@ class MerRender(torch.autograd.Function):
     def backward(ctx, grad_image):
         r = ctx.renderer
         verts, attr, cams, tex, _, *saved = ctx.saved_tensors
+        saved = [_as_buffer(t, like) for t, like in zip(saved, r.drawn())]
         if r.renders != ctx.renders or r.replayed:  # the buffers hold another drawing: put back what is differentiated
             for dst, src in zip(r.drawn(), saved):
                 if dst is not None:
