@@ -203,13 +203,20 @@ def mer_workspace_size(V: int, T: int, n: int, H: int, W: int, tile: int, bin_ca
     return int(lib().mer_workspace_size(V, T, n, H, W, tile, bin_capacity))
 
 
+def _check_records(V: int, n: int, vpix: torch.Tensor):
+    if vpix.numel() < n * V * VERTEX_FLOATS:
+        raise ValueError(f"{n} views of {V} vertices do not fit the vertex records {tuple(vpix.shape)}")
+
+
 def mer_project(verts: torch.Tensor, cams: torch.Tensor, vpix: torch.Tensor):
     V, n = verts.shape[0], cams.shape[0]
+    _check_records(V, n, vpix)
     _check(lib().mer_project(_ptr(verts), V, _ptr(cams), n, _ptr(vpix), _stream()), "mer_project")
 
 
 def mer_project_screen(scr: torch.Tensor, vpix: torch.Tensor):
     n, V = scr.shape[0], scr.shape[1]
+    _check_records(V, n, vpix)
     _check(lib().mer_project_screen(_ptr(scr), V, n, _ptr(vpix), _stream()), "mer_project_screen")
 
 
@@ -261,7 +268,8 @@ def mer_interpolate_backward(attr, tris, vpix, index, grad_out, grad_attr, grad_
 
 
 def mer_project_backward(cams, vpix, grad_vpix, grad_verts):
-    n, V = vpix.shape[0], vpix.shape[1]
+    """The sum over the views that have a camera: the first cams.shape[0] of vpix."""
+    n, V = min(vpix.shape[0], cams.shape[0]), vpix.shape[1]
     _check(lib().mer_project_backward(V, _ptr(cams), n, _ptr(vpix), _ptr(grad_vpix), _ptr(grad_verts), _stream()),
            "mer_project_backward")
 
@@ -281,7 +289,10 @@ def mer_forward_grad(vpix, tris, index, image, tangent, attr, tex, sh: MerShadin
 
 
 def mer_project_jvp(tangent_world, cams, vpix, out):
-    n, V = vpix.shape[0], vpix.shape[1]
+    """Of the views that have a camera: the first cams.shape[0] of vpix; the rest of out is left alone."""
+    n, V = min(vpix.shape[0], cams.shape[0]), vpix.shape[1]
+    if tangent_world.shape[0] < V:
+        raise ValueError(f"a tangent of {tangent_world.shape[0]} vertices for records of {V}")
     _check(lib().mer_project_jvp(_ptr(tangent_world), V, _ptr(cams), n, _ptr(vpix), _ptr(out), _stream()),
            "mer_project_jvp")
 
@@ -340,6 +351,8 @@ def mer_view_forward_grad(view: MerView, cams, tangent_world, attr, tex, terms: 
 
 def mer_rasterize_world(verts, tris, cams, H, W, tile, workspace, index, vpix, depth=None, bary=None):
     n, V = vpix.shape[0], vpix.shape[1]
+    if verts.shape[0] < V or cams.shape[0] < n:
+        raise ValueError(f"{cams.shape[0]} views of {verts.shape[0]} vertices for the records {tuple(vpix.shape)}")
     _check(lib().mer_rasterize_world(_ptr(verts), V, _ptr(tris), tris.shape[0], _ptr(cams), n, H, W, tile,
                                      _ptr(workspace), workspace.numel() * workspace.element_size(), _ptr(index),
                                      _ptr(depth), _ptr(bary), _ptr(vpix), _stream()), "mer_rasterize_world")

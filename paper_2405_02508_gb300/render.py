@@ -48,7 +48,7 @@ class Renderer:
             self.sh.tex_c = int(tex_shape[2]) if len(tex_shape) > 2 else shading.n_main
         self.bg = shading.bg_array()
         n, H, W = self.n, self.H, self.W
-        self.vpix = torch.empty((n, self.V, B.VERTEX_FLOATS), dtype=torch.float32, device=device)
+        self.vpix = torch.zeros((n, self.V, B.VERTEX_FLOATS), dtype=torch.float32, device=device)  # (nothing in front)
         self.index = torch.empty((n, H, W), dtype=torch.int32, device=device)
         self.image = torch.empty((n, H, W, self.C), dtype=torch.float32, device=device)
         self.cover = torch.empty((n, H, W), dtype=torch.uint8, device=device) if cover_hint else None
@@ -71,12 +71,30 @@ class Renderer:
 
     # -- forward -----------------------------------------------------------------------------------
     def project(self, verts: torch.Tensor, cams: torch.Tensor):
+        """Fewer vertices or cameras than the buffers hold give the first records of the first views; the others stay."""
+        self._check_sizes(verts.shape[0], cams.shape[0])
         self._drawing()
-        B.mer_project(verts.contiguous(), cams, self.vpix)
+        verts = verts.contiguous()
+        if verts.shape[0] == self.V:
+            B.mer_project(verts, cams, self.vpix)
+            return
+        for k in range(cams.shape[0]):  # a view's records start at a multiple of V
+            B.mer_project(verts, cams[k:k + 1], self.vpix[k:k + 1])
 
     def project_screen(self, scr: torch.Tensor):
+        """As ``project``, from screen positions [views, vertices, 3]."""
+        self._check_sizes(scr.shape[1], scr.shape[0])
         self._drawing()
-        B.mer_project_screen(scr.contiguous(), self.vpix)
+        scr = scr.contiguous()
+        if scr.shape[1] == self.V:
+            B.mer_project_screen(scr, self.vpix)
+            return
+        for k in range(scr.shape[0]):
+            B.mer_project_screen(scr[k:k + 1], self.vpix[k:k + 1])
+
+    def _check_sizes(self, V: int, n: int):
+        if V > self.V or n > self.n:
+            raise ValueError(f"{n} views of {V} vertices for a renderer of {self.n} views of {self.V}")
 
     def rasterize(self, depth: torch.Tensor | None = None, bary: torch.Tensor | None = None, checked: bool = True):
         self._drawing()
@@ -143,44 +161,49 @@ class Renderer:
     # -- backward ----------------------------------------------------------------------------------
     def backward(self, grad_image: torch.Tensor, cams: torch.Tensor, attr: torch.Tensor, tex=None,
                  terms: int = B.MER_EDGE | B.MER_INTERIOR | B.MER_INTERSECT, grad_attr=None, zero: bool = True):
-        if cams.shape[0] != self.n:
-            return self._backward_stages(grad_image, cams, attr, tex, terms, grad_attr, zero)
-        return self._backward(self.drawn(), grad_image, cams, attr, tex, terms, grad_attr,
-                              None, int(bool(zero)))
+        return self._backward(self.drawn(), grad_image, cams, attr, tex, terms, grad_attr, None, int(bool(zero)))
 
     def _backward(self, drawn, grad_image, cams, attr, tex, terms, grad_attr, grad_verts_copy, zero):
         """drawn: the vpix, index, image and cover (if any) that the gradient is of; zero: 0, 1 or 2 as in
-        mer_view_backward."""
+        mer_view_backward.  With fewer cameras than views, the vertex gradient is of the views that have one."""
+        vpix, index, image, *cover = drawn
+        cover = cover[0] if cover else None
+        grad_image, attr = grad_image.contiguous(), attr.contiguous()
         if terms & B.MER_DETERMINISTIC:
             self._ensure_backward_workspace(terms, grad_attr)
-        vpix, index, image, *cover = drawn
-        view = B.view_struct(self.tris, self.V, self.n, self.H, self.W, self.tile, self.workspace, vpix, index,
-                             cover[0] if cover else None, image, self.sh)
-        B.mer_view_backward(view, cams, grad_image.contiguous(), attr.contiguous(), tex, terms, self.grad_vpix,
-                            grad_attr, self.grad_verts, grad_verts_copy, zero)
-        return self.grad_verts
-
-    def _backward_stages(self, grad_image, cams, attr, tex, terms, grad_attr, zero):
+        if cams.shape[0] >= self.n:
+            view = B.view_struct(self.tris, self.V, self.n, self.H, self.W, self.tile, self.workspace, vpix, index, cover,
+                                 image, self.sh)
+            B.mer_view_backward(view, cams, grad_image, attr, tex, terms, self.grad_vpix, grad_attr, self.grad_verts,
+                                grad_verts_copy, zero)
+            return self.grad_verts
         if zero:
             self.grad_vpix.zero_()
             self.grad_verts.zero_()
-        self._ensure_backward_workspace(terms, grad_attr)
-        B.mer_backward(self.vpix, self.tris, self.index, self.image, grad_image.contiguous(), attr.contiguous(), tex,
-                       self.sh, terms, self.grad_vpix, grad_attr, self.workspace, self.cover)
-        B.mer_project_backward(cams, self.vpix, self.grad_vpix, self.grad_verts)
+        if zero > 1 and grad_attr is not None:
+            grad_attr.zero_()
+        B.mer_backward(vpix, self.tris, index, image, grad_image, attr, tex, self.sh, terms, self.grad_vpix, grad_attr,
+                       self.workspace, cover)
+        B.mer_project_backward(cams, vpix, self.grad_vpix, self.grad_verts)
+        if grad_verts_copy is not None:
+            grad_verts_copy.copy_(self.grad_verts)
         return self.grad_verts
 
     # -- forward gradients ---------------------------------------------------------------------------
     def forward_grad(self, tangent_world: torch.Tensor, cams: torch.Tensor, attr: torch.Tensor, tex=None,
                      terms: int = B.MER_EDGE | B.MER_INTERIOR | B.MER_INTERSECT) -> torch.Tensor:
-        """d(image)/d(theta) [n,H,W,C] for a world-space vertex tangent [V,3] (after ``forward``)."""
-        tv = torch.empty((self.n, self.V, 3), dtype=torch.float32, device=self.device)
+        """d(image)/d(theta) [n,H,W,C] for a world-space vertex tangent [V,3] (after ``forward``).  Vertices without a
+        tangent and views without a camera (fewer than the buffers hold) do not move."""
         out = torch.empty_like(self.image)
-        if tangent_world.shape[0] != self.V or cams.shape[0] != self.n:
-            B.mer_project_jvp(tangent_world.contiguous(), cams, self.vpix, tv)
+        if tangent_world.shape[0] < self.V or cams.shape[0] < self.n:
+            tv = torch.zeros((self.n, self.V, 3), dtype=torch.float32, device=self.device)
+            moved = torch.zeros((self.V, 3), dtype=torch.float32, device=self.device)
+            moved[:tangent_world.shape[0]] = tangent_world[:self.V]
+            B.mer_project_jvp(moved, cams, self.vpix, tv)
             B.mer_forward_grad(self.vpix, self.tris, self.index, self.image, tv, attr.contiguous(), tex, self.sh, terms,
                                out, self.workspace)
             return out
+        tv = torch.empty((self.n, self.V, 3), dtype=torch.float32, device=self.device)
         B.mer_view_forward_grad(self._view(), cams, tangent_world.contiguous(), attr.contiguous(), tex, terms, tv, out)
         return out
 

@@ -45,3 +45,44 @@ def test_no_views_autograd():
     del stale
     gv, ga = torch.autograd.grad(image, (v, a), torch.empty_like(image))
     assert (gv == 0).all() and (ga == 0).all()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("autograd", [False, True])
+def test_fewer_cameras(autograd):
+    """Two cameras on a renderer of three views: the two views and the gradient over them, as a renderer of two gives; the
+    third view stays empty."""
+    r, verts, attr, cams = _setup(3)
+    two, _, _, _ = _setup(2)
+    g = torch.randn(r.image.shape, generator=torch.Generator(device="cuda").manual_seed(1), device="cuda")
+    r.terms = two.terms = 7 | B.MER_DETERMINISTIC
+    ga, gt = torch.zeros_like(attr), torch.zeros_like(attr)
+    two.forward(verts, cams[:2], attr)
+    want = two.backward(g[:2].contiguous(), cams[:2], attr, terms=two.terms, grad_attr=gt)
+    if autograd:
+        v, a = verts.clone().requires_grad_(True), attr.clone().requires_grad_(True)
+        image = MerRender.apply(v, a, None, cams[:2], r)
+        got, ga = torch.autograd.grad(image, (v, a), g)
+    else:
+        image = r.forward(verts, cams[:2], attr)
+        got = r.backward(g, cams[:2], attr, terms=r.terms, grad_attr=ga)
+    assert torch.equal(image[:2], two.image) and (r.index[2] == -1).all()
+    assert torch.equal(got, want) and torch.equal(ga, gt)
+    t = torch.randn(verts.shape, generator=torch.Generator(device="cuda").manual_seed(2), device="cuda")
+    d = r.forward_grad(t, cams[:2], attr)
+    assert torch.equal(d[:2], two.forward_grad(t, cams[:2], attr)) and (d[2] == 0).all()
+
+
+@pytest.mark.gpu
+def test_fewer_vertices():
+    """The first vertices moved on a renderer of two views: both views show them, the other vertices stay."""
+    r, verts, attr, cams = _setup(2)
+    few = len(verts) // 2
+    moved = verts.clone()
+    moved[:few] *= 1.1
+    want = r.forward(moved, cams, attr).clone()
+    r.forward(verts, cams, attr)
+    assert torch.equal(r.forward(moved[:few], cams, attr), want)
+    t = torch.zeros_like(verts)
+    t[:few] = 1.0
+    assert torch.equal(r.forward_grad(t[:few], cams, attr), r.forward_grad(t, cams, attr))
