@@ -454,7 +454,9 @@ size_t mer_precond_solve_workspace_size(int64_t V);
 int mer_precond_solve(const int64_t* row_ptr, const int32_t* col, int64_t V, float lambda, const float* b,
                       float* x, int max_iters, float rel_tol, void* workspace, size_t workspace_bytes,
                       void* stream);
-/* Synchronises `stream` and reports the last solve in `workspace`: iterations run and |r| / |b|. */
+/* Synchronises `stream` and reports the last solve in `workspace`: iterations run and |r| / |b|.  MER_ECUDA also if the solve
+ * gave up: the one-launch form waits for its other thread blocks about a second at most; if one does not answer, some or all
+ * of x is not a number. */
 int mer_precond_solve_info(const void* workspace, int* iters, double* rel_residual, void* stream);
 
 /* Synchronises `stream`, reads and clears the device status word of a

@@ -204,7 +204,7 @@ __global__ void k_cg_next(CgState* st) {
 constexpr int kCgThreads = 512;         // per CTA of the cluster form (one CTA per SM, up to 128 registers a thread)
 constexpr int kCgLocalThreads = 1024;   // the single-CTA form
 constexpr int kCgNeighbours = 8;        // neighbour ids kept in registers (a closed mesh averages 6)
-constexpr unsigned kCgSpinLimit = 1u << 21;  // polls of one exchange (about a second) before the solve gives up
+constexpr unsigned kCgPolls = 1u << 21;  // polls of one exchange (about a second) before the solve gives up
 constexpr int kCgCluster = 8;           // CTAs of a cluster
 constexpr int kCgMaxClusters = 32;      // one slot per lane of a warp
 
@@ -309,7 +309,7 @@ __device__ __forceinline__ void cluster_sync() {
 // writes to the exchanged vectors made before the call are visible to every thread after it (without it, only that
 // every thread has done its reads).
 template <bool CLUSTER, bool PUBLISH, typename T, typename Then>
-__device__ __forceinline__ void cg_sum(T v, unsigned step, CgSlot* slots, CgShared& S, Then then) {
+__device__ __forceinline__ void cg_sum(T v, unsigned step, CgSlot* slots, unsigned max_polls, CgShared& S, Then then) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const T zero = from_bits<T>(0u, 0u);
     T* part = reinterpret_cast<T*>(S.part);
@@ -349,7 +349,7 @@ __device__ __forceinline__ void cg_sum(T v, unsigned step, CgSlot* slots, CgShar
                     asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];"
                                  : "=l"(wa), "=l"(wb) : "l"(set + lane) : "memory");
                 if (__all_sync(0xffffffffu, (unsigned)(wa >> 32) == step && (unsigned)(wb >> 32) == step)) break;
-                if (polls > kCgSpinLimit) {
+                if (polls >= max_polls) {
                     ok = false;
                     break;
                 }
@@ -386,7 +386,7 @@ template <int R, bool CLUSTER>
 __global__ void __launch_bounds__(CLUSTER ? kCgThreads : kCgLocalThreads, 1)
     k_cg_solve(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int V, float lambda,
                const float* __restrict__ b, float* __restrict__ x, float4* r_ws, float4* p_ws, CgSlot* slots, CgState* st,
-               int max_iters, float rel_tol, int rows) {
+               int max_iters, float rel_tol, int rows, unsigned max_polls) {
     extern __shared__ float4 sm[];
     __shared__ CgShared S;
     // residual and search direction (two buffers) of the CTA's rows; CLUSTER: also in the workspace, for the other CTAs
@@ -439,8 +439,8 @@ __global__ void __launch_bounds__(CLUSTER ? kCgThreads : kCgLocalThreads, 1)
     if (threadIdx.x == 0) S.stop = S.failed = 0;
     if (CLUSTER) cluster_sync();  // every CTA of the cluster has started and cleared its words
     unsigned step = 1;
-    cg_sum<CLUSTER, true>(s_bb, step++, slots, S, [&](double v) { rr0 = v; });
-    cg_sum<CLUSTER, false>(s_rr, step++, slots, S, [&](double v) {
+    cg_sum<CLUSTER, true>(s_bb, step++, slots, max_polls, S, [&](double v) { rr0 = v; });
+    cg_sum<CLUSTER, false>(s_rr, step++, slots, max_polls, S, [&](double v) {
         const int e = min(max((int)((__double2hiint(v) >> 20) & 0x7ff) - 1023, -240), 240) / 2;
         S.coef = __int_as_float((127 - e) << 23);  // 2^-e
         unit = (double)S.coef * (double)S.coef;
@@ -502,7 +502,7 @@ __global__ void __launch_bounds__(CLUSTER ? kCgThreads : kCgLocalThreads, 1)
             if (CLUSTER) cg_store(p_new + row[k], pr[k][0], pr[k][1], pr[k][2]);
         }
         // p_new is read after the next exchange only, so this one publishes nothing
-        cg_sum<CLUSTER, false>(d, step++, slots, S, [&](F2 v) { S.coef = v.hi > 0.f ? f2_ratio(rr, v) : 0.f; });
+        cg_sum<CLUSTER, false>(d, step++, slots, max_polls, S, [&](F2 v) { S.coef = v.hi > 0.f ? f2_ratio(rr, v) : 0.f; });
         if (S.stop) break;
         // x += alpha p, r -= alpha M p, r . r
         const float alpha = S.coef;
@@ -519,7 +519,7 @@ __global__ void __launch_bounds__(CLUSTER ? kCgThreads : kCgLocalThreads, 1)
             sm[row[k] - base] = make_float4(rr_[k][0], rr_[k][1], rr_[k][2], 0.f);
             if (CLUSTER) cg_store(r_ws + row[k], rr_[k][0], rr_[k][1], rr_[k][2]);
         }
-        cg_sum<CLUSTER, true>(d, step++, slots, S, [&](F2 v) {
+        cg_sum<CLUSTER, true>(d, step++, slots, max_polls, S, [&](F2 v) {
             S.coef = rr.hi > 0.f ? f2_ratio(v, rr) : 0.f;
             rr = v;
             if (((double)v.hi + (double)v.lo) <= tol2 * unit) S.stop = 1;
@@ -531,7 +531,8 @@ __global__ void __launch_bounds__(CLUSTER ? kCgThreads : kCgLocalThreads, 1)
     for (int k = 0; k < R; ++k) {
         if (row[k] < 0) continue;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) x[3 * (size_t)row[k] + c] = xr[k][c];
+        for (int c = 0; c < 3; ++c)  // a solve that gave up must not pass for one
+            x[3 * (size_t)row[k] + c] = S.failed ? __int_as_float(0x7fffffff) : xr[k][c];
     }
     if (threadIdx.x == 0) {
         if (blockIdx.x == 0) {
@@ -560,7 +561,8 @@ constexpr size_t kCgSlotBytes = 2 * kCgMaxClusters * sizeof(CgSlot);
 // all fit on the device at once.
 template <int R, bool CLUSTER>
 cudaError_t launch_cg(const int64_t* row_ptr, const int32_t* col, int V, float lambda, const float* b, float* x,
-                      float4* r, float4* p, CgSlot* slots, CgState* st, int max_iters, float rel_tol, cudaStream_t s) {
+                      float4* r, float4* p, CgSlot* slots, CgState* st, int max_iters, float rel_tol, unsigned max_polls,
+                      cudaStream_t s) {
     constexpr int kT = CLUSTER ? kCgThreads : kCgLocalThreads;
     constexpr int kBytes = 3 * kT * R * (int)sizeof(float4);
     constexpr int kUnit = CLUSTER ? kCgCluster : 1;
@@ -591,7 +593,8 @@ cudaError_t launch_cg(const int64_t* row_ptr, const int32_t* col, int V, float l
         }
     }
     const int rows = (V + units * kUnit - 1) / (units * kUnit);
-    return cudaLaunchKernelEx(&c, kernel, row_ptr, col, V, lambda, b, x, r, p, slots, st, max_iters, rel_tol, rows);
+    return cudaLaunchKernelEx(&c, kernel, row_ptr, col, V, lambda, b, x, r, p, slots, st, max_iters, rel_tol, rows,
+                              max_polls);
 }
 
 // The solve as a fixed sequence of launches (the state cleared before).
@@ -664,18 +667,14 @@ extern "C" size_t mer_precond_solve_workspace_size(int64_t V) {
     return align256(sizeof(CgState)) + kCgSlotBytes + 3 * align256((size_t)V * sizeof(float4));
 }
 
-extern "C" int mer_precond_solve(const int64_t* row_ptr, const int32_t* col, int64_t V, float lambda,
-                                 const float* b, float* x, int max_iters, float rel_tol, void* workspace,
-                                 size_t workspace_bytes, void* stream) {
-    if (V < 0 || !(lambda >= 0.f) || max_iters < 0 || !(rel_tol >= 0.f)) return MER_EINVAL;
-    if (V == 0) return MER_OK;
-    if (!row_ptr || !col || !b || !x || b == x || !workspace) return MER_EINVAL;
-    if ((reinterpret_cast<uintptr_t>(workspace) & 255u) != 0) return MER_EINVAL;
-    if (workspace_bytes < mer_precond_solve_workspace_size(V)) return MER_EINVAL;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
+// The solve with its choices open: max_polls of an exchange, and `launches` for the fixed sequence whatever the size.
+extern "C" int mer_launch_precond_solve(const int64_t* row_ptr, const int32_t* col, int64_t V, float lambda, const float* b,
+                                        float* x, int max_iters, float rel_tol, void* workspace, unsigned max_polls,
+                                        int launches, cudaStream_t s) {
     char* base = static_cast<char*>(workspace);
     CgState* st = reinterpret_cast<CgState*>(base);
     if (cudaMemsetAsync(st, 0, align256(sizeof(CgState)) + kCgSlotBytes, s) != cudaSuccess) return MER_ECUDA;
+    if (launches) return solve_launches(row_ptr, col, V, lambda, b, x, max_iters, rel_tol, base, s);
     CgSlot* slots = reinterpret_cast<CgSlot*>(base + align256(sizeof(CgState)));
     float4* r4 = reinterpret_cast<float4*>(base + align256(sizeof(CgState)) + kCgSlotBytes);
     float4* p4 = r4 + V;
@@ -687,16 +686,28 @@ extern "C" int mer_precond_solve(const int64_t* row_ptr, const int32_t* col, int
     constexpr int64_t kClusterRows = kCgCluster * kCgThreads;
     cudaError_t e = cudaErrorNotSupported;
     if (V <= kCgLocalThreads)
-        e = launch_cg<1, false>(row_ptr, col, (int)V, lambda, b, x, r4, p4, slots, st, max_iters, rel_tol, s);
+        e = launch_cg<1, false>(row_ptr, col, (int)V, lambda, b, x, r4, p4, slots, st, max_iters, rel_tol, max_polls, s);
     else if (V <= kCgMaxClusters * kClusterRows && (V <= kClusterRows || V > 2 * kClusterRows))
-        e = launch_cg<1, true>(row_ptr, col, (int)V, lambda, b, x, r4, p4, slots, st, max_iters, rel_tol, s);
+        e = launch_cg<1, true>(row_ptr, col, (int)V, lambda, b, x, r4, p4, slots, st, max_iters, rel_tol, max_polls, s);
     if (e == cudaErrorNotSupported && V <= 2 * kCgMaxClusters * kClusterRows)
-        e = launch_cg<2, true>(row_ptr, col, (int)V, lambda, b, x, r4, p4, slots, st, max_iters, rel_tol, s);
+        e = launch_cg<2, true>(row_ptr, col, (int)V, lambda, b, x, r4, p4, slots, st, max_iters, rel_tol, max_polls, s);
     if (e == cudaErrorNotSupported && V <= 4 * kCgMaxClusters * kClusterRows)
-        e = launch_cg<4, true>(row_ptr, col, (int)V, lambda, b, x, r4, p4, slots, st, max_iters, rel_tol, s);
+        e = launch_cg<4, true>(row_ptr, col, (int)V, lambda, b, x, r4, p4, slots, st, max_iters, rel_tol, max_polls, s);
     if (e == cudaErrorNotSupported)
         return solve_launches(row_ptr, col, V, lambda, b, x, max_iters, rel_tol, base, s);
     return e == cudaSuccess ? MER_OK : MER_ECUDA;
+}
+
+extern "C" int mer_precond_solve(const int64_t* row_ptr, const int32_t* col, int64_t V, float lambda,
+                                 const float* b, float* x, int max_iters, float rel_tol, void* workspace,
+                                 size_t workspace_bytes, void* stream) {
+    if (V < 0 || !(lambda >= 0.f) || max_iters < 0 || !(rel_tol >= 0.f)) return MER_EINVAL;
+    if (V == 0) return MER_OK;
+    if (!row_ptr || !col || !b || !x || b == x || !workspace) return MER_EINVAL;
+    if ((reinterpret_cast<uintptr_t>(workspace) & 255u) != 0) return MER_EINVAL;
+    if (workspace_bytes < mer_precond_solve_workspace_size(V)) return MER_EINVAL;
+    return mer_launch_precond_solve(row_ptr, col, V, lambda, b, x, max_iters, rel_tol, workspace, kCgPolls, 0,
+                                    static_cast<cudaStream_t>(stream));
 }
 
 extern "C" int mer_precond_solve_info(const void* workspace, int* iters, double* rel_residual, void* stream) {

@@ -35,7 +35,8 @@ class LaplacianPreconditioner:
         return y
 
     def solve(self, b: torch.Tensor, x0: torch.Tensor | None = None) -> torch.Tensor:
-        """M^-1 b, starting from x0 (zeros if None)."""
+        """M^-1 b, starting from x0 (zeros if None).  A solve that the device gave up holds values that are not numbers
+        (``last_solve`` raises)."""
         x = torch.zeros_like(b) if x0 is None else x0.clone()
         B.mer_precond_solve(self.row_ptr, self.col, self.lam, b.contiguous(), x, self.max_iters, self.rel_tol,
                             self.workspace)
