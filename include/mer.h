@@ -445,8 +445,9 @@ int mer_laplacian_csr(const int32_t* tris, int64_t T, int64_t V, int64_t* row_pt
 int mer_precond_apply(const int64_t* row_ptr, const int32_t* col, int64_t V, float lambda, const float* x,
                       float* y, void* stream);
 size_t mer_precond_solve_workspace_size(int64_t V);
-/* Solve (I + lambda L) x = b by conjugate gradients on the device (FP32 vectors, FP64 dot products), the
- * three columns as one block-diagonal system.  x holds the initial guess (a warm start) and receives the
+/* Solve (I + lambda L) x = b by conjugate gradients on the device (FP32 vectors; dot products of exact
+ * products, summed to about 48 bits in the one-launch form and in FP64 in the sequence), the three columns as one
+ * block-diagonal system.  x holds the initial guess (a warm start) and receives the
  * solution.  Runs at most max_iters iterations and ends when the residual norm falls to rel_tol * |b|: in
  * one launch while the rows fit one resident grid (about 260,000 on GB300), beyond that as a fixed
  * launch sequence whose later iterations return immediately.  Either can be captured in a graph.  workspace: 256-byte aligned device memory of

@@ -6,7 +6,7 @@
 // step then needs M x (once, to start) and two solves M y = b per step: the gradient with respect to u,
 // M^-1 dL/dx, and the positions x = M^-1 u after the update.  M is symmetric positive definite (its
 // eigenvalues are 1 + lambda * those of L, all >= 1), so the solves are conjugate gradients on the device:
-// FP32 vectors, FP64 dot products, all three coordinate columns as one block-diagonal system, the iteration
+// FP32 vectors, dot products of exact products in FP64 or two-float sums (about 48 bits), all three coordinate columns as one block-diagonal system, the iteration
 // scalars kept on the device (so a solve can be captured in a graph): one launch that ends once the residual is below
 // the tolerance, or, for systems beyond one resident grid, a fixed sequence of launches that become no-ops then.
 //
@@ -196,11 +196,14 @@ __global__ void k_cg_next(CgState* st) {
 // A step is a sum over the CTA, over the CTAs of its cluster (in shared memory, with the hardware's cluster barrier),
 // and over the clusters: the first CTA of each publishes the sum with the step's number and reads the others'.  All
 // CTAs reading all CTAs' sums instead cost 5,000 cycles an exchange with 128 of them.
-// The dot products are sums of exact products (each split in two floats by an FMA) in two-float arithmetic, about 48
-// bits, and so are the iteration's two quotients: GB300's FP64 pipe issues one warp instruction in 16 cycles, and the
-// 64-bit sums and divisions took longer than the exchanges (9 us an iteration of 258 rows, now 2.8).
-// Measured (lambda 16, residual 1e-6, 79 and 49 iterations): 65,538 rows 3,520 -> 612 us, 642 rows 2,350 -> 155 us,
-// with the same bits as the launches gave.
+// The first two sums are FP64; those of the iterations are sums of exact products (each split in two floats by an FMA) in
+// two-float arithmetic, about 48 bits against FP64's 53, and so are the iteration's two quotients before they are rounded to
+// the FP32 factors alpha and beta.  GB300's FP64 pipe issues one warp instruction in 16 cycles, and the 64-bit sums and
+// divisions took longer than the exchanges (9 us an iteration of 258 rows, now 2.8).  The vectors are FP32, so the five bits
+// are far below what a solve can show: in 576 solves of 258 to 211,602 rows (lambda 8, 16 and 32, rough, smooth and mixed
+// right-hand sides, cold and warm starts) iterations and solutions had the same bits as the launch sequence, whose sums
+// are FP64, hence the same errors against a 64-bit solution.
+// Measured (lambda 16, residual 1e-6, 79 and 49 iterations): 65,538 rows 3,520 -> 612 us, 642 rows 2,350 -> 155 us.
 constexpr int kCgThreads = 512;         // per CTA of the cluster form (one CTA per SM, up to 128 registers a thread)
 constexpr int kCgLocalThreads = 1024;   // the single-CTA form
 constexpr int kCgNeighbours = 8;        // neighbour ids kept in registers (a closed mesh averages 6)
@@ -681,8 +684,9 @@ extern "C" int mer_launch_precond_solve(const int64_t* row_ptr, const int32_t* c
     // One CTA up to its 1,024 threads (902 rows: 3.9 us an iteration, the same as a cluster; 258 rows: 2.8 against 4.0).
     // One cluster, with two rows a thread where that saves the exchange between clusters (6,402 rows: 5.4 against 6.4 us).
     // Then the fewest rows a thread whose clusters all fit on the device (16 clusters of 8 with one CTA per SM): 32,402
-    // rows 6.9 us with one row, 7.9 with two; 65,538 rows 7.8 us with two.  Larger systems, which one grid cannot hold,
-    // and devices without room take the launches, 45-55 us an iteration at any of these sizes.
+    // rows 6.9 us with one row, 7.9 with two; 65,538 rows 7.8 us with two; 131,046 rows 11.7 us with four, although that
+    // form spills, 211,602 rows 12.6 (the launches 52 and 57).  Larger systems, which one grid cannot hold,
+    // and devices without room take the launches, 36-60 us an iteration up to 262,146 rows, 91 at 620,946.
     constexpr int64_t kClusterRows = kCgCluster * kCgThreads;
     cudaError_t e = cudaErrorNotSupported;
     if (V <= kCgLocalThreads)
