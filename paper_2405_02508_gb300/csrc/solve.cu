@@ -303,7 +303,9 @@ __device__ __forceinline__ unsigned peer_shared(const void* p, unsigned rank) {
     return a;
 }
 
+// (Aligned: a warp executes it together, and callers come from code that only some of its lanes ran.)
 __device__ __forceinline__ void cluster_sync() {
+    __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
