@@ -175,20 +175,17 @@ __global__ void __launch_bounds__(kFTW * kFTH) k_forward_grad(const mer_vertex* 
         for (int k = 0; k < 3; ++k) load_tangent(tb, vid[k], tv[k]);
         const float Tx = B.lam[0] * tv[0][0] + B.lam[1] * tv[1][0] + B.lam[2] * tv[2][0];
         const float Ty = B.lam[0] * tv[0][1] + B.lam[1] * tv[1][1] + B.lam[2] * tv[2][1];
-        float dl[3], z[3];
-        float s = 0.f, ds = 0.f;
+        float dl[3], z[3], b[3], db[3];
+        float ds = 0.f;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             dl[k] = -(B.gx[k] * Tx + B.gy[k] * Ty);
             z[k] = rv[k].zeta;
-            s += B.lam[k] * z[k];
             ds += dl[k] * z[k] + B.lam[k] * tv[k][2];
         }
-        const float is = rcp_nr(s);
-        float b[3], db[3];
+        const float is = perspective(B, rv, b);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            b[k] = B.lam[k] * z[k] * is;
             db[k] = (dl[k] * z[k] + B.lam[k] * tv[k][2]) * is - b[k] * ds * is;
         }
         const int Ca = a.sh.C_attr;

@@ -283,6 +283,7 @@ __device__ __forceinline__ double i2d(int v) {
 // a*b - c*d, the second product rounded.  The values that decide which texel cell a pixel reads (barycentrics, perspective
 // weights, texel coordinates) are written with their roundings fixed: left to the compiler, the contraction into FMAs
 // depends on the code around them, and a kernel's variants then disagree at cell borders, where the derivative jumps.
+// (The backward's weights have an order of their own, that of its first version, so its gradients stay what they were.)
 __device__ __forceinline__ float det2(float a, float b, float c, float d) { return __fmaf_rn(a, b, -__fmul_rn(c, d)); }
 
 // A projected vertex record loaded with two 128-bit loads (records are 32-byte aligned).

@@ -61,6 +61,18 @@ __device__ __forceinline__ void load_uv(const float* __restrict__ attr, int Ca, 
     }
 }
 
+// Perspective-correct weights b of a pixel's screen barycentrics; returns the depth.  With fixed roundings (see det2), the same
+// for the image and its derivative along a parameter, in every form.
+__device__ __forceinline__ float perspective(const Bary& B, const VRec v[3], float b[3]) {
+    float q[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) q[k] = __fmul_rn(B.lam[k], v[k].zeta);
+    const float is = rcp_nr(__fadd_rn(__fadd_rn(q[0], q[1]), q[2]));
+#pragma unroll
+    for (int k = 0; k < 3; ++k) b[k] = __fmul_rn(q[k], is);
+    return is;
+}
+
 // The C channels of pixel (x, y) covered by triangle t (t < 0: background), written to o[0..C).  vb / tris /
 // attr are the item's bases.  CHECK: t and the vertex ids may be out of range (the fused raster's are not: its setup
 // drops such triangles).  DUAL: also to o2.
@@ -96,12 +108,8 @@ __device__ __forceinline__ void shade_fragment(const mer_vertex* __restrict__ vb
     }
     const VRec v[3] = {load_vrec(vb + vid[0]), load_vrec(vb + vid[1]), load_vrec(vb + vid[2])};
     const Bary B = screen_bary(v, x, y);
-    float q[3], b[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) q[k] = __fmul_rn(B.lam[k], v[k].zeta);
-    const float is = rcp_nr(__fadd_rn(__fadd_rn(q[0], q[1]), q[2]));
-#pragma unroll
-    for (int k = 0; k < 3; ++k) b[k] = __fmul_rn(q[k], is);
+    float b[3];
+    const float is = perspective(B, v, b);
     const int Ca = a.sh.C_attr;
     if (FORM == kAttr3) {
         float acc[3] = {0.f, 0.f, 0.f};
