@@ -152,6 +152,7 @@ __global__ void k_project_backward_batch(const mer_camera* __restrict__ cams, co
     __shared__ CameraF s_cam[8];  // of each warp's first item, converted by its lanes together
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
+    if (i - lane >= vrecs) return;  // a warp past the end: the item found for it may be an empty one, whose camera nothing checks
     const int k = warp_find_item(items, n_items, i - lane, i, kFieldVrec);
     const int first = __shfl_sync(0xffffffffu, k, 0);
     CameraF& cam = s_cam[threadIdx.x >> 5];
