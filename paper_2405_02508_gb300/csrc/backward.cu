@@ -76,7 +76,7 @@ struct BwdArgs {
 // Vertex ids of triangle t; false if one is out of range.
 __device__ __forceinline__ bool tri_ids(const int* __restrict__ tris, int t, int V, int id[3]) {
 #pragma unroll
-    for (int k = 0; k < 3; ++k) id[k] = __ldg(tris + 3 * (size_t)t + k);
+    for (int k = 0; k < 3; ++k) id[k] = load(tris + 3 * (size_t)t + k);
     return max(max((unsigned)id[0], (unsigned)id[1]), (unsigned)id[2]) < (unsigned)V;
 }
 
@@ -284,7 +284,7 @@ __device__ __forceinline__ bool edge_rows(const BItem& it, const BwdArgs& a, Bwd
                     int Xq[3], Yq[3];
 #pragma unroll
                     for (int k = 0; k < 3; ++k) {  // snapped position only: one 64-bit load per vertex
-                        const int2 xy = __ldg(reinterpret_cast<const int2*>(vb + vq[k]));
+                        const int2 xy = load(reinterpret_cast<const int2*>(vb + vq[k]));
                         Xq[k] = xy.x;
                         Yq[k] = xy.y;
                     }
@@ -320,7 +320,7 @@ __device__ __forceinline__ bool edge_rows(const BItem& it, const BwdArgs& a, Bwd
             }
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                const int2 xy = __ldg(reinterpret_cast<const int2*>(vb + vs[k]));
+                const int2 xy = load(reinterpret_cast<const int2*>(vb + vs[k]));
                 Xs[k] = xy.x;
                 Ys[k] = xy.y;
             }
@@ -339,8 +339,8 @@ __device__ __forceinline__ bool edge_rows(const BItem& it, const BwdArgs& a, Bwd
         const bool p_is_a = ddx > 0 || ddy > 0;
         float dLdp = 0.f;
         for (int c = 0; c < C; ++c) {
-            const float diff = __ldg(ip + c) - __ldg(iq + c);
-            dLdp += 0.5f * (__ldg(gp + c) + __ldg(gq + c)) * (p_is_a ? diff : -diff);
+            const float diff = load(ip + c) - load(iq + c);
+            dLdp += 0.5f * (load(gp + c) + load(gq + c)) * (p_is_a ? diff : -diff);
         }
         float ex = 0.f, ey = 0.f, ez = 0.f;
         if (!inter) {
@@ -349,8 +349,8 @@ __device__ __forceinline__ bool edge_rows(const BItem& it, const BwdArgs& a, Bwd
                 const int e = exit_edge(Xs, Ys, 256 * px + 128, 256 * y + 128, 256 * qx + 128, 256 * qy + 128);
                 if (e >= 0) {
                     const int j = (e + 1) % 3, l = (e + 2) % 3;
-                    const float4 rj = __ldg(reinterpret_cast<const float4*>(vb + vs[j]));
-                    const float4 rl = __ldg(reinterpret_cast<const float4*>(vb + vs[l]));
+                    const float4 rj = load(reinterpret_cast<const float4*>(vb + vs[j]));
+                    const float4 rl = load(reinterpret_cast<const float4*>(vb + vs[l]));
                     const float u = axis == 0 ? crossing_u(Ys[j], rj.w, Ys[l], rl.w, 256 * y + 128)
                                               : crossing_u(Xs[j], rj.z, Xs[l], rl.z, 256 * px + 128);
                     atomicAdd(&S.evert[row][src][j][axis], (1.0f - u) * dLdp);
@@ -429,8 +429,8 @@ __device__ __forceinline__ bool tile_halo(const BItem& it, const BwdArgs& a, int
         const int h = warp + q * kWarps, y = y0 + h;
         const bool in = h < kHH && y >= 0 && y < H && x < W;
         const int o = in ? y * W + x : 0;
-        v[q] = in ? __ldg(ib + o) : -2;
-        c[q] = in && cb ? __ldg(cb + o) : (unsigned char)0;
+        v[q] = in ? load(ib + o) : -2;
+        c[q] = in && cb ? load(cb + o) : (unsigned char)0;
     }
     const int e = (int)threadIdx.x - (kThreads - 64);  // halo entry: row e / 2, left or right
     const bool side = e >= 0 && e < 2 * kHH;
@@ -438,8 +438,8 @@ __device__ __forceinline__ bool tile_halo(const BItem& it, const BwdArgs& a, int
         const int hx = tx * kTW + (e & 1 ? kTW : -1), hy = y0 + (e >> 1);
         const bool in = hx >= 0 && hx < W && hy >= 0 && hy < H;
         const int o = in ? hy * W + hx : 0;
-        v[kN] = in ? __ldg(ib + o) : -2;
-        c[kN] = in && cb ? __ldg(cb + o) : (unsigned char)0;
+        v[kN] = in ? load(ib + o) : -2;
+        c[kN] = in && cb ? load(cb + o) : (unsigned char)0;
     }
     bool covered = false;
 #pragma unroll
@@ -519,8 +519,8 @@ __device__ __forceinline__ void row_pass(const BItem& it, int tx, int ty, int ro
                             *q2 = attr + (long long)vid[2] * Ca;
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
-                    const float gc = __ldg(gp + c);
-                    const float a0 = __ldg(q0 + c), a1 = __ldg(q1 + c), a2 = __ldg(q2 + c);
+                    const float gc = load(gp + c);
+                    const float a0 = load(q0 + c), a1 = load(q1 + c), a2 = load(q2 + c);
                     D01 += gc * (a0 - a1);
                     D02 += gc * (a0 - a2);
                     D12 += gc * (a1 - a2);
@@ -531,10 +531,10 @@ __device__ __forceinline__ void row_pass(const BItem& it, int tx, int ty, int ro
                 }
             } else if (FORM != kTex3 && a.sh.uv_offset < 0) {
                 for (int c = 0; c < a.sh.n_main; ++c) {
-                    const float gc = __ldg(gp + c);
-                    const float a0 = __ldg(attr + (size_t)vid[0] * Ca + c);
-                    const float a1 = __ldg(attr + (size_t)vid[1] * Ca + c);
-                    const float a2 = __ldg(attr + (size_t)vid[2] * Ca + c);
+                    const float gc = load(gp + c);
+                    const float a0 = load(attr + (size_t)vid[0] * Ca + c);
+                    const float a1 = load(attr + (size_t)vid[1] * Ca + c);
+                    const float a2 = load(attr + (size_t)vid[2] * Ca + c);
                     D01 += gc * (a0 - a1);
                     D02 += gc * (a0 - a2);
                     D12 += gc * (a1 - a2);
@@ -558,9 +558,9 @@ __device__ __forceinline__ void row_pass(const BItem& it, int tx, int ty, int ro
                 if (FORM == kTex3) {
                     const TexQuad q = tex_quad(tex, a.sh.tex_w, taps);
                     float su = 0.f, sv = 0.f;
-                    tex_lerp_grad(q.a00.x, q.a10.x, q.a01.x, q.a11.x, taps, __ldg(gp), su, sv);
-                    tex_lerp_grad(q.a00.y, q.a10.y, q.a01.y, q.a11.y, taps, __ldg(gp + 1), su, sv);
-                    tex_lerp_grad(q.a00.z, q.a10.z, q.a01.z, q.a11.z, taps, __ldg(gp + 2), su, sv);
+                    tex_lerp_grad(q.a00.x, q.a10.x, q.a01.x, q.a11.x, taps, load(gp), su, sv);
+                    tex_lerp_grad(q.a00.y, q.a10.y, q.a01.y, q.a11.y, taps, load(gp + 1), su, sv);
+                    tex_lerp_grad(q.a00.z, q.a10.z, q.a01.z, q.a11.z, taps, load(gp + 2), su, sv);
                     gu = (float)a.sh.tex_w * su;
                     gv = taps.clamped ? 0.0f : (float)a.sh.tex_h * sv;
                 } else {
@@ -579,7 +579,7 @@ __device__ __forceinline__ void row_pass(const BItem& it, int tx, int ty, int ro
             }
             // G_k - Gbar = sum_i b_i (G_k - G_i)
             const float GmG[3] = {b[1] * D01 + b[2] * D02, b[2] * D12 - b[0] * D01, -(b[0] * D02 + b[1] * D12)};
-            const float gZ = a.sh.depth_ch >= 0 ? __ldg(gp + a.sh.depth_ch) : 0.f;
+            const float gZ = a.sh.depth_ch >= 0 ? load(gp + a.sh.depth_ch) : 0.f;
             // w = sum_k (dL/d lambda_k) grad lambda_k with dL/d lambda_k = zeta_k is (GmG_k - gZ is).  The depth
             // part -gZ is^2 sum_k zeta_k grad lambda_k equals -gZ is^2 sum_k (zeta_k - zeta_0) grad lambda_k
             // (the gradients sum to zero); the zeta differences come from the hi + lo split, so the near
@@ -739,13 +739,13 @@ __device__ __forceinline__ void tile_flush(const BItem& it, const BwdArgs& a, Bw
 }
 
 template <int FORM, int NA, bool EXACT, int BITS>
-__global__ void __launch_bounds__(kThreads, kCtasPerSm) k_backward(const mer_vertex* __restrict__ vpix, const int* __restrict__ tris,
-                                                       const int* __restrict__ index,
-                                                       const unsigned char* __restrict__ cover,
-                                                       const float* __restrict__ image,
-                                                       const float* __restrict__ grad, const float* __restrict__ attr,
-                                                       const float* __restrict__ tex, BwdArgs a,
-                                                       double* __restrict__ grad_vpix, float* __restrict__ grad_attr,
+__global__ void __launch_bounds__(kThreads, kCtasPerSm) k_backward(const mer_vertex* vpix, const int* tris,
+                                                       const int* index,
+                                                       const unsigned char* cover,
+                                                       const float* image,
+                                                       const float* grad, const float* attr,
+                                                       const float* tex, BwdArgs a,
+                                                       double* grad_vpix, float* grad_attr,
                                                        void* ws) {
     after_previous();
     __shared__ BwdShared<NA, EXACT, BITS> S;
@@ -809,17 +809,17 @@ __device__ __forceinline__ void take_tile(WsHeader* hdr, const mer_item* __restr
 
 // Persistent: each CTA takes the next backward tile of any item from the work queue.
 template <int FORM, int NA, bool EXACT, int BITS>
-__global__ void __launch_bounds__(kThreads, kCtasPerSm) k_backward_batch(const mer_vertex* __restrict__ vpix,
-                                                             const int* __restrict__ tris,
-                                                             const mer_item* __restrict__ items, int n_items,
-                                                             long long btiles, const int* __restrict__ index,
-                                                             const unsigned char* __restrict__ cover,
-                                                             const float* __restrict__ image,
-                                                             const float* __restrict__ grad,
-                                                             const float* __restrict__ attr,
-                                                             const float* __restrict__ tex, BwdArgs a,
-                                                             double* __restrict__ grad_vpix,
-                                                             float* __restrict__ grad_attr, void* ws) {
+__global__ void __launch_bounds__(kThreads, kCtasPerSm) k_backward_batch(const mer_vertex* vpix,
+                                                             const int* tris,
+                                                             const mer_item* items, int n_items,
+                                                             long long btiles, const int* index,
+                                                             const unsigned char* cover,
+                                                             const float* image,
+                                                             const float* grad,
+                                                             const float* attr,
+                                                             const float* tex, BwdArgs a,
+                                                             double* grad_vpix,
+                                                             float* grad_attr, void* ws) {
     after_previous();
     __shared__ BwdShared<NA, EXACT, BITS> S;
     __shared__ TileJob s_job[2];

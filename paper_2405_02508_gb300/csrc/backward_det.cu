@@ -108,7 +108,7 @@ __device__ __forceinline__ void tri_normal_f64(const VRec r[3], double N[3]) {
 __device__ __forceinline__ bool ids_of(const int* __restrict__ tris, int t, int V, int id[3]) {
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        id[k] = __ldg(tris + 3 * (size_t)t + k);
+        id[k] = load(tris + 3 * (size_t)t + k);
         if ((unsigned)id[k] >= (unsigned)V) return false;
     }
     return true;
@@ -123,7 +123,7 @@ template <bool ATTR>
 __device__ int det_pixel(const DetItem& it, const DetArgs& a, const float* __restrict__ tex, int x, int y, void* ws,
                          int vid[3], Fix cv[3][3], Fix ca[3][ATTR ? kDetMaxA : 1]) {
     const size_t p = (size_t)y * it.W + x;
-    int t = __ldg(it.index + p);
+    int t = load(it.index + p);
     if (t < 0) return -1;
     if (t >= it.T || !ids_of(it.tris, t, it.V, vid)) {
         set_status(ws, kStatusRange);
@@ -155,10 +155,10 @@ __device__ int det_pixel(const DetItem& it, const DetArgs& a, const float* __res
         const int Ca = a.sh.C_attr;
         if (a.sh.uv_offset < 0) {
             for (int c = 0; c < a.sh.n_main; ++c) {
-                const double gc = (double)__ldg(gp + c);
-                const double a0 = __ldg(it.attr + (size_t)vid[0] * Ca + c);
-                const double a1 = __ldg(it.attr + (size_t)vid[1] * Ca + c);
-                const double a2 = __ldg(it.attr + (size_t)vid[2] * Ca + c);
+                const double gc = (double)load(gp + c);
+                const double a0 = load(it.attr + (size_t)vid[0] * Ca + c);
+                const double a1 = load(it.attr + (size_t)vid[1] * Ca + c);
+                const double a2 = load(it.attr + (size_t)vid[2] * Ca + c);
                 D01 += gc * (a0 - a1);
                 D02 += gc * (a0 - a2);
                 D12 += gc * (a1 - a2);
@@ -175,8 +175,8 @@ __device__ int det_pixel(const DetItem& it, const DetArgs& a, const float* __res
             float uk[3], vk[3];
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                uk[k] = __ldg(it.attr + (size_t)vid[k] * Ca + a.sh.uv_offset);
-                vk[k] = __ldg(it.attr + (size_t)vid[k] * Ca + a.sh.uv_offset + 1);
+                uk[k] = load(it.attr + (size_t)vid[k] * Ca + a.sh.uv_offset);
+                vk[k] = load(it.attr + (size_t)vid[k] * Ca + a.sh.uv_offset + 1);
             }
             const DTexCoord cx = tex_coord_f64(uk[0], uk[1], uk[2], b[1], b[2], a.sh.tex_w);
             const DTexCoord cy = tex_coord_f64(vk[0], vk[1], vk[2], b[1], b[2], a.sh.tex_h);
@@ -196,7 +196,7 @@ __device__ int det_pixel(const DetItem& it, const DetArgs& a, const float* __res
             }
         }
         const double GmG[3] = {b[1] * D01 + b[2] * D02, b[2] * D12 - b[0] * D01, -(b[0] * D02 + b[1] * D12)};
-        const double gZ = a.sh.depth_ch >= 0 ? (double)__ldg(gp + a.sh.depth_ch) : 0.0;
+        const double gZ = a.sh.depth_ch >= 0 ? (double)load(gp + a.sh.depth_ch) : 0.0;
         const double dz1 = z[1] - z[0], dz2 = z[2] - z[0];
         double wx = 0.0, wy = 0.0;
 #pragma unroll
@@ -227,7 +227,7 @@ __device__ int det_pixel(const DetItem& it, const DetArgs& a, const float* __res
             const int qx = x + ddx, qy = y + ddy;
             if (qx < 0 || qx >= it.W || qy < 0 || qy >= it.H) continue;  // no pair across the image border
             const size_t q = (size_t)qy * it.W + qx;
-            const int tq = __ldg(it.index + q);
+            const int tq = load(it.index + q);
             if (tq == t) continue;
             const int axis = ddx != 0 ? 0 : 1;
             bool inter = false;
@@ -240,7 +240,7 @@ __device__ int det_pixel(const DetItem& it, const DetArgs& a, const float* __res
                 int Xq[3], Yq[3];
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
-                    const int2 xy = __ldg(reinterpret_cast<const int2*>(it.vb + vq[k]));
+                    const int2 xy = load(reinterpret_cast<const int2*>(it.vb + vq[k]));
                     Xq[k] = xy.x;
                     Yq[k] = xy.y;
                 }
@@ -257,8 +257,8 @@ __device__ int det_pixel(const DetItem& it, const DetArgs& a, const float* __res
             const bool p_is_a = ddx > 0 || ddy > 0;
             double dLdp = 0.0;
             for (int c = 0; c < C; ++c) {
-                const double diff = (double)__ldg(ip + c) - (double)__ldg(iq + c);
-                dLdp += 0.5 * ((double)__ldg(gp + c) + (double)__ldg(gq + c)) * (p_is_a ? diff : -diff);
+                const double diff = (double)load(ip + c) - (double)load(iq + c);
+                dLdp += 0.5 * ((double)load(gp + c) + (double)load(gq + c)) * (p_is_a ? diff : -diff);
             }
             if (!inter) {
                 if (a.terms & MER_EXACT_CROSSING) {
@@ -363,12 +363,12 @@ __device__ __forceinline__ void det_warp_add(const DetItem& it, const DetArgs& a
 
 // Per-view launch: n views of one mesh, pixels of all views in order.
 template <bool ATTR>
-__global__ void __launch_bounds__(kDetThreads) k_backward_det(const mer_vertex* __restrict__ vpix,
-                                                              const int* __restrict__ tris, const int* __restrict__ index,
-                                                              const float* __restrict__ image,
-                                                              const float* __restrict__ grad,
-                                                              const float* __restrict__ attr,
-                                                              const float* __restrict__ tex, DetArgs a, int n, int H,
+__global__ void __launch_bounds__(kDetThreads) k_backward_det(const mer_vertex* vpix,
+                                                              const int* tris, const int* index,
+                                                              const float* image,
+                                                              const float* grad,
+                                                              const float* attr,
+                                                              const float* tex, DetArgs a, int n, int H,
                                                               int W, int V, int T, unsigned long long* acc_v,
                                                               unsigned long long* acc_a, void* ws) {
     after_previous();
@@ -396,14 +396,14 @@ __global__ void __launch_bounds__(kDetThreads) k_backward_det(const mer_vertex* 
 
 // Batched launch: the pixels of all items in order (item.pix).
 template <bool ATTR>
-__global__ void __launch_bounds__(kDetThreads) k_backward_det_batch(const mer_vertex* __restrict__ vpix,
-                                                                    const int* __restrict__ tris,
-                                                                    const mer_item* __restrict__ items, int n_items,
-                                                                    long long pixels, const int* __restrict__ index,
-                                                                    const float* __restrict__ image,
-                                                                    const float* __restrict__ grad,
-                                                                    const float* __restrict__ attr,
-                                                                    const float* __restrict__ tex, DetArgs a,
+__global__ void __launch_bounds__(kDetThreads) k_backward_det_batch(const mer_vertex* vpix,
+                                                                    const int* tris,
+                                                                    const mer_item* items, int n_items,
+                                                                    long long pixels, const int* index,
+                                                                    const float* image,
+                                                                    const float* grad,
+                                                                    const float* attr,
+                                                                    const float* tex, DetArgs a,
                                                                     unsigned long long* acc_v,
                                                                     unsigned long long* acc_a, void* ws) {
     after_previous();
@@ -434,9 +434,9 @@ __global__ void __launch_bounds__(kDetThreads) k_backward_det_batch(const mer_ve
 }
 
 // grad_vpix += the accumulated sums (FP64); grad_attr[:, a0 + j] += those of acc_a (rounded to FP32).
-__global__ void k_det_finalize(const unsigned long long* __restrict__ acc_v, long long nv, double* __restrict__ grad_vpix,
-                               const unsigned long long* __restrict__ acc_a, long long arows, int A, int a0, int Ca,
-                               float* __restrict__ grad_attr) {
+__global__ void k_det_finalize(const unsigned long long* acc_v, long long nv, double* grad_vpix,
+                               const unsigned long long* acc_a, long long arows, int A, int a0, int Ca,
+                               float* grad_attr) {
     after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < nv) grad_vpix[i] += fix_value((long long)acc_v[2 * i], (long long)acc_v[2 * i + 1]);

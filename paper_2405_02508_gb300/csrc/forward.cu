@@ -38,16 +38,16 @@ struct FwdArgs {
 };
 
 __device__ __forceinline__ bool fwd_tri_ids(const int* __restrict__ tris, int t, int V, int v[3]) {
-    v[0] = __ldg(tris + 3 * (size_t)t);
-    v[1] = __ldg(tris + 3 * (size_t)t + 1);
-    v[2] = __ldg(tris + 3 * (size_t)t + 2);
+    v[0] = load(tris + 3 * (size_t)t);
+    v[1] = load(tris + 3 * (size_t)t + 1);
+    v[2] = load(tris + 3 * (size_t)t + 2);
     return (unsigned)v[0] < (unsigned)V && (unsigned)v[1] < (unsigned)V && (unsigned)v[2] < (unsigned)V;
 }
 
 __device__ __forceinline__ void load_tangent(const float* __restrict__ tb, int v, float t[3]) {
-    t[0] = __ldg(tb + 3 * (size_t)v);
-    t[1] = __ldg(tb + 3 * (size_t)v + 1);
-    t[2] = __ldg(tb + 3 * (size_t)v + 2);
+    t[0] = load(tb + 3 * (size_t)v);
+    t[1] = load(tb + 3 * (size_t)v + 1);
+    t[2] = load(tb + 3 * (size_t)v + 2);
 }
 
 // Motion dr = sum_i lambda_i t_i of the fragment of triangle (vid, rv) at pixel (x, y).
@@ -78,7 +78,7 @@ __device__ __forceinline__ float overhang_rate(const VRec rv[3], const int vid[3
             const int ij = k == 0 ? vid[1] : (k == 1 ? vid[2] : vid[0]), il = k == 0 ? vid[2] : (k == 1 ? vid[0] : vid[1]);
             const float u = axis == 0 ? crossing_u(vj.Y, vj.ry, vl.Y, vl.ry, 256 * fy + 128)
                                       : crossing_u(vj.X, vj.rx, vl.X, vl.rx, 256 * fx + 128);
-            const float tj = __ldg(tb + 3 * (size_t)ij + axis), tl = __ldg(tb + 3 * (size_t)il + axis);
+            const float tj = load(tb + 3 * (size_t)ij + axis), tl = load(tb + 3 * (size_t)il + axis);
             return (1.0f - u) * tj + u * tl;
         }
     }
@@ -107,7 +107,7 @@ __device__ __forceinline__ bool covers_centre(const mer_vertex* __restrict__ vb,
     int X[3], Y[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {  // snapped position only: one 64-bit load per vertex
-        const int2 xy = __ldg(reinterpret_cast<const int2*>(vb + v[k]));
+        const int2 xy = load(reinterpret_cast<const int2*>(vb + v[k]));
         X[k] = xy.x;
         Y[k] = xy.y;
     }
@@ -120,14 +120,14 @@ constexpr int kNoRate = (int)0xffc0deadu;  // no rate: bits that arithmetic does
 constexpr int kFastC = 8;
 
 template <int FORM>
-__global__ void __launch_bounds__(kFTW * kFTH) k_forward_grad(const mer_vertex* __restrict__ vpix,
-                                                            const int* __restrict__ tris,
-                                                            const int* __restrict__ index,
-                                                            const float* __restrict__ image,
-                                                            const float* __restrict__ tangent,
-                                                            const float* __restrict__ attr,
-                                                            const float* __restrict__ tex, FwdArgs a,
-                                                            float* __restrict__ out, void* ws) {
+__global__ void __launch_bounds__(kFTW * kFTH) k_forward_grad(const mer_vertex* vpix,
+                                                            const int* tris,
+                                                            const int* index,
+                                                            const float* image,
+                                                            const float* tangent,
+                                                            const float* attr,
+                                                            const float* tex, FwdArgs a,
+                                                            float* out, void* ws) {
     after_previous();
     constexpr int kC = FORM == kGeneric ? kMaxC : kFastC;
     __shared__ int sidx[kFTH + 2][kFTW + 2];
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(kFTW * kFTH) k_forward_grad(const mer_vertex* 
     for (int i = ty * kFTW + tx; i < (kFTH + 2) * (kFTW + 2); i += kFTW * kFTH) {
         const int hy = i / (kFTW + 2), hx = i % (kFTW + 2);
         const int gx = blockIdx.x * kFTW + hx - 1, gy = blockIdx.y * kFTH + hy - 1;
-        sidx[hy][hx] = (gx >= 0 && gx < a.W && gy >= 0 && gy < a.H) ? __ldg(idx + (size_t)gy * a.W + gx) : -2;
+        sidx[hy][hx] = (gx >= 0 && gx < a.W && gy >= 0 && gy < a.H) ? load(idx + (size_t)gy * a.W + gx) : -2;
     }
     __syncthreads();
     const bool live = x < a.W && y < a.H;  // a row's lanes stay together for its list of pairs
@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(kFTW * kFTH) k_forward_grad(const mer_vertex* 
 #pragma unroll
             for (int c = 0; c < (FORM == kAttr3 ? 3 : kC); ++c) {
                 if (FORM == kGeneric && c >= a.sh.n_main) break;
-                const float a0 = __ldg(q0 + c), a1 = __ldg(q1 + c), a2 = __ldg(q2 + c);
+                const float a0 = load(q0 + c), a1 = load(q1 + c), a2 = load(q2 + c);
                 acc[c] += db[1] * (a1 - a0) + db[2] * (a2 - a0);  // sum_k db_k = 0
             }
         } else {
@@ -223,8 +223,8 @@ __global__ void __launch_bounds__(kFTW * kFTH) k_forward_grad(const mer_vertex* 
                     if (c >= a.sh.n_main) break;
                     const float* r0 = tex + (size_t)taps.j0 * a.sh.tex_w * a.tex_stride;
                     const float* r1 = tex + (size_t)taps.j1 * a.sh.tex_w * a.tex_stride;
-                    acc[c] += tap(__ldg(r0 + (size_t)taps.i0 * a.tex_stride + c), __ldg(r0 + (size_t)taps.i1 * a.tex_stride + c),
-                                  __ldg(r1 + (size_t)taps.i0 * a.tex_stride + c), __ldg(r1 + (size_t)taps.i1 * a.tex_stride + c));
+                    acc[c] += tap(load(r0 + (size_t)taps.i0 * a.tex_stride + c), load(r0 + (size_t)taps.i1 * a.tex_stride + c),
+                                  load(r1 + (size_t)taps.i0 * a.tex_stride + c), load(r1 + (size_t)taps.i1 * a.tex_stride + c));
                 }
             }
         }
@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(kFTW * kFTH) k_forward_grad(const mer_vertex* 
 #pragma unroll
             for (int c = 0; c < kC; ++c) {
                 if (c >= C) break;
-                acc[c] += 0.5f * (__ldg(ia + c) - __ldg(ib + c)) * rate;
+                acc[c] += 0.5f * (load(ia + c) - load(ib + c)) * rate;
             }
         }
     }
@@ -354,8 +354,8 @@ __global__ void __launch_bounds__(kFTW * kFTH) k_forward_grad(const mer_vertex* 
 
 // Tangent of the projected vertices for a world-space vertex tangent (shared by all views):
 // d(x_s, y_s, zeta) = J(X_c) R d(X_w), J as in the projection backward.
-__global__ void k_project_jvp(const float* __restrict__ tw, int V, const mer_camera* __restrict__ cams, int n,
-                              const mer_vertex* __restrict__ vpix, float* __restrict__ out) {
+__global__ void k_project_jvp(const float* tw, int V, const mer_camera* cams, int n,
+                              const mer_vertex* vpix, float* out) {
     after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (long long)V * n) return;

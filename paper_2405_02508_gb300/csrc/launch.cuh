@@ -4,9 +4,11 @@
 // device is idle for about a microsecond while the next grid is set up.  With programmatic stream serialization a grid is
 // set up as soon as all blocks of the one before it have started, and its blocks wait (after_previous) until that grid has
 // completed and its writes are visible.  Every kernel launched through launch_chained calls after_previous first, in all
-// its threads, so when a grid has completed, all grids before it have.  After anything else on the stream (a copy, another
-// library's kernel) such a launch starts as an ordinary one does.  Measured: a view of 40,960 triangles at 512 x 512 72.3 us a
-// pass with ordinary launches, 59.5 with these; three views at 333 x 517 84.6 and 73.7; 48 uneven meshes 1,792 and 1,757.
+// its threads, so when a grid has completed, all grids before it have.  Such a kernel runs at the same time as the writers of
+// what it reads, so it reads nothing as read-only data: no __restrict__ on its parameters, no __ldg (see load).
+// After anything else on the stream (a copy, another library's kernel) such a launch starts as an ordinary one does.
+// Measured: a view of 40,960 triangles at 512 x 512 72.3 us a pass with ordinary launches, 59.5 with these; three views at
+// 333 x 517 84.6 and 73.7; 48 uneven meshes 1,792 and 1,757.
 #pragma once
 
 #include <cuda_runtime.h>

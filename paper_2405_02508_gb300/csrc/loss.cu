@@ -10,8 +10,8 @@
 
 namespace mer {
 
-__global__ void k_l2_loss_grad(const float* __restrict__ image, const float* __restrict__ target, long long n,
-                               float* __restrict__ grad, double* __restrict__ loss) {
+__global__ void k_l2_loss_grad(const float* image, const float* target, long long n,
+                               float* grad, double* loss) {
     after_previous();
     __shared__ double sh[8];
     double acc = 0.0;

@@ -11,6 +11,15 @@
 
 namespace mer {
 
+// A plain load.  Kernels that overlap the one before them (launch.cuh) read global memory with these, through kernel parameters
+// without __restrict__: a read-only load (__ldg, or one that the compiler makes of a const __restrict__ parameter) is for data
+// that nothing writes while the kernel runs, so it may be moved ahead of the wait for the writer, and the kernel then reads
+// what was there before.
+template <typename T>
+__device__ __forceinline__ T load(const T* p) {
+    return *p;
+}
+
 constexpr int kMaxDim = 8192;
 constexpr double kGuard = 536870912.0;  // 2^29 (snapped units)
 constexpr uint32_t kValid = 3u;         // in front of the near plane and inside the guard band
@@ -293,8 +302,8 @@ struct VRec {
 };
 
 __device__ __forceinline__ VRec load_vrec(const mer_vertex* p) {
-    const float4 a = __ldg(reinterpret_cast<const float4*>(p));
-    const float2 b = __ldg(reinterpret_cast<const float2*>(p) + 2);
+    const float4 a = load(reinterpret_cast<const float4*>(p));
+    const float2 b = load(reinterpret_cast<const float2*>(p) + 2);
     VRec r;
     r.X = __float_as_int(a.x);
     r.Y = __float_as_int(a.y);
@@ -448,10 +457,10 @@ __device__ __forceinline__ TexQuad tex_quad(const float* __restrict__ tex, int T
     const float4* q = reinterpret_cast<const float4*>(tex);
     const unsigned r0 = (unsigned)t.j0 * (unsigned)TW, r1 = (unsigned)t.j1 * (unsigned)TW;
     TexQuad v;
-    v.a00 = __ldg(q + (r0 + (unsigned)t.i0));
-    v.a10 = __ldg(q + (r0 + (unsigned)t.i1));
-    v.a01 = __ldg(q + (r1 + (unsigned)t.i0));
-    v.a11 = __ldg(q + (r1 + (unsigned)t.i1));
+    v.a00 = load(q + (r0 + (unsigned)t.i0));
+    v.a10 = load(q + (r0 + (unsigned)t.i1));
+    v.a01 = load(q + (r1 + (unsigned)t.i0));
+    v.a11 = load(q + (r1 + (unsigned)t.i1));
     return v;
 }
 
@@ -460,12 +469,12 @@ __device__ __forceinline__ TexQuad tex_quad(const float* __restrict__ tex, int T
 __device__ __forceinline__ float4 texel4(const float* __restrict__ tex, int TW, int stride, bool vec4, int nc, int j,
                                          int i) {
     const float* q = tex + ((size_t)j * TW + i) * stride;
-    if (vec4) return __ldg(reinterpret_cast<const float4*>(q));
+    if (vec4) return load(reinterpret_cast<const float4*>(q));
     float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
-    r.x = __ldg(q);
-    if (nc > 1) r.y = __ldg(q + 1);
-    if (nc > 2) r.z = __ldg(q + 2);
-    if (nc > 3) r.w = __ldg(q + 3);
+    r.x = load(q);
+    if (nc > 1) r.y = load(q + 1);
+    if (nc > 2) r.z = load(q + 2);
+    if (nc > 3) r.w = load(q + 3);
     return r;
 }
 
@@ -503,8 +512,8 @@ __device__ __forceinline__ void tex_values(const float* __restrict__ tex, int TW
     const float* r0 = tex + (size_t)t.j0 * TW * stride;
     const float* r1 = tex + (size_t)t.j1 * TW * stride;
     for (int c = 0; c < nc; ++c) {
-        const float t00 = __ldg(r0 + (size_t)t.i0 * stride + c), t10 = __ldg(r0 + (size_t)t.i1 * stride + c);
-        const float t01 = __ldg(r1 + (size_t)t.i0 * stride + c), t11 = __ldg(r1 + (size_t)t.i1 * stride + c);
+        const float t00 = load(r0 + (size_t)t.i0 * stride + c), t10 = load(r0 + (size_t)t.i1 * stride + c);
+        const float t01 = load(r1 + (size_t)t.i0 * stride + c), t11 = load(r1 + (size_t)t.i1 * stride + c);
         out[c] = tex_lerp(t00, t10, t01, t11, t);
     }
 }
@@ -521,15 +530,15 @@ __device__ __forceinline__ void tex_grad_uv(const float* __restrict__ tex, int T
         for (int c = 0; c < 4; ++c) {
             if (c >= nc) break;
             const float t00 = comp(a00, c), t10 = comp(a10, c), t01 = comp(a01, c), t11 = comp(a11, c);
-            tex_lerp_grad(t00, t10, t01, t11, t, __ldg(g + c), su, sv);
+            tex_lerp_grad(t00, t10, t01, t11, t, load(g + c), su, sv);
         }
     } else {
         const float* r0 = tex + (size_t)t.j0 * TW * stride;
         const float* r1 = tex + (size_t)t.j1 * TW * stride;
         for (int c = 0; c < nc; ++c) {
-            const float t00 = __ldg(r0 + (size_t)t.i0 * stride + c), t10 = __ldg(r0 + (size_t)t.i1 * stride + c);
-            const float t01 = __ldg(r1 + (size_t)t.i0 * stride + c), t11 = __ldg(r1 + (size_t)t.i1 * stride + c);
-            tex_lerp_grad(t00, t10, t01, t11, t, __ldg(g + c), su, sv);
+            const float t00 = load(r0 + (size_t)t.i0 * stride + c), t10 = load(r0 + (size_t)t.i1 * stride + c);
+            const float t01 = load(r1 + (size_t)t.i0 * stride + c), t11 = load(r1 + (size_t)t.i1 * stride + c);
+            tex_lerp_grad(t00, t10, t01, t11, t, load(g + c), su, sv);
         }
     }
     gu = (float)TW * su;

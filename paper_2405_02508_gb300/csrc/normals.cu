@@ -31,8 +31,8 @@ __device__ __forceinline__ bool tri_fetch(const int* __restrict__ tris, long lon
     return (unsigned)v[0] < (unsigned)V && (unsigned)v[1] < (unsigned)V && (unsigned)v[2] < (unsigned)V;
 }
 
-__global__ void k_face_accumulate(const float* __restrict__ verts, const int* __restrict__ tris, long long T, int V,
-                                  float* __restrict__ acc, void* ws) {
+__global__ void k_face_accumulate(const float* verts, const int* tris, long long T, int V,
+                                  float* acc, void* ws) {
     after_previous();
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= T) return;
@@ -56,7 +56,7 @@ __global__ void k_face_accumulate(const float* __restrict__ verts, const int* __
         for (int c = 0; c < 3; ++c) atomicAdd(acc + 3 * (size_t)v[k] + c, fn[c]);
 }
 
-__global__ void k_normalize(const float* __restrict__ acc, long long V, float* __restrict__ out) {
+__global__ void k_normalize(const float* acc, long long V, float* out) {
     after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= V) return;
@@ -68,7 +68,7 @@ __global__ void k_normalize(const float* __restrict__ acc, long long V, float* _
 }
 
 // dL/da_v in place of dL/dn_v.
-__global__ void k_normalize_backward(const float* __restrict__ acc, long long V, float* __restrict__ g) {
+__global__ void k_normalize_backward(const float* acc, long long V, float* g) {
     after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= V) return;
@@ -89,8 +89,8 @@ __global__ void k_normalize_backward(const float* __restrict__ acc, long long V,
 
 // Face normal fn = e1 x e2 (e1 = p1 - p0, e2 = p2 - p0) with dL/dfn = sum of dL/da over its vertices:
 // dL/dp1 = e2 x G, dL/dp2 = G x e1, dL/dp0 = -(dL/dp1 + dL/dp2).
-__global__ void k_face_backward(const float* __restrict__ verts, const int* __restrict__ tris, long long T, int V,
-                                const float* __restrict__ ga, float* __restrict__ grad_verts, void* ws) {
+__global__ void k_face_backward(const float* verts, const int* tris, long long T, int V,
+                                const float* ga, float* grad_verts, void* ws) {
     after_previous();
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= T) return;

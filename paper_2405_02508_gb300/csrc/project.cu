@@ -62,8 +62,8 @@ __device__ __forceinline__ void project_one(const float* __restrict__ w, const m
 
 // out2 (optional): a second copy.  clear (optional): n_clear words set to zero (the raster's tile counts, which the next
 // kernel adds to: one launch less).
-__global__ void k_project(const float* __restrict__ verts, int V, const mer_camera* __restrict__ cams, int n,
-                          mer_vertex* __restrict__ out, mer_vertex* __restrict__ out2, int* __restrict__ clear,
+__global__ void k_project(const float* verts, int V, const mer_camera* cams, int n,
+                          mer_vertex* out, mer_vertex* out2, int* clear,
                           long long n_clear) {
     after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -73,9 +73,9 @@ __global__ void k_project(const float* __restrict__ verts, int V, const mer_came
     project_one(verts + 3 * (size_t)v, cams[view], out + i, out2 ? out2 + i : nullptr);
 }
 
-__global__ void k_project_batch(const float* __restrict__ verts, const mer_camera* __restrict__ cams,
-                                const mer_item* __restrict__ items, int n_items, long long vrecs,
-                                mer_vertex* __restrict__ out) {
+__global__ void k_project_batch(const float* verts, const mer_camera* cams,
+                                const mer_item* items, int n_items, long long vrecs,
+                                mer_vertex* out) {
     after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int k = warp_find_item(items, n_items, i - (threadIdx.x & 31), i, kFieldVrec);
@@ -84,7 +84,7 @@ __global__ void k_project_batch(const float* __restrict__ verts, const mer_camer
     project_one(verts + 3 * (size_t)(m.vert + (i - m.vrec)), cams[m.cam], out + i);
 }
 
-__global__ void k_project_screen(const double* __restrict__ scr, int V, int n, mer_vertex* __restrict__ out) {
+__global__ void k_project_screen(const double* scr, int V, int n, mer_vertex* out) {
     after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (long long)V * n) return;
@@ -145,9 +145,9 @@ __device__ __forceinline__ bool world_grad_f64(const mer_vertex& r, const mer_ca
 }
 
 // Batched: one thread per (item, vertex); items sharing a mesh add into the same rows.
-__global__ void k_project_backward_batch(const mer_camera* __restrict__ cams, const mer_item* __restrict__ items,
-                                         int n_items, long long vrecs, const mer_vertex* __restrict__ vpix,
-                                         const double* __restrict__ grad_vpix, float* __restrict__ grad_verts) {
+__global__ void k_project_backward_batch(const mer_camera* cams, const mer_item* items,
+                                         int n_items, long long vrecs, const mer_vertex* vpix,
+                                         const double* grad_vpix, float* grad_verts) {
     after_previous();
     __shared__ CameraF s_cam[8];  // of each warp's first item, converted by its lanes together
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -178,9 +178,9 @@ __global__ void k_project_backward_batch(const mer_camera* __restrict__ cams, co
 // Batched, reproducible: FP64 products rounded once to fixed point with 52 fractional bits, held as two
 // 64-bit words (hi = floor(w 2^20), lo = the remainder in units of 2^-52, in [0, 2^32]), and added with
 // integer atomics into acc [mesh rows, 3, 2] (exact, so the order does not matter); k_world_finalize converts.
-__global__ void k_project_backward_batch_fixed(const mer_camera* __restrict__ cams, const mer_item* __restrict__ items,
-                                               int n_items, long long vrecs, const mer_vertex* __restrict__ vpix,
-                                               const double* __restrict__ grad_vpix, unsigned long long* acc,
+__global__ void k_project_backward_batch_fixed(const mer_camera* cams, const mer_item* items,
+                                               int n_items, long long vrecs, const mer_vertex* vpix,
+                                               const double* grad_vpix, unsigned long long* acc,
                                                void* ws) {
     after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -204,7 +204,7 @@ __global__ void k_project_backward_batch_fixed(const mer_camera* __restrict__ ca
     }
 }
 
-__global__ void k_world_finalize(const unsigned long long* __restrict__ acc, long long n, float* __restrict__ grad_verts) {
+__global__ void k_world_finalize(const unsigned long long* acc, long long n, float* grad_verts) {
     after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -216,9 +216,9 @@ __global__ void k_world_finalize(const unsigned long long* __restrict__ acc, lon
 // One thread per vertex, looping over the views: grad_world = sum_views R^T J^T g (FP64).  STORE: overwrite grad_verts (and
 // the second copy) instead of adding to it.
 template <bool STORE>
-__global__ void k_project_backward(int V, const mer_camera* __restrict__ cams, int n,
-                                   const mer_vertex* __restrict__ vpix, const double* __restrict__ grad_vpix,
-                                   float* __restrict__ grad_verts, float* __restrict__ copy) {
+__global__ void k_project_backward(int V, const mer_camera* cams, int n,
+                                   const mer_vertex* vpix, const double* grad_vpix,
+                                   float* grad_verts, float* copy) {
     after_previous();
     const int v = blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= V) return;
@@ -301,7 +301,7 @@ extern "C" int mer_launch_project_backward_batch(const mer_camera* cams, const m
 }
 
 namespace mer {
-__global__ void k_clear(double* __restrict__ a, long long na, float* __restrict__ b, long long nb) {
+__global__ void k_clear(double* a, long long na, float* b, long long nb) {
     after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < na) a[i] = 0.0;

@@ -75,8 +75,8 @@ __device__ __forceinline__ void setup_count_one(const RItem& it, int t, int tile
     float zeta[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {  // the 32-byte vertex record as two 128-bit loads (records are 32-byte aligned)
-        const float4 a = __ldg(reinterpret_cast<const float4*>(it.vpix + vid[k]));
-        const float4 b = __ldg(reinterpret_cast<const float4*>(it.vpix + vid[k]) + 1);
+        const float4 a = load(reinterpret_cast<const float4*>(it.vpix + vid[k]));
+        const float4 b = load(reinterpret_cast<const float4*>(it.vpix + vid[k]) + 1);
         if ((__float_as_uint(b.z) & kValid) != kValid) ok = false;  // flags
         r.X[k] = __float_as_int(a.x);
         r.Y[k] = __float_as_int(a.y);
@@ -202,7 +202,7 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* sh, int& total) 
     return before + x - v;
 }
 
-__global__ void k_scan_blocks(const int* __restrict__ in, long long N, int* __restrict__ out, int* __restrict__ sums) {
+__global__ void k_scan_blocks(const int* in, long long N, int* out, int* sums) {
     after_previous();
     __shared__ int sh[32];
     const long long i = (long long)blockIdx.x * kScanBlock + threadIdx.x;
@@ -214,7 +214,7 @@ __global__ void k_scan_blocks(const int* __restrict__ in, long long N, int* __re
 }
 
 // Single CTA: exclusive scan of the block sums (looping), total written to the header.
-__global__ void k_scan_sums(int* __restrict__ sums, int nb, void* ws, long long capacity) {
+__global__ void k_scan_sums(int* sums, int nb, void* ws, long long capacity) {
     after_previous();
     __shared__ int sh[32];
     int carry = 0;
@@ -236,7 +236,7 @@ __global__ void k_scan_sums(int* __restrict__ sums, int nb, void* ws, long long 
 }
 
 // Adds the block offsets and clears the front and back fill cursors (cursor[0, 2N)).
-__global__ void k_scan_add(int* __restrict__ out, long long N, const int* __restrict__ sums, int* __restrict__ cursor) {
+__global__ void k_scan_add(int* out, long long N, const int* sums, int* cursor) {
     after_previous();
     const long long i = (long long)blockIdx.x * kScanBlock + threadIdx.x;
     if (i < N) {
@@ -252,8 +252,8 @@ __global__ void k_scan_add(int* __restrict__ out, long long N, const int* __rest
 constexpr int kScanEach = 16;
 constexpr long long kHostReady = 1LL << 32;
 
-__global__ void __launch_bounds__(kScanBlock) k_scan_all(const int* __restrict__ in, int N, int* __restrict__ out,
-                                                         int* __restrict__ cursor, void* ws, long long capacity,
+__global__ void __launch_bounds__(kScanBlock) k_scan_all(const int* in, int N, int* out,
+                                                         int* cursor, void* ws, long long capacity,
                                                          volatile long long* host) {
     after_previous();
     __shared__ int sh[32];
@@ -556,8 +556,8 @@ __device__ __forceinline__ RItem view_item(const BinGeom& g, const mer_vertex* v
     return it;
 }
 
-__global__ void k_setup_count(const mer_vertex* __restrict__ vpix, const int* __restrict__ tris, BinGeom g,
-                              TriRaster* __restrict__ recs, int* __restrict__ counts, void* ws) {
+__global__ void k_setup_count(const mer_vertex* vpix, const int* tris, BinGeom g,
+                              TriRaster* recs, int* counts, void* ws) {
     after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (long long)g.T * g.n) return;
@@ -565,9 +565,9 @@ __global__ void k_setup_count(const mer_vertex* __restrict__ vpix, const int* __
     setup_count_one(view_item(g, vpix, tris, recs, view), t, g.tile, counts, ws);
 }
 
-__global__ void k_bin_fill(const mer_vertex* __restrict__ vpix, const int* __restrict__ tris, BinGeom g,
-                           TriRaster* __restrict__ recs, const int* __restrict__ offs, const int* __restrict__ counts,
-                           int* __restrict__ cursor, int* __restrict__ list, long long capacity) {
+__global__ void k_bin_fill(const mer_vertex* vpix, const int* tris, BinGeom g,
+                           TriRaster* recs, const int* offs, const int* counts,
+                           int* cursor, int* list, long long capacity) {
     after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (long long)g.T * g.n) return;
@@ -577,13 +577,13 @@ __global__ void k_bin_fill(const mer_vertex* __restrict__ vpix, const int* __res
 }
 
 template <int TS, int FORM, bool DUAL>
-__global__ void __launch_bounds__(kRasterThreads, kRasterCtasPerSm) k_raster(TriRaster* __restrict__ recs, BinGeom g,
-                                                           const int* __restrict__ offs, const int* __restrict__ cnts,
-                                                           const int* __restrict__ nfront,
-                                                           const int* __restrict__ list, const mer_vertex* __restrict__ vpix,
-                                                           const int* __restrict__ tris, void* ws, long long capacity,
-                                                           int* __restrict__ index, float* __restrict__ depth,
-                                                           float* __restrict__ bary, unsigned char* __restrict__ cover,
+__global__ void __launch_bounds__(kRasterThreads, kRasterCtasPerSm) k_raster(TriRaster* recs, BinGeom g,
+                                                           const int* offs, const int* cnts,
+                                                           const int* nfront,
+                                                           const int* list, const mer_vertex* vpix,
+                                                           const int* tris, void* ws, long long capacity,
+                                                           int* index, float* depth,
+                                                           float* bary, unsigned char* cover,
                                                            ShadeOut so) {
     after_previous();
     __shared__ RasterShared<TS> S;
@@ -618,8 +618,8 @@ __device__ __forceinline__ RItem batch_item(const mer_item& m, int tile, const m
     return it;
 }
 
-__global__ void k_setup_count_batch(const mer_vertex* __restrict__ vpix, const int* __restrict__ tris, BatchGeom b,
-                                    TriRaster* __restrict__ recs, int* __restrict__ counts, void* ws) {
+__global__ void k_setup_count_batch(const mer_vertex* vpix, const int* tris, BatchGeom b,
+                                    TriRaster* recs, int* counts, void* ws) {
     after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int k = warp_find_item(b.items, b.n_items, i - (threadIdx.x & 31), i, kFieldTrec);
@@ -628,9 +628,9 @@ __global__ void k_setup_count_batch(const mer_vertex* __restrict__ vpix, const i
     setup_count_one(batch_item(m, b.tile, vpix, tris, recs), (int)(i - m.trec), b.tile, counts, ws);
 }
 
-__global__ void k_bin_fill_batch(const mer_vertex* __restrict__ vpix, const int* __restrict__ tris, BatchGeom b,
-                                 TriRaster* __restrict__ recs, const int* __restrict__ offs,
-                                 const int* __restrict__ counts, int* __restrict__ cursor, int* __restrict__ list,
+__global__ void k_bin_fill_batch(const mer_vertex* vpix, const int* tris, BatchGeom b,
+                                 TriRaster* recs, const int* offs,
+                                 const int* counts, int* cursor, int* list,
                                  long long capacity) {
     after_previous();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -643,16 +643,16 @@ __global__ void k_bin_fill_batch(const mer_vertex* __restrict__ vpix, const int*
 
 // Persistent: each CTA takes the next global tile from the work queue until none is left.
 template <int TS, int FORM>
-__global__ void __launch_bounds__(kRasterThreads, kRasterCtasPerSm) k_raster_batch(TriRaster* __restrict__ recs, BatchGeom b,
-                                                                 const int* __restrict__ offs,
-                                                                 const int* __restrict__ cnts,
-                                                                 const int* __restrict__ nfront,
-                                                                 const int* __restrict__ list,
-                                                                 const mer_vertex* __restrict__ vpix,
-                                                                 const int* __restrict__ tris, void* ws,
-                                                                 long long capacity, int* __restrict__ index,
-                                                                 float* __restrict__ depth, float* __restrict__ bary,
-                                                                 unsigned char* __restrict__ cover, ShadeOut so) {
+__global__ void __launch_bounds__(kRasterThreads, kRasterCtasPerSm) k_raster_batch(TriRaster* recs, BatchGeom b,
+                                                                 const int* offs,
+                                                                 const int* cnts,
+                                                                 const int* nfront,
+                                                                 const int* list,
+                                                                 const mer_vertex* vpix,
+                                                                 const int* tris, void* ws,
+                                                                 long long capacity, int* index,
+                                                                 float* depth, float* bary,
+                                                                 unsigned char* cover, ShadeOut so) {
     after_previous();
     __shared__ RasterShared<TS> S;
     __shared__ long long s_tile;

@@ -27,9 +27,9 @@ __device__ __forceinline__ void shade_pixel(const mer_vertex* __restrict__ vb, i
 }
 
 template <int FORM>
-__global__ void k_shade(const mer_vertex* __restrict__ vpix, int V, const int* __restrict__ tris, int T, int n, int H,
-                        int W, const int* __restrict__ index, const float* __restrict__ attr,
-                        const float* __restrict__ tex, ShadeArgs a, float* __restrict__ image, void* ws) {
+__global__ void k_shade(const mer_vertex* vpix, int V, const int* tris, int T, int n, int H,
+                        int W, const int* index, const float* attr,
+                        const float* tex, ShadeArgs a, float* image, void* ws) {
     after_previous();
     const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long npix = (long long)n * H * W;
@@ -40,10 +40,10 @@ __global__ void k_shade(const mer_vertex* __restrict__ vpix, int V, const int* _
 }
 
 template <int FORM>
-__global__ void k_shade_batch(const mer_vertex* __restrict__ vpix, const int* __restrict__ tris,
-                              const mer_item* __restrict__ items, int n_items, long long pixels,
-                              const int* __restrict__ index, const float* __restrict__ attr,
-                              const float* __restrict__ tex, ShadeArgs a, float* __restrict__ image, void* ws) {
+__global__ void k_shade_batch(const mer_vertex* vpix, const int* tris,
+                              const mer_item* items, int n_items, long long pixels,
+                              const int* index, const float* attr,
+                              const float* tex, ShadeArgs a, float* image, void* ws) {
     after_previous();
     const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int k = warp_find_item(items, n_items, p - (threadIdx.x & 31), p, kFieldPix);

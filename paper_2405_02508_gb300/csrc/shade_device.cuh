@@ -51,12 +51,12 @@ __device__ __forceinline__ void load_uv(const float* __restrict__ attr, int Ca, 
     for (int k = 0; k < 3; ++k) {
         const float* q = attr + ((long long)vid[k] * Ca + uv_offset);
         if (FORM == kTex3) {
-            const float2 uv = __ldg(reinterpret_cast<const float2*>(q));
+            const float2 uv = load(reinterpret_cast<const float2*>(q));
             uk[k] = uv.x;
             vk[k] = uv.y;
         } else {
-            uk[k] = __ldg(q);
-            vk[k] = __ldg(q + 1);
+            uk[k] = load(q);
+            vk[k] = load(q + 1);
         }
     }
 }
@@ -117,7 +117,7 @@ __device__ __forceinline__ void shade_fragment(const mer_vertex* __restrict__ vb
         for (int k = 0; k < 3; ++k) {
             const float* q = attr + (long long)vid[k] * Ca;
 #pragma unroll
-            for (int c = 0; c < 3; ++c) acc[c] += b[k] * __ldg(q + c);
+            for (int c = 0; c < 3; ++c) acc[c] += b[k] * load(q + c);
         }
 #pragma unroll
         for (int c = 0; c < 3; ++c) put(c, acc[c]);
@@ -125,7 +125,7 @@ __device__ __forceinline__ void shade_fragment(const mer_vertex* __restrict__ vb
         for (int c = 0; c < a.sh.n_main; ++c) {
             float acc = 0.f;
 #pragma unroll
-            for (int k = 0; k < 3; ++k) acc += b[k] * __ldg(attr + (size_t)vid[k] * Ca + c);
+            for (int k = 0; k < 3; ++k) acc += b[k] * load(attr + (size_t)vid[k] * Ca + c);
             put(c, acc);
         }
     } else {
@@ -252,7 +252,7 @@ __device__ __forceinline__ DTexTaps tex_taps_f64(int TH, int TW, DTexCoord cx, D
 }
 
 __device__ __forceinline__ double texel_f64(const float* __restrict__ tex, int TW, int stride, int j, int i, int c) {
-    return (double)__ldg(tex + ((size_t)j * TW + i) * stride + c);
+    return (double)load(tex + ((size_t)j * TW + i) * stride + c);
 }
 
 // Bilinear value of channel c in FP64.
@@ -273,7 +273,7 @@ __device__ __forceinline__ void tex_grad_uv_f64(const float* __restrict__ tex, i
     for (int c = 0; c < nc; ++c) {
         const double t00 = texel_f64(tex, TW, stride, t.j0, t.i0, c), t10 = texel_f64(tex, TW, stride, t.j0, t.i1, c);
         const double t01 = texel_f64(tex, TW, stride, t.j1, t.i0, c), t11 = texel_f64(tex, TW, stride, t.j1, t.i1, c);
-        const double gc = (double)__ldg(g + c);
+        const double gc = (double)load(g + c);
         su += gc * ((1.0 - t.fy) * (t10 - t00) + t.fy * (t11 - t01));
         const double a = t00 + t.fx * (t10 - t00);
         const double b = t01 + t.fx * (t11 - t01);
@@ -319,15 +319,15 @@ __device__ __forceinline__ void shade_fragment_f64(const mer_vertex* __restrict_
         for (int c = 0; c < a.sh.n_main; ++c) {
             double acc = 0.0;
 #pragma unroll
-            for (int k = 0; k < 3; ++k) acc += b[k] * (double)__ldg(attr + (size_t)vid[k] * Ca + c);
+            for (int k = 0; k < 3; ++k) acc += b[k] * (double)load(attr + (size_t)vid[k] * Ca + c);
             o[c] = __double2float_rn(acc);
         }
     } else {
         float uk[3], vk[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            uk[k] = __ldg(attr + (size_t)vid[k] * Ca + a.sh.uv_offset);
-            vk[k] = __ldg(attr + (size_t)vid[k] * Ca + a.sh.uv_offset + 1);
+            uk[k] = load(attr + (size_t)vid[k] * Ca + a.sh.uv_offset);
+            vk[k] = load(attr + (size_t)vid[k] * Ca + a.sh.uv_offset + 1);
         }
         const DTexCoord cx = tex_coord_f64(uk[0], uk[1], uk[2], b[1], b[2], a.sh.tex_w);
         const DTexCoord cy = tex_coord_f64(vk[0], vk[1], vk[2], b[1], b[2], a.sh.tex_h);
