@@ -316,11 +316,17 @@ __device__ __forceinline__ void shade_fragment_f64(const mer_vertex* __restrict_
     for (int k = 0; k < 3; ++k) b[k] = B.lam[k] * z[k] * is;
     const int Ca = a.sh.C_attr;
     if (a.sh.uv_offset < 0) {
-        for (int c = 0; c < a.sh.n_main; ++c) {
-            double acc = 0.0;
+        for (int c0 = 0; c0 < a.sh.n_main; c0 += 4) {  // four channels' loads in flight
+            double acc[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-            for (int k = 0; k < 3; ++k) acc += b[k] * (double)load(attr + (size_t)vid[k] * Ca + c);
-            o[c] = __double2float_rn(acc);
+            for (int j = 0; j < 4; ++j) {
+                if (c0 + j >= a.sh.n_main) break;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) acc[j] += b[k] * (double)load(attr + (size_t)vid[k] * Ca + (c0 + j));
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (c0 + j < a.sh.n_main) o[c0 + j] = __double2float_rn(acc[j]);
         }
     } else {
         float uk[3], vk[3];
@@ -332,8 +338,15 @@ __device__ __forceinline__ void shade_fragment_f64(const mer_vertex* __restrict_
         const DTexCoord cx = tex_coord_f64(uk[0], uk[1], uk[2], b[1], b[2], a.sh.tex_w);
         const DTexCoord cy = tex_coord_f64(vk[0], vk[1], vk[2], b[1], b[2], a.sh.tex_h);
         const DTexTaps taps = tex_taps_f64(a.sh.tex_h, a.sh.tex_w, cx, cy);
-        for (int c = 0; c < a.sh.n_main && c < kMaxC; ++c)
-            o[c] = __double2float_rn(tex_value_f64(tex, a.sh.tex_w, a.tex_stride, taps, c));
+        for (int c0 = 0; c0 < a.sh.n_main; c0 += 4) {
+            double value[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (c0 + j < a.sh.n_main) value[j] = tex_value_f64(tex, a.sh.tex_w, a.tex_stride, taps, c0 + j);
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (c0 + j < a.sh.n_main) o[c0 + j] = __double2float_rn(value[j]);
+        }
     }
     if (a.sh.mask_ch >= 0) o[a.sh.mask_ch] = 1.0f;
     if (a.sh.depth_ch >= 0) o[a.sh.depth_ch] = __double2float_rn(is);
