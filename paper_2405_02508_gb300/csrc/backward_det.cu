@@ -390,9 +390,10 @@ __global__ void __launch_bounds__(kDetThreads) k_backward_det(const mer_vertex* 
     det_warp_add<ATTR>(it, a, view, t, vid, cv, ca);
 }
 
-// Batched launch: the pixels of all items in order (item.pix).
+// Batched launch: the pixels of all items in order (item.pix).  512 threads an SM, 128 registers each: with attribute gradients
+// it would take 151, and one block fewer (256 meshes at 64 x 64 with three interpolated channels: 966 us, now 836).
 template <bool ATTR>
-__global__ void __launch_bounds__(kDetThreads) k_backward_det_batch(const mer_vertex* vpix,
+__global__ void __launch_bounds__(kDetThreads, 512 / kDetThreads) k_backward_det_batch(const mer_vertex* vpix,
                                                                     const int* tris,
                                                                     const mer_item* items, int n_items,
                                                                     long long pixels, const int* index,
