@@ -200,13 +200,19 @@ __global__ void k_cg_next(CgState* st) {
 // two-float arithmetic, about 48 bits against FP64's 53, and so are the iteration's two quotients before they are rounded to
 // the FP32 factors alpha and beta.  GB300's FP64 pipe issues one warp instruction in 16 cycles, and the 64-bit sums and
 // divisions took longer than the exchanges (9 us an iteration of 258 rows, now 2.8).  The vectors are FP32, so the five bits
-// are far below what a solve can show: in 576 solves of 258 to 211,602 rows (lambda 8, 16 and 32, rough, smooth and mixed
+// are far below what a solve can show: in 576 solves of 258 to 211,602 rows of at most 8 neighbours (lambda 8, 16 and 32, rough, smooth and mixed
 // right-hand sides, cold and warm starts) iterations and solutions had the same bits as the launch sequence, whose sums
 // are FP64, hence the same errors against a 64-bit solution.
 // Measured (lambda 16, residual 1e-6, 79 and 49 iterations): 65,538 rows 3,520 -> 612 us, 642 rows 2,350 -> 155 us.
 constexpr int kCgThreads = 512;         // per CTA of the cluster form (one CTA per SM, up to 128 registers a thread)
 constexpr int kCgLocalThreads = 1024;   // the single-CTA form
 constexpr int kCgNeighbours = 8;        // neighbour ids kept in registers (a closed mesh averages 6)
+// Rows with more neighbours than this (the poles of a sphere of meridians, the hub of a fan) are summed by their warp, 32
+// neighbours at a time (hub_sums): one thread going through them, each a trip to L2 and back, held up every iteration of the
+// whole solve.  A sphere of 64 x 1,024 quads 21,455 us (the launches 12,852), now 1,430; one of 200 x 1,024 22,600 (13,930) and
+// 3,550; a fan of 5,000 28,360 (15,620) and 900.  (In the one-CTA form the trip is to shared memory: a fan of 900 478, the
+// launches 4,104.)
+constexpr int kCgHub = 64;
 constexpr unsigned kCgPolls = 1u << 21;  // polls of one exchange (about a second) before the solve gives up
 constexpr int kCgCluster = 8;           // CTAs of a cluster
 constexpr int kCgMaxClusters = 32;      // one slot per lane of a warp
@@ -378,6 +384,40 @@ __device__ __forceinline__ void cg_sum(T v, unsigned step, CgSlot* slots, unsign
     cluster_sync();
 }
 
+// Sums over the neighbours beyond kCgNeighbours of the rows of a warp's lanes that have more than kCgHub, each by all the
+// lanes of mask m (the first ones of the warp); zero for the other lanes.  Out of line: inlined, its registers cost every
+// iteration of every solve 2 to 4 % (now below 1 %; 7 % in the form of four rows a thread, which spills).
+__device__ __noinline__ float4 hub_sums(const int32_t* col, int64_t first, int deg, const float4* r, const float4* p, float beta,
+                                        unsigned m) {
+    const int lane = threadIdx.x & 31, lanes = __popc(m);
+    float4 mine = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (unsigned hubs = __ballot_sync(m, deg > kCgHub); hubs; hubs &= hubs - 1) {
+        const int src = __ffs((int)hubs) - 1;
+        const long long f = __shfl_sync(m, (long long)first, src);
+        const int n = __shfl_sync(m, deg, src);
+        float s[3] = {0.f, 0.f, 0.f};
+#pragma unroll 4
+        for (int j = kCgNeighbours + lane; j < n; j += lanes) {
+            const int q = __ldg(col + f + j);
+            const float4 a = cg_load(r + q), o = cg_load(p + q);
+            s[0] += a.x + beta * o.x;
+            s[1] += a.y + beta * o.y;
+            s[2] += a.z + beta * o.z;
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const float v = __shfl_down_sync(m, s[c], o);
+                if (lane + o < lanes) s[c] += v;
+            }
+            s[c] = __shfl_sync(m, s[c], 0);
+        }
+        if (lane == src) mine = make_float4(s[0], s[1], s[2], 0.f);
+    }
+    return mine;
+}
+
 // a / b rounded to a float, for two-float a and b > 0: the correctly rounded quotient of the high parts and one
 // correction with the exact remainder.
 __device__ __forceinline__ float f2_ratio(F2 a, F2 b) {
@@ -458,6 +498,12 @@ __global__ void __launch_bounds__(CLUSTER ? kCgThreads : kCgLocalThreads, 1)
     const float scale = S.coef;
     float beta = 0.f;
     int it = 0;
+    bool hub = false;  // a lane of the warp has a row for hub_sums
+    if (CLUSTER) {
+#pragma unroll
+        for (int k = 0; k < R; ++k) hub |= deg[k] > kCgHub;
+        hub = __any_sync(0xffffffffu, hub);
+    }
     while (!S.stop && it < max_iters) {
         // p = r + beta p for the row and its neighbours, M p, p . M p
         const float4 *p_old = p_ws + (size_t)(it & 1) * V, *ps_old = sm + kN + (it & 1) * kN;
@@ -465,6 +511,7 @@ __global__ void __launch_bounds__(CLUSTER ? kCgThreads : kCgLocalThreads, 1)
         F2 d = {0.f, 0.f};
 #pragma unroll
         for (int k = 0; k < R; ++k) {
+            const unsigned have = CLUSTER && hub ? __ballot_sync(0xffffffffu, row[k] >= 0) : 0u;
             if (row[k] < 0) continue;
             float4 nr[kCgNeighbours], np[kCgNeighbours];
 #pragma unroll
@@ -488,7 +535,15 @@ __global__ void __launch_bounds__(CLUSTER ? kCgThreads : kCgLocalThreads, 1)
                     sz += pz;
                 }
             }
-            for (int j = kCgNeighbours; j < deg[k]; ++j) {
+            int end = deg[k];
+            if (CLUSTER && hub) {
+                const float4 h = hub_sums(col, first[k], deg[k], r_ws, p_old, beta, have);
+                sx += h.x;
+                sy += h.y;
+                sz += h.z;
+                if (end > kCgHub) end = 0;
+            }
+            for (int j = kCgNeighbours; j < end; ++j) {
                 const int q = __ldg(col + first[k] + j);
                 const float4 a = CLUSTER ? cg_load(r_ws + q) : sm[q], o = CLUSTER ? cg_load(p_old + q) : ps_old[q];
                 sx += a.x + beta * o.x;
@@ -686,8 +741,8 @@ extern "C" int mer_launch_precond_solve(const int64_t* row_ptr, const int32_t* c
     // One CTA up to its 1,024 threads (902 rows: 3.9 us an iteration, the same as a cluster; 258 rows: 2.8 against 4.0).
     // One cluster, with two rows a thread where that saves the exchange between clusters (6,402 rows: 5.4 against 6.4 us).
     // Then the fewest rows a thread whose clusters all fit on the device (16 clusters of 8 with one CTA per SM): 32,402
-    // rows 6.9 us with one row, 7.9 with two; 65,538 rows 7.8 us with two; 131,046 rows 11.7 us with four, although that
-    // form spills, 211,602 rows 12.6 (the launches 52 and 57).  Larger systems, which one grid cannot hold,
+    // rows 6.9 us with one row, 7.9 with two; 65,538 rows 7.8 us with two; 131,046 rows 12.5 us with four, although that
+    // form spills, 211,602 rows 13.3 (the launches 52 and 57).  Larger systems, which one grid cannot hold,
     // and devices without room take the launches, 36-60 us an iteration up to 262,146 rows, 91 at 620,946.
     constexpr int64_t kClusterRows = kCgCluster * kCgThreads;
     cudaError_t e = cudaErrorNotSupported;
