@@ -339,6 +339,9 @@ constexpr int kRasterThreads = 256;
 // smallest 15.8 / 88.3 / 2,120.
 constexpr int kTinyPx = 8;     // boxes of at most this many pixels: 2 lanes each
 constexpr int kSmallPx = 64;   // of at most this many: 8 lanes each; larger ones: a warp
+// In tiles of 8 x 8 every box is small, and with one to eight of them in a tile a warp each is faster: 512 triangles at
+// 1024 x 1024 404 us a pass with 8 lanes (365 with a warp for each triangle whatever its box), 344 so; 2,048 there 222 (203)
+// and 186; 131,072 there 144 (149) and 136.  In tiles of 16 no difference above 1 % but at 300 x 400 (50.7 and 48.4).
 // Resident CTAs per SM: 48 registers a thread, and a stage of the 64 x 64 tile small enough that its shared memory allows
 // five.  32 head views (tile 64) 1,855 us with four and 64 registers, 1,780 with five; 48 uneven meshes (tile 32) 651 and 586,
 // 588 with six at 40 registers; 8 views at 512 x 512 (tile 32) 78, 75 and 84.
@@ -504,7 +507,11 @@ __device__ __forceinline__ void raster_tile(const RItem& it, int local_tile, con
         }
         __syncthreads();
         raster_class<TS, 2, 32>(S, it.recs, n_todo[2], ox, oy, back, cover != nullptr);
-        raster_class<TS, 1, 8>(S, it.recs, n_todo[1], ox, oy, back, cover != nullptr);
+        // small tiles with few records: a warp each is at least as many lanes, and a quarter of the passes
+        if (TS <= 16 && n_todo[1] <= kRasterThreads / 32)
+            raster_class<TS, 1, 32>(S, it.recs, n_todo[1], ox, oy, back, cover != nullptr);
+        else
+            raster_class<TS, 1, 8>(S, it.recs, n_todo[1], ox, oy, back, cover != nullptr);
         raster_class<TS, 0, 2>(S, it.recs, n_todo[0], ox, oy, back, cover != nullptr);
     }
     __syncthreads();
