@@ -118,8 +118,8 @@ class ClockSampler:
 # one k_backward_batch launch, from an ncu capture of the same workload at 4 views (inputs already larger than
 # L2), per pixel of the launch, with the sha256 of the kernel's sources they were taken on: a launch of n views
 # moves / issues n*H*W times these.  They are reported only while the sources are unchanged.
-BACKWARD_TRAFFIC = {"bytes_per_pixel": 23.7104, "warp_instructions_per_pixel": 22.9500,
-                    "sources_sha256": "8d555ee5f28b14e4a4819876b9f0754fc3b945b1c685974725f0505e4b70e9ca",
+BACKWARD_TRAFFIC = {"bytes_per_pixel": 23.8159, "warp_instructions_per_pixel": 23.5593,
+                    "sources_sha256": "fcb92dc0c7870cbcb79baad832af67965261b36144d1c775ea96e4f46d35317e",
                     "profile": "profiles/ncu_head_4x1334x2048.md"}
 
 

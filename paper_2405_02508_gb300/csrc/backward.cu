@@ -31,14 +31,14 @@ constexpr int kTW = kBwdTileW, kTH = kBwdTileH;  // tile: 8 warps, two rows each
 constexpr int kRows = 2;                          // rows per warp
 constexpr int kHW = kTW + 2, kHH = kTH + 2;
 constexpr int kThreads = 256;
-// Resident CTAs per SM, at most 51 registers a thread.  32 head views 2,354 us with six (42 registers) and 2,320 with five,
+// Resident CTAs per SM (48 registers a thread).  32 head views 2,354 us with six (40 registers) and 2,320 with five,
 // 2,410 with four, once the tile's place and item were kept in shared memory; 8 views at 512 x 512 75.4, 71.9 and 72.2; 48
 // uneven meshes with attribute gradients 638, 637 and 688.  A per-view launch (three views at 333 x 517) 19.6, 17.5 and 16.5;
 // 1024 x 1024 with attribute gradients 52.4, 48.3 and 48.9.
 constexpr int kCtasPerSm = 5;
 static_assert(kTW == 32 && kTH == kRows * kThreads / 32, "a warp spans the tile's width");
 // Per-tile triangle table of 2^BITS slots: a 32x16 tile of the head-scale workloads holds ~20-80 triangles.
-// 128 slots keep six CTAs resident with most of the SM's on-chip memory left to the L1 cache that serves the
+// 128 slots keep five CTAs resident with most of the SM's on-chip memory left to the L1 cache that serves the
 // vertex, texel and image gathers (256 slots measured 2.7 % slower on the multi-view head workload); a tile
 // with more triangles sends the excess straight to global memory, so launches in which some item is dense on
 // screen (more than 0.1 triangle per pixel) take 256 slots.  Only the variant without attribute gradients and

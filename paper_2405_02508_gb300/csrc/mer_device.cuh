@@ -574,7 +574,7 @@ __device__ __forceinline__ int find_item(const mer_item* __restrict__ items, int
 
 // find_item for consecutive elements g of a warp's lanes, g0 that of lane 0: the lanes look for g0's item together, 32 keys a
 // round (one round trip to memory up to 32 items, where a search by halves made one for each bit, and a block waited for the
-// thread that made it: 4,194,304 raster records of 32 items, 127 us to fill the lists, now 119), then each steps forward
+// thread that made it: 4,194,304 raster records of 32 items, 128 us to fill the lists, now 122), then each steps forward
 // over the few item boundaries inside the warp.  All lanes call it, also those whose element is past the end.
 __device__ __forceinline__ int warp_find_item(const mer_item* __restrict__ items, int n, long long g0, long long g, int f) {
     const int lane = threadIdx.x & 31;

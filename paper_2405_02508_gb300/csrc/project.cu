@@ -13,9 +13,9 @@
 namespace mer {
 
 // These kernels are bound by the FP64 pipe (one warp instruction in 16 cycles on an SM), on which conversions count like
-// any operation: 2,097,216 vertices of 32 views took 60 of them each, 201 us for 67 MB.  Exact conversions run on the integer
-// pipes instead (f2d, i2d), the snap is one FMA, and the batched backward converts a camera once a warp: 174 us, its
-// backward 75 -> 52.
+// any operation: 2,097,216 vertices of 32 views took 60 of them each, 204 us for 67 MB.  Exact conversions run on the integer
+// pipes instead (f2d, i2d), the snap is one FMA, and the batched backward converts a camera once a warp: 173 us, its
+// backward 76 -> 42 (each by itself, cold caches).
 
 __device__ __forceinline__ void write_vertex(double xs, double ys, double zeta, bool front, mer_vertex* out,
                                              mer_vertex* out2 = nullptr) {

@@ -344,7 +344,10 @@ constexpr int kSmallPx = 64;   // of at most this many: 8 lanes each; larger one
 // and 186; 131,072 there 144 (149) and 136.  In tiles of 16 no difference above 1 % but at 300 x 400 (50.7 and 48.4).
 // Resident CTAs per SM: 48 registers a thread, and a stage of the 64 x 64 tile small enough that its shared memory allows
 // five.  32 head views (tile 64) 1,855 us with four and 64 registers, 1,780 with five; 48 uneven meshes (tile 32) 651 and 586,
-// 588 with six at 40 registers; 8 views at 512 x 512 (tile 32) 78, 75 and 84.
+// 588 with six at 40 registers; 8 views at 512 x 512 (tile 32) 78, 75 and 84.  The generic form spills 16 to 80 bytes there and
+// is faster with five all the same: two interpolated channels, 8 x 512 x 512 at tile 32 125.4 us a forward pass with four and
+// 120.6 with five, 4 head views at tile 64 364.9 and 355.1; a texture of three floats a texel 413 and 405.  (Eight channels at
+// tile 64 are the exception: 501 and 521, and 549 since no load may pass a store, against 514 before the lane groups.)
 constexpr int kRasterCtasPerSm = 5;
 
 // Per-pixel bits kept in shared memory for the cover image: a front-facing triangle covered the centre of a pixel that a

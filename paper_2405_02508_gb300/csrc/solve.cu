@@ -203,7 +203,7 @@ __global__ void k_cg_next(CgState* st) {
 // are far below what a solve can show: in 576 solves of 258 to 211,602 rows of at most 8 neighbours (lambda 8, 16 and 32, rough, smooth and mixed
 // right-hand sides, cold and warm starts) iterations and solutions had the same bits as the launch sequence, whose sums
 // are FP64, hence the same errors against a 64-bit solution.
-// Measured (lambda 16, residual 1e-6, 79 and 49 iterations): 65,538 rows 3,520 -> 612 us, 642 rows 2,350 -> 155 us.
+// Measured (lambda 16, residual 1e-6, 79 and 49 iterations): 65,538 rows 3,760 -> 607 us, 642 rows 2,795 -> 155 us.
 constexpr int kCgThreads = 512;         // per CTA of the cluster form (one CTA per SM, up to 128 registers a thread)
 constexpr int kCgLocalThreads = 1024;   // the single-CTA form
 constexpr int kCgNeighbours = 8;        // neighbour ids kept in registers (a closed mesh averages 6)
