@@ -674,8 +674,8 @@ __global__ void k_bin_fill_batch(const mer_vertex* vpix, const int* tris, BatchG
 }
 
 // Persistent: each CTA takes the next global tile from the work queue until none is left.
-template <int TS, int FORM>
-__global__ void __launch_bounds__(kRasterThreads, kRasterCtasPerSm) k_raster_batch(TriRaster* recs, BatchGeom b,
+template <int TS, int FORM, int CTAS>
+__global__ void __launch_bounds__(kRasterThreads, CTAS) k_raster_batch(TriRaster* recs, BatchGeom b,
                                                                  const int* offs,
                                                                  const int* cnts,
                                                                  const int* nfront,
@@ -885,7 +885,7 @@ extern "C" size_t mer_batch_raster_workspace_size(long long tiles, long long tre
     return layout_for(tiles, trecs, capacity).total;
 }
 
-template <int TS, int FORM>
+template <int TS, int FORM, int CTAS = kRasterCtasPerSm>
 static int launch_raster_batch(unsigned grid, TriRaster* recs, BatchGeom b, const int* offs, const int* counts,
                                const int* nfront, const int* list, const mer_vertex* vpix, const int* tris, void* hdr, long long capacity,
                                int* index, float* depth, float* bary, unsigned char* cover, const ShadeOut& so,
@@ -894,12 +894,12 @@ static int launch_raster_batch(unsigned grid, TriRaster* recs, BatchGeom b, cons
         int per_sm = 0, sms = 0, dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess) return 2;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 2;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_raster_batch<TS, FORM>, kRasterThreads, 0) !=
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_raster_batch<TS, FORM, CTAS>, kRasterThreads, 0) !=
             cudaSuccess)
             return 2;
         grid = (unsigned)(sms * (per_sm > 0 ? per_sm : 1));
     }
-    launch_chained(k_raster_batch<TS, FORM>, grid, kRasterThreads, s, recs, b, offs, counts, nfront, list, vpix, tris, hdr, capacity,
+    launch_chained(k_raster_batch<TS, FORM, CTAS>, grid, kRasterThreads, s, recs, b, offs, counts, nfront, list, vpix, tris, hdr, capacity,
                                                               index, depth, bary, cover, so);
     return 0;
 }
@@ -912,7 +912,18 @@ static int launch_raster_batch_tile(int tile, unsigned grid, TriRaster* recs, Ba
     switch (tile) {
         case 16: return launch_raster_batch<16, FORM>(grid, recs, b, offs, counts, nfront, list, vpix, tris, hdr, capacity, index, depth, bary, cover, so, s);
         case 32: return launch_raster_batch<32, FORM>(grid, recs, b, offs, counts, nfront, list, vpix, tris, hdr, capacity, index, depth, bary, cover, so, s);
-        case 64: return launch_raster_batch<64, FORM>(grid, recs, b, offs, counts, nfront, list, vpix, tris, hdr, capacity, index, depth, bary, cover, so, s);
+        case 64:
+            // The generic form with all the registers it wants, while every tile has a CTA of its own all the same: 16 views
+            // of 3,200 triangles at 256 x 256, a texture of three floats a texel 139 us a forward pass with 48 registers
+            // and spills (132 before there were forms), 122 so; four large views, 1,400 tiles, 407 and 415.
+            if (FORM == kGeneric) {
+                int sms = 0, dev = 0;
+                if (cudaGetDevice(&dev) != cudaSuccess) return 2;
+                if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 2;
+                if (b.tiles <= 4LL * sms)
+                    return launch_raster_batch<64, kGeneric, 4>(grid > 4u * sms ? 4u * sms : grid, recs, b, offs, counts, nfront, list, vpix, tris, hdr, capacity, index, depth, bary, cover, so, s);
+            }
+            return launch_raster_batch<64, FORM>(grid, recs, b, offs, counts, nfront, list, vpix, tris, hdr, capacity, index, depth, bary, cover, so, s);
         default: return 1;
     }
 }
