@@ -6,8 +6,8 @@
 // step then needs M x (once, to start) and two solves M y = b per step: the gradient with respect to u,
 // M^-1 dL/dx, and the positions x = M^-1 u after the update.  M is symmetric positive definite (its
 // eigenvalues are 1 + lambda * those of L, all >= 1), so the solves are conjugate gradients on the device:
-// FP32 vectors, dot products of exact products in FP64 or two-float sums (about 48 bits), all three coordinate columns as one block-diagonal system, the iteration
-// scalars kept on the device (so a solve can be captured in a graph): one launch that ends once the residual is below
+// FP32 vectors, dot products of exact products in FP64 or two-float sums (about 48 bits), all three coordinate
+// columns as one block-diagonal system, the iteration scalars kept on the device (so a solve can be captured in a graph): one launch that ends once the residual is below
 // the tolerance, or, for systems beyond one resident grid, a fixed sequence of launches that become no-ops then.
 //
 // The CSR edge graph is built once per mesh on the host (mer_laplacian_csr).
@@ -200,9 +200,9 @@ __global__ void k_cg_next(CgState* st) {
 // two-float arithmetic, about 48 bits against FP64's 53, and so are the iteration's two quotients before they are rounded to
 // the FP32 factors alpha and beta.  GB300's FP64 pipe issues one warp instruction in 16 cycles, and the 64-bit sums and
 // divisions took longer than the exchanges (9 us an iteration of 258 rows, now 2.8).  The vectors are FP32, so the five bits
-// are far below what a solve can show: in 576 solves of 258 to 211,602 rows of at most 8 neighbours (lambda 8, 16 and 32, rough, smooth and mixed
-// right-hand sides, cold and warm starts) iterations and solutions had the same bits as the launch sequence, whose sums
-// are FP64, hence the same errors against a 64-bit solution.
+// are far below what a solve can show: in 576 solves of 258 to 211,602 rows of at most 8 neighbours (lambda 8, 16 and
+// 32, rough, smooth and mixed right-hand sides, cold and warm starts) iterations and solutions had the same bits as the
+// launch sequence, whose sums are FP64, hence the same errors against a 64-bit solution.
 // Measured (lambda 16, residual 1e-6, 79 and 49 iterations): 65,538 rows 3,760 -> 607 us, 642 rows 2,795 -> 155 us.
 constexpr int kCgThreads = 512;         // per CTA of the cluster form (one CTA per SM, up to 128 registers a thread)
 constexpr int kCgLocalThreads = 1024;   // the single-CTA form
